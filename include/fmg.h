@@ -213,7 +213,7 @@ fmg_status fmg_batch_create(fmg_ctx** cs, int count, void* stream, fmg_batch** o
  * the first kernel that is not phase-batchable) instead of falling back to branches.
  * phase_split (phase layout): each set of instances whose schedules agree is dealt round-robin
  * (after sorting by level count) into that many groups, which run as parallel branches of
- * phases, so that one group's latency-bound phases (the Newton kernels, the one-CTA coarse
+ * phases, so that one group's latency-bound phases (the Newton kernels, the coarse
  * cycles) overlap another's streaming ones; 0: the default; 1..1024. */
 fmg_status fmg_batch_create_mode(fmg_ctx** cs, int count, void* stream, int mode, int phase_split,
                                  fmg_batch** out);

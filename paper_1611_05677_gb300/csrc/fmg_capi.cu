@@ -37,7 +37,7 @@ struct fmg_ctx {
   double* dd[kMaxLevels] = {};
   ChebCoef cheb = {};
   double* Ainv = nullptr;
-  float* Ainv32 = nullptr;   // FP32 copy of A_1^{-1} for the FP32 one-CTA cycles
+  float* Ainv32 = nullptr;   // FP32 copy of A_1^{-1} for the FP32 cluster cycles
   DevState* st = nullptr;
   AugBuffers ab = {};
   VarCoef vc = {};   // the coefficient A(x) on the device (vc.a64 == nullptr: A = I)
@@ -310,17 +310,10 @@ cudaError_t cheb_steps(fmg_ctx* c, int j, T* u, T* alt, T* d, const T* b, int st
 // The coefficient for the launch calls: nullptr when A = I (the constant-coefficient kernels).
 const VarCoef* vcp(const fmg_ctx* c) { return c->vc.a64 ? &c->vc : nullptr; }
 
-// Largest level handled by the one-CTA coarse cycle: its level arrays (u and b of every level
-// up to it) must fit in shared memory; 2D up to 64 cells per side, 3D up to 16.  With a
-// variable coefficient every level above 1 runs the per-level kernels.
-template <typename T>
+// Largest level the cluster coarse cycle takes (1: none).
 int coarse_cycle_top(const fmg_ctx* c) {
-  if (c->vc.a64) return 1;
-  const int nmax = c->p.dim == 2 ? 64 : 16;
   int j = 1;
-  while (j < c->nlev && c->geo[j].n <= nmax &&
-         coarse_cycle_smem<T>(c->p.dim, c->p.coarse_cells, j + 1, c->p.smoother == FMG_SMOOTHER_CHEBYSHEV) <= 200 * 1024)
-    ++j;
+  while (j < c->nlev && c->geo[j].n <= coarse_cycle_cells(c->p.dim)) ++j;
   return j;
 }
 
@@ -332,9 +325,8 @@ double cheb_e0(const fmg_ctx* c, int j) {
 
 // Whether a coarse level j, entered from zero by the restriction, takes its first Chebyshev
 // step inside that restriction (it runs the per-level kernels and pre-smooths at all).
-template <typename T>
 bool fuse_first_step(const fmg_ctx* c, int j) {
-  return c->p.smoother == FMG_SMOOTHER_CHEBYSHEV && c->p.nu_pre >= 1 && j > coarse_cycle_top<T>(c);
+  return c->p.smoother == FMG_SMOOTHER_CHEBYSHEV && c->p.nu_pre >= 1 && j > coarse_cycle_top(c);
 }
 
 // Whether the mixed cycle on level k runs the fused 2D FP32 kernels (red-black smoothing with
@@ -350,10 +342,10 @@ cudaError_t vcycle(fmg_ctx* c, int j, double* u, const double* b, bool top = fal
     TRY(launch_coarse_solve_f64(dim, c->geo[0], c->Ainv, b, u, s));
     return cudaSuccess;
   }
-  if (j <= coarse_cycle_top<double>(c)) {
+  if (j <= coarse_cycle_top(c)) {
     // below the top level the restriction has zeroed u
     TRY(launch_coarse_cycle<double>(dim, c->p.coarse_cells, j, u, b, c->p.nu_pre, c->p.nu_post, c->Ainv, nullptr,
-                                    cheb_coef(c), !top, s));
+                                    cheb_coef(c), !top, s, vcp(c)));
     return cudaSuccess;
   }
   const LevelGeo gf = c->geo[j - 1], gc = c->geo[j - 2];
@@ -366,7 +358,7 @@ cudaError_t vcycle(fmg_ctx* c, int j, double* u, const double* b, bool top = fal
     TRY(launch_rbgs<double>(dim, gf, u, b, 1, s, vcp(c)));
     TRY(tend(c, slot));
   }
-  const bool fuse = fuse_first_step<double>(c, j - 1);
+  const bool fuse = fuse_first_step(c, j - 1);
   double* uc0 = fuse ? cheb_start(c->u[j - 2], c->ua[j - 2], c->p.nu_pre) : c->u[j - 2];
   TRY(launch_residual_restrict<double, double>(dim, gf, u, b, gc, c->b[j - 2], uc0, s,
                                                fuse ? c->dd[j - 2] : nullptr, fuse ? cheb_e0(c, j - 1) : 0.0, vcp(c)));
@@ -391,16 +383,11 @@ cudaError_t vcycle(fmg_ctx* c, int j, double* u, const double* b, bool top = fal
 cudaError_t vcycle32_fused(fmg_ctx* c, int j, double* u64_top, bool top_ff = false) {
   const int dim = c->p.dim;
   cudaStream_t s = c->stream;
-  if (j == 1) {
-    TRY(launch_coarse_solve_f32(dim, c->geo[0], c->Ainv, c->b32[0], c->u32[0], s));
-    return cudaSuccess;
-  }
-  if (j <= coarse_cycle_top<float>(c)) {
+  if (j <= coarse_cycle_top(c)) {
     // the FP32 cycles solve for a correction from zero on every level
     TRY(launch_coarse_cycle<float>(dim, c->p.coarse_cells, j, c->u32[j - 1], c->b32[j - 1], c->p.nu_pre,
-                                   c->p.nu_post, c->Ainv, c->Ainv32, cheb_coef(c), true, s));
-    if (u64_top && top_ff) TRY(launch_add_f32_ff(c->geo[j - 1], u64_top, c->u32[j - 1], s));
-    if (u64_top && !top_ff) TRY(launch_add_f32(c->geo[j - 1], dim, u64_top, c->u32[j - 1], s));
+                                   c->p.nu_post, c->Ainv, c->Ainv32, cheb_coef(c), true, s, nullptr, u64_top,
+                                   u64_top ? (top_ff ? 2 : 1) : 0));
     return cudaSuccess;
   }
   const LevelGeo gf = c->geo[j - 1];
@@ -425,13 +412,9 @@ cudaError_t vcycle32(fmg_ctx* c, int j, bool top = false, bool started = false, 
   cudaStream_t s = c->stream;
   float* u = c->u32[j - 1];
   const float* b = c->b32[j - 1];
-  if (j == 1) {
-    TRY(launch_coarse_solve_f32(dim, c->geo[0], c->Ainv, b, u, s));
-    return cudaSuccess;
-  }
-  if (j <= coarse_cycle_top<float>(c)) {
+  if (j <= coarse_cycle_top(c)) {
     TRY(launch_coarse_cycle<float>(dim, c->p.coarse_cells, j, u, b, c->p.nu_pre, c->p.nu_post, c->Ainv, c->Ainv32,
-                                   cheb_coef(c), true, s));
+                                   cheb_coef(c), true, s, vcp(c), u64_top, u64_top ? (top_ff ? 2 : 1) : 0));
     return cudaSuccess;
   }
   const LevelGeo gf = c->geo[j - 1], gc = c->geo[j - 2];
@@ -444,7 +427,7 @@ cudaError_t vcycle32(fmg_ctx* c, int j, bool top = false, bool started = false, 
     TRY(launch_rbgs<float>(dim, gf, u, b, 1, s, vcp(c)));
     TRY(tend(c, slot));
   }
-  const bool fuse = fuse_first_step<float>(c, j - 1);
+  const bool fuse = fuse_first_step(c, j - 1);
   float* uc0 = fuse ? cheb_start(c->u32[j - 2], c->u32b[j - 2], c->p.nu_pre) : c->u32[j - 2];
   TRY(launch_residual_restrict<float, float>(dim, gf, u, b, gc, c->b32[j - 2], uc0, s,
                                              fuse ? c->d32[j - 2] : nullptr, fuse ? cheb_e0(c, j - 1) : 0.0, vcp(c)));
@@ -483,15 +466,12 @@ cudaError_t top_cycle(fmg_ctx* c, int k, double* u, const double* b) {
   const LevelGeo g = c->geo[k - 1];
   // defect correction: FP64 residual -> FP32 cycle from e = 0 -> FP64 update (with Chebyshev
   // smoothing the cycle's first step is fused into the residual and its last into the update)
-  const bool fuse = fuse_first_step<float>(c, k);
+  const bool fuse = fuse_first_step(c, k);
   float* e0buf = fuse ? cheb_start(c->u32[k - 1], c->u32b[k - 1], c->p.nu_pre) : c->u32[k - 1];
   TRY(launch_residual_to_f32(c->p.dim, g, u, b, c->b32[k - 1], e0buf, c->stream,
                              fuse ? c->d32[k - 1] : nullptr, fuse ? cheb_e0(c, k) : 0.0, vcp(c)));
   if (fused_cycle_used(c, k)) return vcycle32_fused(c, k, u);
-  if (k > coarse_cycle_top<float>(c)) return vcycle32(c, k, true, fuse, u);
-  TRY(vcycle32(c, k, true));
-  TRY(launch_add_f32(g, c->p.dim, u, c->u32[k - 1], c->stream));
-  return cudaSuccess;
+  return vcycle32(c, k, true, fuse, u);
 }
 
 // The same cycle on the mixed solve's float-float level data: float-float residual -> FP32
@@ -501,16 +481,13 @@ cudaError_t top_cycle(fmg_ctx* c, int k, double* u, const double* b) {
 // level start computed it).
 cudaError_t top_cycle_ff(fmg_ctx* c, int k, double* u, const double* b, bool residual_ready = false) {
   const LevelGeo g = c->geo[k - 1];
-  const bool fuse = fuse_first_step<float>(c, k);
+  const bool fuse = fuse_first_step(c, k);
   float* e0buf = fuse ? cheb_start(c->u32[k - 1], c->u32b[k - 1], c->p.nu_pre) : c->u32[k - 1];
   if (!residual_ready)
     TRY(launch_residual_ff(c->p.dim, g, u, b, c->b32[k - 1], e0buf, c->stream, fuse ? c->d32[k - 1] : nullptr,
                            fuse ? cheb_e0(c, k) : 0.0, vcp(c)));
   if (fused_cycle_used(c, k)) return vcycle32_fused(c, k, u, true);
-  if (k > coarse_cycle_top<float>(c)) return vcycle32(c, k, true, fuse, u, true);
-  TRY(vcycle32(c, k, true));
-  TRY(launch_add_f32_ff(g, u, c->u32[k - 1], c->stream));
-  return cudaSuccess;
+  return vcycle32(c, k, true, fuse, u, true);
 }
 
 // Algorithm 3.1 at level k >= 2 on the level-k array u (FP64 contexts).
@@ -542,7 +519,7 @@ cudaError_t correction_step_ff(fmg_ctx* c, int k, bool out_f64, bool from_coarse
   TRY(tbegin(c, FMG_KT_CORRECTION, k, &slot_step));
   // step 1: b = (g, v) - (f(x, u^{(l)}), v)   (eq. 3.4)
   if (from_coarse) {
-    const bool fuse = fuse_first_step<float>(c, k);
+    const bool fuse = fuse_first_step(c, k);
     float* e0buf = fuse ? cheb_start(c->u32[k - 1], c->u32b[k - 1], c->p.nu_pre) : c->u32[k - 1];
     TRY(launch_level_start_ff(c->p.dim, c->geo[k - 2], c->u[k - 2], g, u, c->gf[k - 1], c->b[k - 1], c->p.f,
                               c->p.f_scale, c->b32[k - 1], e0buf, fuse ? c->d32[k - 1] : nullptr,
@@ -694,6 +671,7 @@ const std::vector<PhaseKernel>& phase_registry() {
     phase_kernels_stencil(r);
     phase_kernels_ff(r);
     phase_kernels_fused(r);
+    phase_kernels_coarse(r);
     phase_kernels_newton(r);
     return r;
   }();
@@ -1426,7 +1404,7 @@ fmg_status fmg_autotune(fmg_ctx* c, int* tuned) {
   if (c->p.smoother != FMG_SMOOTHER_CHEBYSHEV) return FMG_OK;   // the other kernels' shapes are fixed
   CK(c, cudaStreamSynchronize(c->stream));
   const bool mixed = c->p.precision == FMG_PREC_MIXED;
-  const int top_cta = mixed ? coarse_cycle_top<float>(c) : coarse_cycle_top<double>(c);
+  const int top_cta = coarse_cycle_top(c);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   CK(c, cudaEventCreate(&e0));
   cudaError_t ce = cudaEventCreate(&e1);

@@ -35,11 +35,20 @@ constexpr unsigned kFlagTimeout = 16u;
 // so that, in a captured graph, the launch of a kernel and the start of its blocks overlap its
 // predecessor's last blocks; the results are those of plain serialization.  Without the
 // attribute both instructions are no-ops.
-__device__ __forceinline__ void pdl_start() {
+// (A kernel with work of its own to do first calls the two halves apart.)
+__device__ __forceinline__ void pdl_launch() {
 #if defined(__CUDA_ARCH__)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void pdl_wait() {
+#if defined(__CUDA_ARCH__)
   asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void pdl_start() {
+  pdl_launch();
+  pdl_wait();
 }
 
 // Grids of more blocks launch without it: many waves hide the launch anyway, and a grid's blocks
@@ -264,10 +273,8 @@ cudaError_t launch_nonlinear_rhs(int dim, LevelGeo g, const double* u, const dou
 // copy nodal array (same level)
 cudaError_t launch_copy(const double* src, double* dst, long long n, cudaStream_t s);
 
-// FP32 V-cycle coarsest solve: e32 = (float)(Ainv (double) b32); FP64: e = Ainv b
+// coarsest solve of a V-cycle that starts on level 1: u = Ainv b
 cudaError_t launch_coarse_solve_f64(int dim, LevelGeo g1, const double* Ainv, const double* b, double* u,
-                                    cudaStream_t s);
-cudaError_t launch_coarse_solve_f32(int dim, LevelGeo g1, const double* Ainv, const float* b, float* u,
                                     cudaStream_t s);
 
 // Chebyshev-Jacobi smoothing, the colour-free alternative smoother: step k of the three-term
@@ -305,18 +312,20 @@ cudaError_t launch_cheb_add64(int dim, LevelGeo g, const float* u, const float* 
 template <typename T>
 cudaError_t launch_copy_t(const T* src, T* dst, long long n, cudaStream_t s);
 
-// The whole V-cycle on levels jtop..1 in one CTA with shared-memory level arrays (level j
-// has n0 << (j-1) cells per side); u (in/out) and b are level jtop's nodal arrays.  cheb:
-// NULL for red-black Gauss-Seidel smoothing, else Chebyshev-Jacobi steps (nu_pre / nu_post
-// of them), which need two more arrays per level.
+// The V(nu_pre, nu_post) cycle on levels jtop..1 (jtop >= 2) in one launch of one thread-block
+// cluster with shared-memory level arrays (level j has n0 << (j-1) <= coarse_cycle_cells(dim)
+// cells per side); u (in/out) and b are level jtop's nodal arrays.  cheb: NULL for red-black
+// Gauss-Seidel smoothing, else Chebyshev-Jacobi steps (nu_pre / nu_post of them), which need one
+// more array per level.  Ainv32: FP32 copy of A_1^{-1} (required for T = float with A = I).
+// zero_start: u is zero on entry (not read).  add_mode 1 / 2: instead of being stored, u is added
+// to the FP64 / float-float nodal array `add`.
+int coarse_cycle_cells(int dim);
 template <typename T>
 size_t coarse_cycle_smem(int dim, int n0, int jtop, bool cheb);
-// The V(nu_pre, nu_post) cycle on levels jtop..1 in one CTA.  Ainv32: FP32 copy of A_1^{-1}
-// (required for T = float).  zero_start: u is zero on entry (not read).
 template <typename T>
 cudaError_t launch_coarse_cycle(int dim, int n0, int jtop, T* u, const T* b, int nu_pre, int nu_post,
                                 const double* Ainv, const float* Ainv32, const ChebCoef* cheb, bool zero_start,
-                                cudaStream_t s);
+                                cudaStream_t s, const VarCoef* vc = nullptr, double* add = nullptr, int add_mode = 0);
 // dst = (float) src, n values
 cudaError_t launch_to_f32(const double* src, float* dst, long long n, cudaStream_t s);
 

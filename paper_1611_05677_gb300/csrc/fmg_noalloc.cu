@@ -65,11 +65,10 @@ struct Ctx {
   double* b(int j) const { return u(j) + geo(j).nodes; }
 };
 
-// Largest level the one-CTA coarse cycle takes (same rule as the context's schedule).
+// Largest level the cluster coarse cycle takes (same rule as the context's schedule).
 int coarse_top(const Ctx& c, int level) {
-  const int nmax = c.dim == 2 ? 64 : 16;
   int j = 1;
-  while (j < level && c.geo(j + 1).n <= nmax && coarse_cycle_smem<double>(c.dim, c.nc, j + 1, false) <= 200 * 1024) ++j;
+  while (j < level && c.geo(j + 1).n <= coarse_cycle_cells(c.dim)) ++j;
   return j;
 }
 

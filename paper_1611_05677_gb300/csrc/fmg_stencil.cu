@@ -26,7 +26,6 @@ namespace fmg {
 namespace {
 
 constexpr int kBlock = 128;
-constexpr int kMaxCoarseN = 64;   // level-1 unknowns (2D: (1/H - 1)^2 <= 49, 3D: <= 27)
 
 inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
@@ -571,313 +570,6 @@ template <typename T>
 __global__ void k_coarse_solve(const double* __restrict__ Ainv, const T* __restrict__ b, T* __restrict__ u, int m,
                                int N, int dim) { pdl_start(); k_coarse_solve_body<T>(Ainv, b, u, m, N, dim); }
 
-// ------------------------------------------------------------------ coarse V-cycle in one CTA
-// The V(nu_pre, nu_post) cycle on levels jtop..1 with every level's u and b in shared
-// memory: the same red-black sweeps, restriction P^T, exact level-1 solve (dense
-// A_1^{-1} in FP64) and prolongation as the per-level kernels, separated by __syncthreads
-// instead of launches.  Level jtop's u and b are read from and u written back to global
-// memory.  Level j has n0 << (j-1) cells per side.
-template <typename T, int D>
-struct CoarseLevel {
-  int n;        // cells per side (a power of two)
-  int lg;       // log2(n)
-  int np;       // n + 1
-  T* u;
-  T* b;
-  T* ua;        // Chebyshev smoothing: second iterate buffer and the step direction
-  T* d;
-};
-
-// One colour of a red-black sweep: items are (p, j[, l]) with i = 2p + 1 or 2p + 2, decoded
-// with shifts; rows 0 and n and out-of-range i are skipped.
-template <typename T, int D>
-__device__ __forceinline__ void cta_rbgs(const CoarseLevel<T, D>& L, int colour, T bscale, T inv2d) {
-  const int n = L.n, np = L.np, lgh = L.lg - 1;
-  const int total = D == 2 ? (n << lgh) : (n << (lgh + L.lg));
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int p = t & ((1 << lgh) - 1);
-    const int j = (t >> lgh) & (n - 1);
-    const int l = D == 3 ? (t >> (lgh + L.lg)) : 0;
-    if (j == 0 || (D == 3 && l == 0)) continue;
-    const int par = (colour + j + l) & 1;
-    const int i = par ? 2 * p + 1 : 2 * p + 2;
-    if (i > n - 1) continue;
-    const int c = (l * np + j) * np + i;
-    T s = (L.u[c - 1] + L.u[c + 1]) + (L.u[c - np] + L.u[c + np]);
-    if (D == 3) s += L.u[c - np * np] + L.u[c + np * np];
-    L.u[c] = (L.b[c] * bscale + s) * inv2d;
-  }
-}
-
-// The buffer in which a Chebyshev step 0 taken from a zero start (by the code that writes
-// the level's b) leaves the iterate, so that steps 1..steps-1 end in L.u.
-template <typename T, int D>
-__device__ __forceinline__ T* cta_cheb_start(const CoarseLevel<T, D>& L, int steps) {
-  return ((steps - 1) & 1) ? L.ua : L.u;
-}
-
-// Chebyshev-Jacobi steps k0..steps-1 on level L (colour-free: every interior node per step,
-// the iterate alternating between u and ua); they start in L.u (k0 = 0) or in
-// cta_cheb_start(L, steps) with d set (k0 = 1), and the result ends in L.u.
-template <typename T, int D>
-__device__ void cta_cheb(const CoarseLevel<T, D>& L, const ChebCoef& cf, int steps, T bscale, T inv2d, int k0 = 0) {
-  const int n = L.n, np = L.np, lg = L.lg;
-  const int total = D == 2 ? (1 << (2 * lg)) : (1 << (3 * lg));
-  T* u = k0 ? cta_cheb_start(L, steps) : L.u;
-  T* ua = u == L.u ? L.ua : L.u;
-  for (int k = k0; k < steps; ++k) {
-    const T cd = (T)cf.cd[k], cr = (T)cf.cr[k];
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int i = t & (n - 1), j = (t >> lg) & (n - 1), l = D == 3 ? (t >> (2 * lg)) : 0;
-      if (i == 0 || j == 0 || (D == 3 && l == 0)) continue;
-      const int c = (l * np + j) * np + i;
-      T s = (u[c - 1] + u[c + 1]) + (u[c - np] + u[c + np]);
-      if (D == 3) s += u[c - np * np] + u[c + np * np];
-      const T z = (L.b[c] * bscale + s) * inv2d - u[c];
-      const T dn = k == 0 ? cr * z : cd * L.d[c] + cr * z;
-      L.d[c] = dn;
-      ua[c] = u[c] + dn;
-    }
-    __syncthreads();
-    T* t2 = u;
-    u = ua;
-    ua = t2;
-  }
-  if (u != L.u) {
-    const int nodes = D == 2 ? np * np : np * np * np;
-    for (int c = threadIdx.x; c < nodes; c += blockDim.x) L.u[c] = u[c];
-    __syncthreads();
-  }
-}
-
-template <typename T, int D>
-__device__ __forceinline__ T cta_res(const CoarseLevel<T, D>& L, int c, T sigma) {
-  const int np = L.np;
-  T s = (L.u[c - 1] + L.u[c + 1]) + (L.u[c - np] + L.u[c + np]);
-  if (D == 3) s += L.u[c - np * np] + L.u[c + np * np];
-  return L.b[c] - sigma * (T(2 * D) * L.u[c] - s);
-}
-
-// zero_start: the top level's u is zero on entry (a correction from zero): it is not read,
-// and with Chebyshev smoothing the top level's step 0 (pointwise from zero) is taken while b
-// is loaded.  Below the top level the restriction takes the coarse level's step 0 the same
-// way.  The FP32 cycle's level-1 solve uses an FP32 copy of A_1^{-1} (Ainv32), staged in
-// shared memory while the top level loads; the FP64 cycle reads the FP64 A_1^{-1}.
-template <typename T, int D>
-__device__ __forceinline__ void k_vcycle_coarse_body(T* __restrict__ ug, const T* __restrict__ bg, int n0, int jtop, int nu_pre,
-                                int nu_post, const double* __restrict__ Ainv, const float* __restrict__ Ainv32,
-                                int cheb, const ChebCoef& cf, int zero_start) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  T* sm = reinterpret_cast<T*>(smraw);
-  // level descriptors, the same for every thread: in shared memory (a per-thread copy would
-  // be local memory, 1024 copies of it)
-  __shared__ CoarseLevel<T, D> L[8];
-  __shared__ int ai_off;
-  constexpr bool kStageInv = sizeof(T) == sizeof(float);
-  if (threadIdx.x == 0) {
-    int off = 0;
-    for (int j = 1; j <= jtop; ++j) {
-      const int n = n0 << (j - 1);
-      const int np = n + 1;
-      const int nodes = D == 2 ? np * np : np * np * np;
-      L[j - 1].n = n;
-      L[j - 1].lg = 31 - __clz(n);
-      L[j - 1].np = np;
-      L[j - 1].u = sm + off;
-      L[j - 1].b = sm + off + nodes;
-      L[j - 1].ua = cheb ? sm + off + 2 * nodes : nullptr;
-      L[j - 1].d = cheb ? sm + off + 3 * nodes : nullptr;
-      off += (cheb ? 4 : 2) * nodes;
-    }
-    ai_off = off;
-  }
-  __syncthreads();
-  float* ai = kStageInv ? reinterpret_cast<float*>(sm + ai_off) : nullptr;   // staged FP32 A_1^{-1}
-  const T inv2d = T(1) / T(2 * D);
-  const int m1 = n0 - 1;
-  const int N1 = D == 2 ? m1 * m1 : m1 * m1 * m1;
-  {
-    const CoarseLevel<T, D>& top = L[jtop - 1];
-    const int np = top.np;
-    const int nodes = D == 2 ? np * np : np * np * np;
-    // top level: b, and u (or, from a zero start, u = 0 or the first Chebyshev step); the
-    // FP32 cycle also stages A_1^{-1}.  Every global load of a thread is issued before the
-    // first store, so the phase costs about one memory latency.
-    const bool first_top = cheb && zero_start && nu_pre >= 1 && jtop >= 2;
-    const T e0 = T(cf.cr[0]) * (D == 2 ? T(1) : T(top.n)) * inv2d;   // step 0 from zero: cr_0 D^{-1} b
-    T* ustart = first_top ? cta_cheb_start(top, nu_pre) : top.u;
-    const int nai = kStageInv ? N1 * N1 : 0;
-    for (int i0 = threadIdx.x; i0 < nodes || i0 < nai; i0 += 4 * blockDim.x) {
-      T bv[4], uv[4];
-      float av[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r * blockDim.x;
-        bv[r] = i < nodes ? bg[i] : T(0);
-        uv[r] = (i < nodes && !zero_start) ? ug[i] : T(0);
-        av[r] = i < nai ? __ldg(&Ainv32[i]) : 0.f;
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r * blockDim.x;
-        if (i < nai) ai[i] = av[r];
-        if (i >= nodes) continue;
-        top.b[i] = bv[r];
-        top.u[i] = uv[r];
-        if (first_top) {
-          const int x = i % np, y = (i / np) % np, z = D == 3 ? i / (np * np) : 1;
-          const bool inner = x > 0 && x < np - 1 && y > 0 && y < np - 1 && (D == 2 || (z > 0 && z < np - 1));
-          const T e = inner ? e0 * bv[r] : T(0);
-          ustart[i] = e;
-          top.d[i] = e;
-        }
-      }
-    }
-    // lower levels: zero (boundary rings stay zero); the other Chebyshev buffers too
-    for (int j = 1; j <= jtop; ++j) {
-      const CoarseLevel<T, D>& Lj = L[j - 1];
-      const int nn = D == 2 ? Lj.np * Lj.np : Lj.np * Lj.np * Lj.np;
-      if (j < jtop)
-        for (int i = threadIdx.x; i < 2 * nn; i += blockDim.x) Lj.u[i] = T(0);
-      if (cheb) {
-        if (j < jtop) {
-          for (int i = threadIdx.x; i < 2 * nn; i += blockDim.x) Lj.ua[i] = T(0);
-        } else {
-          T* other = ustart == top.u ? top.ua : top.u;   // the top level's u, d and start are set above
-          for (int i = threadIdx.x; i < nn; i += blockDim.x) {
-            if (other == top.ua) top.ua[i] = T(0);
-            if (!first_top) top.d[i] = T(0);
-          }
-        }
-      }
-    }
-  }
-  __syncthreads();
-  // descend
-  for (int j = jtop; j >= 2; --j) {
-    const CoarseLevel<T, D>& F = L[j - 1];
-    const CoarseLevel<T, D>& C = L[j - 2];
-    const T bscale = D == 2 ? T(1) : T(F.n);
-    const T sigma = D == 2 ? T(1) : T(1) / T(F.n);
-    if (cheb) {
-      // step 0 was taken by the load (top level from zero) or by the restriction (below)
-      const bool started = nu_pre >= 1 && (j < jtop || zero_start);
-      cta_cheb<T, D>(F, cf, nu_pre, bscale, inv2d, started ? 1 : 0);
-    } else {
-      for (int it = 0; it < nu_pre; ++it) {
-        cta_rbgs<T, D>(F, 0, bscale, inv2d);
-        __syncthreads();
-        cta_rbgs<T, D>(F, 1, bscale, inv2d);
-        __syncthreads();
-      }
-    }
-    // b_c = P^T (b - A u), u_c = 0 -- or, when the coarse level is smoothed by Chebyshev
-    // steps, its step 0 from zero: u_c = d_c = cr_0 D^{-1} b_c in the start buffer.  Items
-    // (I, J[, K]) over [0, n_c)^d, boundary skipped.
-    const int lgc = C.lg;
-    const int total = D == 2 ? (1 << (2 * lgc)) : (1 << (3 * lgc));
-    const bool first_c = cheb && nu_pre >= 1 && j - 1 >= 2;
-    const T e0c = T(cf.cr[0]) * (D == 2 ? T(1) : T(C.n)) * inv2d;
-    T* ucs = first_c ? cta_cheb_start(C, nu_pre) : C.u;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int I = t & (C.n - 1), J = (t >> lgc) & (C.n - 1), K = D == 3 ? (t >> (2 * lgc)) : 0;
-      if (I == 0 || J == 0 || (D == 3 && K == 0)) continue;
-      const int np = F.np;
-      const int Fc = ((2 * K) * np + 2 * J) * np + 2 * I;
-      T r = cta_res<T, D>(F, Fc, sigma);
-      T e = (cta_res<T, D>(F, Fc + 1, sigma) + cta_res<T, D>(F, Fc - 1, sigma)) +
-            (cta_res<T, D>(F, Fc + np, sigma) + cta_res<T, D>(F, Fc - np, sigma)) +
-            (cta_res<T, D>(F, Fc + np + 1, sigma) + cta_res<T, D>(F, Fc - np - 1, sigma));
-      if (D == 3) {
-        const int pl = np * np;
-        const int o[4] = {pl, 1 + pl, np + pl, 1 + np + pl};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) e += cta_res<T, D>(F, Fc + o[q], sigma) + cta_res<T, D>(F, Fc - o[q], sigma);
-      }
-      const int cc = (K * C.np + J) * C.np + I;
-      const T bv = r + T(0.5) * e;
-      C.b[cc] = bv;
-      if (first_c) {
-        ucs[cc] = e0c * bv;
-        C.d[cc] = e0c * bv;
-      } else {
-        C.u[cc] = T(0);
-      }
-    }
-    __syncthreads();
-  }
-  // level 1: u_1 = A_1^{-1} b_1 in FP64; b_1 staged as FP64 in the (now unused) level-1 u
-  // slots is not possible for FP32 levels, so it goes to a small shared array
-  {
-    __shared__ double b1[kMaxCoarseN];
-    __shared__ int off1[kMaxCoarseN];
-    const CoarseLevel<T, D>& C = L[0];
-    const int m = C.n - 1;
-    const int N = D == 2 ? m * m : m * m * m;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-      const int i = c % m + 1, j = (c / m) % m + 1, l = D == 3 ? c / (m * m) + 1 : 0;
-      off1[c] = (l * C.np + j) * C.np + i;
-      b1[c] = (double)C.b[off1[c]];
-    }
-    __syncthreads();
-    // row r: lanes of one warp split the columns (row r of the symmetric A_1^{-1} is read
-    // contiguously), then a shuffle sum (fixed order)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int r = warp; r < N; r += nw) {
-      if (kStageInv) {
-        float acc = 0.f;
-        for (int c = lane; c < N; c += 32) acc = fmaf(ai[r * N + c], (float)b1[c], acc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) C.u[off1[r]] = (T)acc;
-      } else {
-        double acc = 0.0;
-        for (int c = lane; c < N; c += 32) acc = fma(__ldg(&Ainv[(long long)r * N + c]), b1[c], acc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) C.u[off1[r]] = (T)acc;
-      }
-    }
-    __syncthreads();
-  }
-  // ascend
-  for (int j = 2; j <= jtop; ++j) {
-    const CoarseLevel<T, D>& F = L[j - 1];
-    const CoarseLevel<T, D>& C = L[j - 2];
-    const T bscale = D == 2 ? T(1) : T(F.n);
-    const int lgf = F.lg;
-    const int total = D == 2 ? (1 << (2 * lgf)) : (1 << (3 * lgf));
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int i = t & (F.n - 1), jj = (t >> lgf) & (F.n - 1), l = D == 3 ? (t >> (2 * lgf)) : 0;
-      if (i == 0 || jj == 0 || (D == 3 && l == 0)) continue;
-      const int a = ((l >> 1) * C.np + (jj >> 1)) * C.np + (i >> 1);
-      const int z = (((l + 1) >> 1) * C.np + ((jj + 1) >> 1)) * C.np + ((i + 1) >> 1);
-      F.u[(l * F.np + jj) * F.np + i] += T(0.5) * (C.u[a] + C.u[z]);
-    }
-    __syncthreads();
-    if (cheb) {
-      cta_cheb<T, D>(F, cf, nu_post, bscale, inv2d);
-    } else {
-      for (int it = 0; it < nu_post; ++it) {
-        cta_rbgs<T, D>(F, 1, bscale, inv2d);
-        __syncthreads();
-        cta_rbgs<T, D>(F, 0, bscale, inv2d);
-        __syncthreads();
-      }
-    }
-  }
-  {
-    const CoarseLevel<T, D>& top = L[jtop - 1];
-    const int nodes = D == 2 ? top.np * top.np : top.np * top.np * top.np;
-    for (int i = threadIdx.x; i < nodes; i += blockDim.x) ug[i] = top.u[i];
-  }
-}
-
-template <typename T, int D>
-__global__ void __launch_bounds__(1024) k_vcycle_coarse(T* __restrict__ ug, const T* __restrict__ bg, int n0, int jtop, int nu_pre,
-                                int nu_post, const double* __restrict__ Ainv, const float* __restrict__ Ainv32,
-                                int cheb, const __grid_constant__ ChebCoef cf, int zero_start) { pdl_start(); k_vcycle_coarse_body<T, D>(ug, bg, n0, jtop, nu_pre, nu_post, Ainv, Ainv32, cheb, cf, zero_start); }
-
 }  // namespace
 
 // ============================================================================ launchers
@@ -1010,47 +702,6 @@ cudaError_t launch_coarse_solve_f64(int dim, LevelGeo g1, const double* Ainv, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_coarse_solve_f32(int dim, LevelGeo g1, const double* Ainv, const float* b, float* u,
-                                    cudaStream_t s) {
-  const int m = g1.n - 1;
-  const int N = (int)ipow(m, dim);
-  launch_k(k_coarse_solve<float>, 1, 64, N * sizeof(double), s, Ainv, b, u, m, N, dim);
-  return cudaGetLastError();
-}
-
-template <typename T>
-size_t coarse_cycle_smem(int dim, int n0, int jtop, bool cheb) {
-  size_t tot = 0;
-  for (int j = 1; j <= jtop; ++j) {
-    const long long np = (long long)(n0 << (j - 1)) + 1;
-    tot += (cheb ? 4 : 2) * (size_t)ipow(np, dim);
-  }
-  // the FP32 cycle stages its FP32 A_1^{-1}
-  const size_t n1 = (size_t)ipow(n0 - 1, dim);
-  return tot * sizeof(T) + (sizeof(T) == sizeof(float) ? n1 * n1 * sizeof(float) : 0);
-}
-
-template <typename T>
-cudaError_t launch_coarse_cycle(int dim, int n0, int jtop, T* u, const T* b, int nu_pre, int nu_post,
-                                const double* Ainv, const float* Ainv32, const ChebCoef* cheb, bool zero_start,
-                                cudaStream_t s) {
-  if (sizeof(T) == sizeof(float) && !Ainv32) return cudaErrorInvalidValue;
-  if (cheb && (nu_pre > kMaxCheb || nu_post > kMaxCheb)) return cudaErrorInvalidValue;
-  const size_t smem = coarse_cycle_smem<T>(dim, n0, jtop, cheb != nullptr);
-  const ChebCoef cf = cheb ? *cheb : ChebCoef{};
-  cudaError_t e;
-  if (dim == 2) {
-    if ((e = raise_dyn_smem((const void*)k_vcycle_coarse<T, 2>, smem)) != cudaSuccess) return e;
-    launch_k(k_vcycle_coarse<T, 2>, 1, 1024, smem, s, u, b, n0, jtop, nu_pre, nu_post, Ainv, Ainv32, cheb ? 1 : 0, cf,
-                                                 zero_start ? 1 : 0);
-  } else {
-    if ((e = raise_dyn_smem((const void*)k_vcycle_coarse<T, 3>, smem)) != cudaSuccess) return e;
-    launch_k(k_vcycle_coarse<T, 3>, 1, 1024, smem, s, u, b, n0, jtop, nu_pre, nu_post, Ainv, Ainv32, cheb ? 1 : 0, cf,
-                                                 zero_start ? 1 : 0);
-  }
-  return cudaGetLastError();
-}
-
 ChebCoef cheb_coefficients() {
   // lmax = 2 bounds the spectrum of D^{-1}A for the 2d+1-point stiffness; the smoother
   // targets [lmax/4, lmax]
@@ -1170,12 +821,6 @@ cudaError_t launch_copy_t(const T* src, T* dst, long long n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template size_t coarse_cycle_smem<double>(int, int, int, bool);
-template size_t coarse_cycle_smem<float>(int, int, int, bool);
-template cudaError_t launch_coarse_cycle<double>(int, int, int, double*, const double*, int, int, const double*,
-                                                 const float*, const ChebCoef*, bool, cudaStream_t);
-template cudaError_t launch_coarse_cycle<float>(int, int, int, float*, const float*, int, int, const double*,
-                                                const float*, const ChebCoef*, bool, cudaStream_t);
 template cudaError_t launch_cheb<double>(int, LevelGeo, const double*, double*, double*, const double*, double, double,
                                          bool, cudaStream_t, const double*);
 template cudaError_t launch_cheb<float>(int, LevelGeo, const float*, float*, float*, const float*, double, double, bool,
@@ -1238,10 +883,7 @@ void phase_kernels_stencil(std::vector<PhaseKernel>& out) {
   out.push_back(phase_kernel<&k_prolong2_body<float, float>, kBlock, 1>(&k_prolong2<float, float>));
   out.push_back(phase_kernel<&k_prolong2_body<double, double>, kBlock, 1>(&k_prolong2<double, double>));
   out.push_back(phase_kernel<&k_nonlinear_rhs_body, kBlock, 1>(&k_nonlinear_rhs));
-  out.push_back(phase_kernel<&k_coarse_solve_body<float>, 64, 24>(&k_coarse_solve<float>));
   out.push_back(phase_kernel<&k_coarse_solve_body<double>, 64, 24>(&k_coarse_solve<double>));
-  out.push_back(phase_kernel<&k_vcycle_coarse_body<float, 2>, 1024, 1>(&k_vcycle_coarse<float, 2>));
-  out.push_back(phase_kernel<&k_vcycle_coarse_body<double, 2>, 1024, 1>(&k_vcycle_coarse<double, 2>));
 }
 
 }  // namespace fmg
