@@ -1337,7 +1337,7 @@ fmg_status fmg_autotune_augmented(fmg_ctx* c, int* tuned) {
       ce = launch_ff_from_f64(c->u[k - 1], pristine, g.nodes, c->stream);
     else
       ce = cudaMemcpyAsync(pristine, c->u[k - 1], g.nodes * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
-    const AugShape rule = aug_shape(c->p.dim, c->p.coarse_cells, k, mixed, c->ab, false);
+    const AugShape rule = aug_shape(c->p.dim, c->p.coarse_cells, k, mixed, c->ab, true, false);
     AugShape best = rule;
     float best_ms = 0.f;
     const int sfine = 1 << (k - 1);
@@ -1394,7 +1394,7 @@ fmg_status fmg_aug_shape(const fmg_ctx* c, int level, int* chunk, int* blocks_pe
   const AugShape sh = aug_shape(c->p.dim, c->p.coarse_cells, level, c->p.precision == FMG_PREC_MIXED, c->ab,
                                 c->cluster_aug == 0);
   if (chunk) *chunk = sh.chunk;
-  if (blocks_per_cell) *blocks_per_cell = c->cluster_aug > 0 ? 1 : sh.bpc;
+  if (blocks_per_cell) *blocks_per_cell = sh.bpc;
   return FMG_OK;
 }
 

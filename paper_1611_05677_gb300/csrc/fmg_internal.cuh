@@ -358,12 +358,14 @@ struct AugBuffers {
 };
 // Launch shape of the cooperative augmented kernel on one level: column-chunk length and
 // blocks per coarse cell.  aug_shape gives the tuned one (set_aug_shape, process-wide; tuned =
-// false: the rule only) within the launch's limits, else the rule of launch_augmented.
+// false: the rule only) within the launch's limits, else the rule's.  coop = false: the cluster
+// variant's chunks (the rule's, one block per cell).
 struct AugShape {
   int chunk;
   int bpc;
 };
-AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const AugBuffers& ab, bool tuned = true);
+AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const AugBuffers& ab, bool coop = true,
+                   bool tuned = true);
 void set_aug_shape(int dim, int coarse_cells, int level, bool mixed, AugShape sh);
 bool aug_shape_tuned(int dim, int coarse_cells, int level, bool mixed, AugShape* out);
 // Fills bpc/nt/smem/partial_items for this device (occupancy-based), outside any capture.

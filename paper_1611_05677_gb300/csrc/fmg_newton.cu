@@ -503,8 +503,8 @@ struct Aug {
   static constexpr int NT = D == 2 ? 256 : 128;
 };
 
-// Channel rows of a block: one row of NT per-thread partial sums per channel.  FP64 path:
-// every channel FP64, already scaled by its quadrature weight.  Mixed path: the residual
+// Channel rows of a block: one row of NT per-thread partial sums per channel, without the
+// quadrature weights, which the block sum applies.  FP64 path: every channel FP64.  Mixed path: the residual
 // channels (RA .. SS) are float-float pairs (hi, lo) in their 8-byte slots and carry no weight
 // (RA is scaled by w/s, SA by w, TT by 1/s when the block sum is converted to FP64), so a pass
 // does no FP64 arithmetic; the Jacobian channels (JB .. JS) are FP32 rows after them (FP32
@@ -547,7 +547,7 @@ struct AugArgs {
   int fixed_point;      // 1: fixed-point iteration (Galerkin stiffness only, no Jacobian)
   int out_f64;          // mixed path: the update writes u as FP64 (the solve's result) instead of float-float
   int split_update;     // 1: the final update is left to k_aug_update (block 0 writes c and alpha to cfin)
-  double a, w, sigma_k, sigma_H, tol;
+  double a, w, inv_s, sigma_k, sigma_H, tol;
   ff a_ff, sigma_ff;    // mixed path: a and sigma_k as float-float
   double* u;            // u~ on entry, u^{(l+1)} on exit (level-k nodal; float-float in the mixed path)
   const double* g;      // level-k nodal g (float-float in the mixed path)
@@ -559,37 +559,42 @@ struct AugArgs {
   long long bar_spins;  // polls of the grid barrier before it times out
   int bar_skip;         // test hook: this block skips its first barrier arrival (-1: none)
   VarCoef vc;           // the coefficient A(x) (vc.a64 == nullptr: A = I)
-  const int* jtab;      // mixed path: the Jacobian gather table (k_aug_jtab)
+  const int* jtab;      // the Jacobian gather table (k_aug_jtab)
+  // FP64 path: the quadrature weight of each channel kind (its rows carry none)
+  double wRA, wSA, wTT, wSS, wJB, wJP, wJS;
 };
 
-// Bounded grid barrier for the cooperative launch (all blocks co-resident).  A waiting block
-// gives up after `spins` polls: the timeout flag and the abort word are set and every block
-// leaves at its next check.  skip (the failure-detection test hook): this block does not
-// arrive, so the others run out of polls; no block waits without bound.
-__device__ void grid_barrier(DevState* st, unsigned nblocks, long long spins_max, bool skip) {
+// Bounded grid barrier for the cooperative launch (all blocks co-resident).  gen: the barrier
+// generation, read once when the kernel starts (it cannot move before this block's first arrival)
+// and then counted by thread 0, so that an arrival costs one atomic with release / acquire
+// semantics and the waiters poll one word.  A waiting block gives up after `spins` polls: the
+// timeout flag and the abort word are set and every block leaves at its next check.  skip (the
+// failure-detection test hook): this block does not arrive, so the others run out of polls; no
+// block waits without bound.
+__device__ void grid_barrier(DevState* st, unsigned nblocks, long long spins_max, bool skip, unsigned& gen) {
   __syncthreads();
   if (nblocks > 1 && threadIdx.x == 0) {
-    volatile unsigned* genp = &st->bar_gen;
-    const unsigned gen = *genp;
-    __threadfence();
-    const unsigned arrived = skip ? 0u : atomicAdd(&st->bar_count, 1u);
+    unsigned arrived = 0u;
+    if (!skip)
+      asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(&st->bar_count) : "memory");
     if (!skip && arrived == nblocks - 1) {
-      atomicExch(&st->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&st->bar_gen, 1u);
+      asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(&st->bar_count) : "memory");
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&st->bar_gen), "r"(gen + 1u) : "memory");
     } else {
       long long spins = 0;
-      while (*genp == gen) {
-        __nanosleep(32);
+      for (;;) {
+        unsigned g;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&st->bar_gen) : "memory");
+        if (g != gen) break;
         if (++spins > spins_max) {
           atomicOr(&st->flags, kFlagTimeout);
           atomicExch(&st->abort, 1);
           break;
         }
-        if (((volatile int*)&st->abort)[0]) break;
+        if ((spins & 15) == 0 && ((volatile int*)&st->abort)[0]) break;
       }
     }
-    __threadfence();
+    ++gen;
   }
   __syncthreads();
 }
@@ -641,6 +646,40 @@ __device__ __forceinline__ int column_segments(const int* o, int s, Seg<D>* sg) 
     sg[2].z0 = hi + 1; sg[2].z1 = s - 1;
     return 3;
   }
+}
+
+// The same segments by the form of their barycentric weights: (p - z) / s at vertex vp,
+// (z - q) / s at vertex vq and constants c / s at the D - 1 others.
+template <int D>
+struct SegW {
+  int vp, vq, vc[D - 1];
+  int p, q, c[D - 1];
+  int z0, z1;
+};
+
+template <int D>
+__device__ __forceinline__ void column_segments_w(const int* o, int s, SegW<D>* sg) {
+  if constexpr (D == 2) {
+    const int ox = o[0];
+    sg[0] = SegW<2>{1, 3, {0}, ox, 0, {s - ox}, 0, ox};
+    sg[1] = SegW<2>{0, 2, {3}, s, ox, {ox}, ox + 1, s - 1};
+  } else {
+    const int ox = o[0], oy = o[1];
+    const bool xhi = ox >= oy;
+    const int hi = xhi ? ox : oy, lo = xhi ? oy : ox;
+    const int bh = xhi ? 1 : 2, bl = xhi ? 2 : 1;
+    sg[0] = SegW<3>{bh | bl, 7, {0, bh}, lo, 0, {s - hi, hi - lo}, 0, lo};
+    sg[1] = SegW<3>{bh, bh | 4, {0, 7}, hi, lo, {s - hi, lo}, lo + 1, hi};
+    sg[2] = SegW<3>{0, 4, {4 | bh, 7}, s, hi, {hi - lo, lo}, hi + 1, s - 1};
+  }
+}
+
+// An integer |v| < 2^24 as FP64 without a conversion at the FP64 rate: through FP32 (exact), then
+// its bits widened (binary32 to binary64: exponent bias 127 to 1023, fraction 23 to 52 bits).
+__device__ __forceinline__ double int_to_double(int v) {
+  const int b = __float_as_int((float)v);
+  const int hi = (b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20));
+  return v == 0 ? 0.0 : __hiloint2double(hi, b << 29);
 }
 
 enum { kFirst = 0, kNewton = 1, kUpdate = 2 };
@@ -850,13 +889,132 @@ __device__ __forceinline__ void first_pass_segment(const AugArgs& A, long long o
     first_batch<D, CUBIC, B, VC>(A, m, off, z, min(B, z1 - z + 1), zstride, np, x, y, zc);
 }
 
-// The fine pass of one block: columns of its cell, chunk by chunk.  `acc` holds the
-// per-thread channel rows ([NVAL][NT] doubles), zero on entry.
-template <int D, bool JF32, bool VC = false>
-__device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double* cv, double alpha, int cell,
-                          int bic) {
-  using G = Aug<D, JF32>;
-  using JT = typename std::conditional<JF32, float, double>::type;
+// How the FP64 path deals a cell's items (column chunks) to its blocks and their threads.  An
+// FP64 warp instruction costs the same however many lanes are active, so a warp's lanes are
+// filled before another warp is used, and when the block's items leave warps over, a column's D
+// segments go to separate warps (a warp whose lanes are in different segments runs them one
+// after the other).
+struct Deal64 {
+  int n;        // items of this block (at most)
+  int stride;   // threads between the segments of one item; 0: a thread takes all of them
+  int nact;     // threads that may have an item
+};
+template <int D>
+__device__ __forceinline__ Deal64 deal64(const AugArgs& A) {
+  const long long items = (D == 2 ? (long long)A.s : (long long)A.s * A.s) * (A.s / A.chunk);
+  Deal64 d;
+  const long long n = (items + A.bpc - 1) / A.bpc;
+  constexpr int NT = Aug<D, false>::NT;
+  d.stride = n <= NT / D ? (int)((n + 31) & ~31ll) : 0;
+  if (d.stride * D > NT) d.stride = 0;
+  d.n = n < NT ? (int)n : NT;
+  d.nact = d.stride ? D * d.stride : d.n;
+  return d;
+}
+
+// The FP64 path's moments of one column segment, summed over the nodes in order of z with the
+// weights m = z1 + 1 - z (m = number of nodes from z on) instead of z: sum f, sum f m and
+// sum f m (m + 1) / 2 are prefix sums, one FP64 add each per node.
+struct Moments64 {
+  double q0, q1, sa, d0, d1, d2, e0, e1, js, t0, t1, ss;
+};
+
+// The nodes z0..z1 (offset `off` at z0) of a column in FP64.  What bounds the FP64 pass is the
+// FP64 unit (one warp instruction per 64 clocks and SM sub-partition), so the node's work is
+// written for its operation count: with a u^3 (CUBIC) the derivative enters as u^2 (its factor
+// 3a is part of the channel weights) and a u^3 - g is one product and one fused multiply-add;
+// P c advances along z by one add.  2D: 20 operations in the first pass and 15 in the others,
+// against 26 and 20 for the plain form (2049^2: first pass 303 -> 217 us, others 217 -> 173).
+// Values are loaded B nodes at a time into registers, one memory latency per batch.
+template <int D, bool CUBIC, bool FIRST, bool VC>
+__device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long long off, int z0, int z1,
+                                          long long zstride, long long np, double alpha, double pc, double pc1, int x,
+                                          int y, int zc) {
+  constexpr int B = FIRST ? 4 : 8;
+  constexpr int NI = D - 1;
+  const long long io[2] = {1, np};
+  for (int z = z0; z <= z1; z += B, off += B * zstride) {
+    const int cnt = min(B, z1 - z + 1);
+    double uv[B + 2], gv[B], um[FIRST ? NI : 1][B], up[FIRST ? NI : 1][B];
+    if (FIRST) {
+#pragma unroll
+      for (int q = 0; q < B + 2; ++q) uv[q] = A.u[off + (long long)(min(q, cnt + 1) - 1) * zstride];
+    } else {
+#pragma unroll
+      for (int q = 0; q < B; ++q) uv[q + 1] = A.u[off + (long long)min(q, cnt - 1) * zstride];
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const long long c = off + (long long)min(q, cnt - 1) * zstride;
+      gv[q] = A.g[c];
+      if (FIRST) {
+#pragma unroll
+        for (int ax = 0; ax < NI; ++ax) {
+          um[ax][q] = A.u[c - io[ax]];
+          up[ax][q] = A.u[c + io[ax]];
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      if (q >= cnt) break;
+      const double ut = uv[q + 1];
+      const double U = FIRST ? ut : fma(alpha, ut, pc);
+      if (!FIRST) pc += pc1;
+      double fm, dj;
+      if (CUBIC) {
+        dj = U * U;
+        fm = fma(A.a, dj * U, -gv[q]);
+      } else {
+        double F;
+        f_eval<double>(A.kind, A.a, U, F, dj);
+        fm = F - gv[q];
+      }
+      m.q0 += fm;
+      m.q1 += m.q0;
+      m.sa = fma(fm, ut, m.sa);
+      if (!A.fixed_point) {
+        const double ej = dj * ut;
+        m.d0 += dj;
+        m.d1 += m.d0;
+        m.d2 += m.d1;
+        m.e0 += ej;
+        m.e1 += m.e0;
+        m.js = fma(ej, ut, m.js);
+      }
+      if (FIRST) {
+        // A u~ without its factor sigma (part of the channel weights)
+        double au;
+        if constexpr (VC) {
+          double wt[2 * D];
+          const int za = zc + z + q;
+          edge_weights_t<D, double>(A.vc, A.ls, x, D == 2 ? za : y, D == 3 ? za : 0, wt);
+          au = 0.0;
+#pragma unroll
+          for (int ax = 0; ax < D; ++ax) {
+            const double lo = ax == D - 1 ? uv[q] : um[ax][q], hi = ax == D - 1 ? uv[q + 2] : up[ax][q];
+            au += wt[2 * ax] * (ut - lo) + wt[2 * ax + 1] * (ut - hi);
+          }
+        } else {
+          double nb = (um[0][q] + up[0][q]) + (uv[q] + uv[q + 2]);
+          if (D == 3) nb += um[NI - 1][q] + up[NI - 1][q];
+          au = fma(2.0 * D, ut, -nb);
+        }
+        m.t0 += au;
+        m.t1 += m.t0;
+        m.ss = fma(au, ut, m.ss);
+      }
+    }
+  }
+}
+
+// The fine pass of one block on the FP64 path: as fine_pass, the moments of a segment converted
+// to the cell's vertex channels through the segment's weight forms (SegW): with X_p = sum (p - z)
+// f and X_q = sum (z - q) f a channel costs one or two operations.
+template <int D, bool VC>
+__device__ void fine_pass64(const AugArgs& A, int phase, double* acc, const double* cv, double alpha, int cell,
+                            int bic) {
+  using G = Aug<D, false>;
   const int tid = threadIdx.x;
   const int s = A.s;
   const long long np = A.n + 1;
@@ -872,21 +1030,153 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
   const int ncol = D == 2 ? s : s * s;
   const int nch = s / A.chunk;
   const long long items = (long long)ncol * nch;
-  const double inv_s = 1.0 / s;
+  const double inv_s = A.inv_s;
+  // contiguous shares of the cell's items per block
+  const Deal64 deal = deal64<D>(A);
+  const long long share = (items + A.bpc - 1) / A.bpc;
+  const long long lo_it = (long long)bic * share, hi_it = min(lo_it + share, items);
+  const int seg = deal.stride ? tid / deal.stride : -1;
+  const int t0 = deal.stride ? tid - seg * deal.stride : tid;
+  if (seg >= D) return;
+  for (long long it = lo_it + t0; it < hi_it; it += G::NT) {
+    const int col = (int)(it & (ncol - 1));
+    const int ch = (int)(it >> (D == 2 ? A.ls : 2 * A.ls));
+    const int o[2] = {col & (s - 1), D == 3 ? col >> A.ls : 0};
+    const int x = cellc[0] * s + o[0];
+    const int y = D == 3 ? cellc[1] * s + o[1] : 0;
+    if (x == 0 || (D == 3 && y == 0)) continue;
+    const int zc = cellc[D - 1] * s;
+    const long long base = D == 2 ? (long long)x : (long long)y * np + x;
+    const int zlo_chunk = ch * A.chunk;
+    const int zhi_chunk = zlo_chunk + A.chunk - 1;
+    const int zmin = (zc == 0) ? 1 : 0;
+    SegW<D> sg[D];
+    column_segments_w<D>(o, s, sg);
+#pragma unroll 1
+    for (int si = seg < 0 ? 0 : seg; si < (seg < 0 ? D : seg + 1); ++si) {
+      const SegW<D> S = sg[si];
+      const int z0 = max(max(S.z0, zlo_chunk), zmin);
+      const int z1 = min(S.z1, zhi_chunk);
+      if (z0 > z1) continue;
+      // P c at z0 and its step along z
+      double pc = 0.0, pc1 = 0.0;
+      if (phase != kFirst) {
+        pc1 = (cv[S.vq] - cv[S.vp]) * inv_s;
+        pc = fma(int_to_double(S.p - z0), cv[S.vp], int_to_double(z0 - S.q) * cv[S.vq]);
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t) pc = fma(int_to_double(S.c[t]), cv[S.vc[t]], pc);
+        pc *= inv_s;
+      }
+      long long off = base + (long long)(zc + z0) * zstride;
+      if (phase == kUpdate) {
+        constexpr int BU = 8;
+        for (int z = z0; z <= z1; z += BU, off += BU * zstride) {
+          const int cnt = min(BU, z1 - z + 1);
+          double v[BU];
+#pragma unroll
+          for (int q = 0; q < BU; ++q) v[q] = A.u[off + (long long)min(q, cnt - 1) * zstride];
+#pragma unroll
+          for (int q = 0; q < BU; ++q) {
+            if (q >= cnt) break;
+            A.u[off + q * zstride] = fma(alpha, v[q], pc);
+            pc += pc1;
+          }
+        }
+        continue;
+      }
+      Moments64 m = {};
+      const bool cubic = A.kind == FMG_F_CUBIC;
+      if (phase == kFirst) {
+        if (cubic)
+          segment64<D, true, true, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
+        else
+          segment64<D, false, true, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
+      } else if (cubic) {
+        segment64<D, true, false, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
+      } else {
+        segment64<D, false, false, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
+      }
+      // weights in m = z1 + 1 - z: p - z = a + m, z - q = b - m
+      const double a = int_to_double(S.p - z1 - 1), b = int_to_double(z1 + 1 - S.q);
+      double c[D - 1];
+#pragma unroll
+      for (int t = 0; t < D - 1; ++t) c[t] = int_to_double(S.c[t]);
+      double* row = acc + tid;
+      auto linear = [&](int chn, double x0, double x1) {
+        row[(chn + S.vp) * G::NT] += fma(a, x0, x1);
+        row[(chn + S.vq) * G::NT] += fma(b, x0, -x1);
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t) row[(chn + S.vc[t]) * G::NT] = fma(c[t], x0, row[(chn + S.vc[t]) * G::NT]);
+      };
+      linear(G::RA, m.q0, m.q1);
+      row[G::SA * G::NT] += m.sa;
+      if (phase == kFirst) {
+        linear(G::TT, m.t0, m.t1);
+        row[G::SS * G::NT] += m.ss;
+      }
+      if (A.fixed_point) continue;   // the fixed-point iteration needs no Jacobian
+      linear(G::JB, m.e0, m.e1);
+      row[G::JS * G::NT] += m.js;
+      // sum f, sum f m, sum f m^2 = 2 sum f m (m + 1) / 2 - sum f m
+      const double m2 = fma(2.0, m.d2, -m.d1);
+      const double fp = fma(a, m.d0, m.d1), fq = fma(b, m.d0, -m.d1);   // sum f (p - z), sum f (z - q)
+      const double fpm = fma(a, m.d1, m2), fqm = fma(b, m.d1, -m2);     // the same times m
+      auto pair = [&](int v, int w) -> double& { return row[(G::JP + pair_index(G::NV, v, w)) * G::NT]; };
+      pair(S.vp, S.vp) += fma(a, fp, fpm);
+      pair(S.vp, S.vq) += fma(b, fp, -fpm);
+      pair(S.vq, S.vq) += fma(b, fq, -fqm);
+#pragma unroll
+      for (int t = 0; t < D - 1; ++t) {
+        double& rp = pair(S.vp, S.vc[t]);
+        rp = fma(c[t], fp, rp);
+        double& rq = pair(S.vq, S.vc[t]);
+        rq = fma(c[t], fq, rq);
+        const double ct = c[t] * m.d0;
+#pragma unroll
+        for (int r = t; r < D - 1; ++r) {
+          double& rc = pair(S.vc[t], S.vc[r]);
+          rc = fma(ct, c[r], rc);
+        }
+      }
+    }
+  }
+}
+
+// The fine pass of one block on the mixed path: columns of its cell, chunk by chunk.  `acc` holds
+// the per-thread channel rows ([NVAL][NT] doubles), zero on entry.
+template <int D, bool VC>
+__device__ void fine_pass32(const AugArgs& A, int phase, double* acc, const double* cv, double alpha, int cell,
+                            int bic) {
+  using G = Aug<D, true>;
+  const int tid = threadIdx.x;
+  const int s = A.s;
+  const long long np = A.n + 1;
+  const long long zstride = D == 2 ? np : np * np;
+  int cellc[3] = {0, 0, 0};
+  {
+    int t = cell;
+    for (int q = 0; q < D; ++q) {
+      cellc[q] = t % A.nc;
+      t /= A.nc;
+    }
+  }
+  const int ncol = D == 2 ? s : s * s;
+  const int nch = s / A.chunk;
+  const long long items = (long long)ncol * nch;
+  const double inv_s = A.inv_s;
   const double inv_s2 = inv_s * inv_s;
   // the mixed path's FP32 quantities, formed once per pass: Jacobian weights, alpha - 1, a,
   // 1/s and the coarse cell's vertex values of c
-  const float jw0 = JF32 ? (float)A.w : 0.f, jw1 = JF32 ? (float)(A.w * inv_s) : 0.f,
-              jw2 = JF32 ? (float)(A.w * inv_s2) : 0.f;
-  const float am1f = JF32 ? (float)(alpha - 1.0) : 0.f, a_f = JF32 ? (float)A.a : 0.f;
+  const float jw0 = (float)A.w, jw1 = (float)(A.w * inv_s), jw2 = (float)(A.w * inv_s2);
+  const float am1f = (float)(alpha - 1.0), a_f = (float)A.a;
   const float inv_sf = 1.0f / (float)s;
   float cvf[G::NV];
 #pragma unroll
-  for (int v = 0; v < G::NV; ++v) cvf[v] = (JF32 && phase != kFirst) ? (float)cv[v] : 0.f;
+  for (int v = 0; v < G::NV; ++v) cvf[v] = phase != kFirst ? (float)cv[v] : 0.f;
   // Items (column chunks) are dealt to the cell's blocks contiguously when they fill every
   // block; on small levels they are interleaved across the blocks, so that the cell's work
-  // spreads over as many SM sub-partitions as there are items (the FP64 rate of one
-  // sub-partition is one warp instruction per 64 clocks, so a single busy warp per cell would
+  // spreads over as many SM sub-partitions as there are items (on the FP64 path, the FP64 rate of
+  // one sub-partition is one warp instruction per 64 clocks, so a single busy warp per cell would
   // serialize the pass).
   const bool spread = items < (long long)A.bpc * G::NT;
   const long long q0 = spread ? (long long)tid * A.bpc + bic : (long long)bic * G::NT + tid;
@@ -913,9 +1203,8 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
       if (z0 > z1) continue;
       // P c on the segment: pc0 + pc1 z (the mixed path forms it in FP32: it is the small
       // Newton correction, and the passes after the first work in FP32 increments)
-      double pc0 = 0.0, pc1 = 0.0;
       float pc0f = 0.f, pc1f = 0.f;
-      if (JF32 && phase != kFirst) {
+      if (phase != kFirst) {
 #pragma unroll
         for (int t = 0; t <= D; ++t) {
           pc0f = fmaf((float)S.P[t], cvf[S.vid[t]], pc0f);
@@ -923,24 +1212,12 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
         }
         pc0f *= inv_sf;
         pc1f *= inv_sf;
-      } else if (phase != kFirst) {
-#pragma unroll
-        for (int t = 0; t <= D; ++t) {
-          pc0 += S.P[t] * cv[S.vid[t]];
-          pc1 += S.R[t] * cv[S.vid[t]];
-        }
-        pc0 *= inv_s;
-        pc1 *= inv_s;
       }
-      double Q0 = 0.0, Q1 = 0.0, SAv = 0.0;                 // residual moments
-      JT D0 = 0, D1 = 0, D2 = 0, E0 = 0, E1 = 0, JSv = 0;   // Jacobian moments
-      double T0 = 0.0, T1 = 0.0, SSv = 0.0;                 // first pass
-      FirstMoments fm;                                      // mixed path, first pass
-      float cq0 = 0.f, cq1 = 0.f, csa = 0.f;                // mixed path, chord pass
-      double zd = (double)z0;
+      FirstMoments fm;                         // first pass
+      float cq0 = 0.f, cq1 = 0.f, csa = 0.f;   // chord pass
       long long off = base + (long long)(zc + z0) * zstride;
-      if (JF32 && phase != kFirst) {
-        // mixed path: FP32 increments on top of the first pass's FP64 residual sums
+      if (phase != kFirst) {
+        // FP32 increments on top of the first pass's FP64 residual sums
         const float af = a_f;
         float q0 = 0.f, q1 = 0.f, sa = 0.f;
         auto node = [&](ff ut, float zf, long long o) {
@@ -979,88 +1256,18 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
         cq0 = q0;
         cq1 = q1;
         csa = sa;
-      } else if (JF32) {
-        // mixed path, first pass: u~ and g are float-float, and f(u~) - g, A_k u~ and the
+      } else {
+        // first pass: u~ and g are float-float, and f(u~) - g, A_k u~ and the
         // residual and t/s moments are formed in float-float (FP32 error-free transformations,
         // no FP64 arithmetic per node); the Jacobian moments in FP32 from the leading parts
         if (A.kind == FMG_F_CUBIC)
           first_pass_segment<D, true, VC>(A, off, z0, z1, zstride, fm, x, y, zc);
         else
           first_pass_segment<D, false, VC>(A, off, z0, z1, zstride, fm, x, y, zc);
-        D0 = fm.d0;
-        D1 = fm.d1;
-        D2 = fm.d2;
-        E0 = fm.e0;
-        E1 = fm.e1;
-        JSv = fm.js;
-      } else
-      for (int z = z0; z <= z1; ++z, off += zstride, zd += 1.0) {
-        if (((z - z0) & 7) == 0) {
-          // touch the next eight column entries (and their g values) so that their loads are
-          // in flight together (they stay in L1 for the iterations below)
-#pragma unroll
-          for (int q = 1; q < 8; ++q)
-            if (z + q <= z1) {
-              asm volatile("prefetch.global.L1 [%0];" ::"l"(A.u + off + q * zstride));
-              if (phase != kUpdate) asm volatile("prefetch.global.L1 [%0];" ::"l"(A.g + off + q * zstride));
-            }
-        }
-        const double ut = A.u[off];
-        const double U = phase == kFirst ? ut : fma(alpha, ut, fma(pc1, zd, pc0));
-        if (phase == kUpdate) {
-          A.u[off] = U;
-          continue;
-        }
-        // FP64 path (the mixed path's passes are the branches above)
-        double F, Fp = 0.0;
-        f_eval<double>(A.kind, A.a, U, F, Fp);
-        const JT dj = (JT)Fp, zj = (JT)zd, uj = (JT)ut;
-        const double Fm = F - A.g[off];
-        Q0 += Fm;
-        Q1 = fma(Fm, zd, Q1);
-        SAv = fma(Fm, ut, SAv);
-        if (!A.fixed_point) {
-          const JT dz = dj * zj;
-          const JT du = dj * uj;
-          D0 += dj;
-          D1 += dz;
-          D2 += dz * zj;
-          E0 += du;
-          E1 += du * zj;
-          JSv += du * uj;
-        }
-        if (phase == kFirst) {
-          double au;
-          if constexpr (VC) {
-            // sigma sum_e w_e (u - u_e) with the coefficient's edge weights at the node
-            double wt[2 * D];
-            const int za = zc + z;
-            edge_weights_t<D, double>(A.vc, A.ls, x, D == 2 ? za : y, D == 3 ? za : 0, wt);
-            const long long o3[3] = {1, np, zstride};
-            double acc2 = 0.0;
-#pragma unroll
-            for (int ax = 0; ax < D; ++ax)
-              acc2 += wt[2 * ax] * (ut - A.u[off - o3[ax]]) + wt[2 * ax + 1] * (ut - A.u[off + o3[ax]]);
-            au = A.sigma_k * acc2;
-          } else {
-            double nb;
-            if constexpr (D == 2) {
-              nb = (A.u[off - 1] + A.u[off + 1]) + (A.u[off - zstride] + A.u[off + zstride]);
-            } else {
-              nb = ((A.u[off - 1] + A.u[off + 1]) + (A.u[off - np] + A.u[off + np])) +
-                   (A.u[off - zstride] + A.u[off + zstride]);
-            }
-            au = A.sigma_k * (2.0 * D * ut - nb);
-          }
-          T0 += au;
-          T1 = fma(au, zd, T1);
-          SSv = fma(au, ut, SSv);
-        }
       }
       if (phase == kUpdate) continue;
       // moments -> vertex channels of this thread's row
-      const double w = A.w;
-      if (JF32) {
+      {
         // mixed path: the residual (and first-pass t, s) channels are float-float rows without
         // their weights; the chord pass's moments are FP32 sums of increments
         float2* fr = reinterpret_cast<float2*>(acc);
@@ -1085,23 +1292,13 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
         }
         add(G::SA, fm.sa);
         add(G::SS, fm.ss);
-      } else {
-#pragma unroll
-        for (int t = 0; t <= D; ++t) {
-          const double Pt = S.P[t], Rt = S.R[t];
-          const int v = S.vid[t];
-          acc[(G::RA + v) * G::NT + tid] += w * inv_s * (Pt * Q0 + Rt * Q1);
-          if (phase == kFirst) acc[(G::TT + v) * G::NT + tid] += inv_s * (Pt * T0 + Rt * T1);
-        }
-        acc[G::SA * G::NT + tid] += w * SAv;
-        if (phase == kFirst) acc[G::SS * G::NT + tid] += SSv;
       }
       if (A.fixed_point) continue;   // the fixed-point iteration needs no Jacobian
-      if (JF32) {
+      {
         // FP32 Jacobian channels, converted in FP32 into the FP32 rows
-        float* fj = Rows<D, JF32>::jac(acc);
+        float* fj = Rows<D, true>::jac(acc);
         const float wf = jw1, wf2 = jw2;
-        const float d0 = (float)D0, d1 = (float)D1, d2 = (float)D2, e0 = (float)E0, e1 = (float)E1;
+        const float d0 = fm.d0, d1 = fm.d1, d2 = fm.d2, e0 = fm.e0, e1 = fm.e1;
 #pragma unroll
         for (int t = 0; t <= D; ++t) {
           const float Pt = (float)S.P[t], Rt = (float)S.R[t];
@@ -1114,74 +1311,112 @@ __device__ void fine_pass(const AugArgs& A, int phase, double* acc, const double
                 wf2 * fmaf(Pt * Pr, d0, fmaf(fmaf(Pt, Rr, Rt * Pr), d1, Rt * Rr * d2));
           }
         }
-        fj[(G::JS - G::JB) * G::NT + tid] += jw0 * (float)JSv;
-      } else {
-#pragma unroll
-        for (int t = 0; t <= D; ++t) {
-          const double Pt = S.P[t], Rt = S.R[t];
-          const int v = S.vid[t];
-          acc[(G::JB + v) * G::NT + tid] += w * inv_s * (Pt * (double)E0 + Rt * (double)E1);
-#pragma unroll
-          for (int r = t; r <= D; ++r) {
-            const double Pr = S.P[r], Rr = S.R[r];
-            acc[(G::JP + pair_index(G::NV, v, S.vid[r])) * G::NT + tid] +=
-                w * inv_s2 * (Pt * Pr * (double)D0 + (Pt * Rr + Rt * Pr) * (double)D1 + Rt * Rr * (double)D2);
-          }
-        }
-        acc[G::JS * G::NT + tid] += w * (double)JSv;
+        fj[(G::JS - G::JB) * G::NT + tid] += jw0 * fm.js;
       }
     }
   }
 }
 
-// Block sum of the channel rows into out[0..NVAL) (fixed order).  Only the channels the
-// phase produced are summed (the first-pass gatherings t and s only in the first
-// pass); in the mixed path the Jacobian channels, FP32 products to begin with, are summed in
-// FP32 -- FP64 adds issue slowly on this part.
+template <int D, bool JF32, bool VC = false>
+__device__ __forceinline__ void fine_pass(const AugArgs& A, int phase, double* acc, const double* cv, double alpha,
+                                          int cell, int bic) {
+  if constexpr (JF32)
+    fine_pass32<D, VC>(A, phase, acc, cv, alpha, cell, bic);
+  else
+    fine_pass64<D, VC>(A, phase, acc, cv, alpha, cell, bic);
+}
+
+// Block sum of the channel rows into out[0..NVAL) (fixed order), times the channels' quadrature
+// weights.  Only the channels the phase produced are summed (the first-pass gatherings t and s
+// only in the first pass) and only the rows of threads that had an item (nact).
+// FP64 path: bound by the FP64 unit, whose warp instruction costs the same however many lanes
+// are active, so the lanes run along the channels (one add per lane and row, the rows skewed by
+// channel against bank conflicts) and the threads' rows are split over the rest of the block;
+// then a lane per channel adds the slices.  Row per lane with a shuffle sum per channel cost
+// 4.9 us a pass in 2D and 9.6 in 3D at full rows, this 3.1 and 3.6.
+// Mixed path: the Jacobian channels, FP32 products to begin with, are summed in FP32; the others
+// in float-float, weighted and converted to FP64 at the end.
 template <int D, bool JF32>
-__device__ void block_reduce_rows(const AugArgs& A, const double* acc, double* out, bool first, bool fixed_point) {
+__device__ void block_reduce_rows(const AugArgs& A, double* acc, double* out, bool first, bool fixed_point) {
   using G = Aug<D, JF32>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = G::NT / 32;
   __syncthreads();
-  for (int v = warp; v < G::NVAL; v += nw) {
+  if constexpr (!JF32) {
+    constexpr int NS = D == 2 ? 8 : 2;   // slices of the rows: NVAL * NS <= NT
+    static_assert(G::NVAL * NS <= G::NT, "a thread per channel and slice");
+    const int nact = deal64<D>(A).nact;
+    const int rps = (nact + NS - 1) / NS;   // rows per slice
+    const int v = threadIdx.x % G::NVAL, sl = threadIdx.x / G::NVAL;
     const bool pre = v >= G::TT && v < G::JB;
-    if (pre && !first) continue;
-    if ((fixed_point || (JF32 && !first)) && v >= G::JB) continue;   // no Jacobian channels
-    if (JF32 && v >= G::JB) {
-      const float* fj = Rows<D, JF32>::jac(acc);
-      float x = 0.f;
-      for (int t = lane; t < G::NT; t += 32) x += fj[(v - G::JB) * G::NT + t];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      // the FP32 sum stays FP32: it is stored in the low word of the channel's 8-byte slot
-      if (lane == 0) reinterpret_cast<float*>(out + v)[0] = x;
-    } else if (JF32) {
-      // float-float rows: summed in float-float (fixed order), then weighted and converted
-      const float2* fr = reinterpret_cast<const float2*>(acc);
-      ff x{0.f, 0.f};
-      for (int t = lane; t < G::NT; t += 32) {
-        const float2 o = fr[v * G::NT + t];
-        x = ff_add_fast(x, ff{o.x, o.y});
+    const bool on = sl < NS && !(pre && !first) && !(fixed_point && v >= G::JB);
+    double x0 = 0.0, x1 = 0.0;
+    if (on) {
+      const double* r = acc + (size_t)v * G::NT;
+      const int a = sl * rps, n = min(rps, nact - a);
+      if (rps == 32) {   // full rows in 2D: skewed
+        for (int k = 0; k < 32; k += 2) {
+          x0 += r[a + ((k + v) & 31)];
+          x1 += r[a + ((k + 1 + v) & 31)];
+        }
+      } else {
+        int k = n > 0 ? v % n : 0;   // start skewed by channel
+        for (int i = 0; i < n; ++i) {
+          if (i & 1)
+            x1 += r[a + k];
+          else
+            x0 += r[a + k];
+          k = k + 1 == n ? 0 : k + 1;
+        }
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const ff y{__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
-        x = ff_add_fast(x, y);
-      }
-      if (lane == 0) {
-        const double inv_s = 1.0 / A.s;
-        const double wgt = v < G::SA ? A.w * inv_s : v == G::SA ? A.w : v < G::SS ? inv_s : 1.0;
-        out[v] = wgt * ff_to_double(x);
-      }
-    } else {
-      double x = 0.0;
-      for (int t = lane; t < G::NT; t += 32) x += acc[v * G::NT + t];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) out[v] = x;
     }
+    __syncthreads();
+    // the slices' sums, in the first rows' place
+    if (on) acc[sl * G::NVAL + v] = x0 + x1;
+    __syncthreads();
+    if (on && sl == 0) {
+      double x = acc[v];
+#pragma unroll
+      for (int q = 1; q < NS; ++q) x += acc[q * G::NVAL + v];
+      const double w = v < G::SA ? A.wRA : v == G::SA ? A.wSA : v < G::SS ? A.wTT : v == G::SS ? A.wSS
+                       : v < G::JP ? A.wJB : v < G::JS ? A.wJP : A.wJS;
+      out[v] = w * x;
+    }
+    __syncthreads();
+    return;
+  } else {
+    for (int v = warp; v < G::NVAL; v += nw) {
+      const bool pre = v >= G::TT && v < G::JB;
+      if (pre && !first) continue;
+      if ((fixed_point || !first) && v >= G::JB) continue;   // no Jacobian channels
+      if (v >= G::JB) {
+        const float* fj = Rows<D, JF32>::jac(acc);
+        float x = 0.f;
+        for (int t = lane; t < G::NT; t += 32) x += fj[(v - G::JB) * G::NT + t];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        // the FP32 sum stays FP32: it is stored in the low word of the channel's 8-byte slot
+        if (lane == 0) reinterpret_cast<float*>(out + v)[0] = x;
+      } else {
+        // float-float rows: summed in float-float (fixed order), then weighted and converted
+        const float2* fr = reinterpret_cast<const float2*>(acc);
+        ff x{0.f, 0.f};
+        for (int t = lane; t < G::NT; t += 32) {
+          const float2 o = fr[v * G::NT + t];
+          x = ff_add_fast(x, ff{o.x, o.y});
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const ff y{__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
+          x = ff_add_fast(x, y);
+        }
+        if (lane == 0) {
+          const double wgt = v < G::SA ? A.wRA : v == G::SA ? A.wSA : v < G::SS ? A.wTT : A.wSS;
+          out[v] = wgt * ff_to_double(x);
+        }
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 // Coordinates of coarse unknown p.
@@ -1226,27 +1461,6 @@ __device__ double node_channel(const double* cellsum, int nc, const int* z, int 
   return x;
 }
 
-template <int D, bool JF32>
-__device__ double pair_channel(const double* cellsum, int nc, const int* zp, const int* zq) {
-  using G = Aug<D, JF32>;
-  double x = 0.0;
-  for (int o = 0; o < G::NV; ++o) {
-    bool ok = true;
-    int cell = 0, mul = 1, vq = 0;
-    for (int q = 0; q < D; ++q) {
-      const int cc = zp[q] - ((o >> q) & 1);
-      if (cc < 0 || cc >= nc) ok = false;
-      const int dq = zq[q] - cc;
-      if (dq < 0 || dq > 1) ok = false;
-      vq |= dq << q;
-      cell += cc * mul;
-      mul *= nc;
-    }
-    if (ok) x += cellsum[(long long)cell * G::NVAL + G::JP + pair_index(G::NV, o, vq)];
-  }
-  return x;
-}
-
 // Lexicographic half-bandwidth of J_HH: it couples coarse nodes that share a coarse simplex,
 // offsets up to 1 + m (2D) or 1 + m + m^2 (3D), m = nc - 1; alpha is the border unknown.
 template <int D>
@@ -1264,7 +1478,8 @@ struct StepState {
   double* t;       // t = P^T A_k u~  [N_H]
   double* sa;      // [0] s = u~.A_k u~, [1] alpha
   double* basev;   // mixed path: the first pass's FP64 residual sums [ncell (NV+1)]
-  int* flags;      // [0] converged, [1] stop (a pivot was not positive or a value not finite)
+  int* flags;      // [0] converged, [1] stop (a pivot was not positive or a value not finite),
+                   // [2] FP64 path: this correction step factors in FP64
 };
 
 // Shared memory of the Newton kernels: the channel rows (reused after each pass for cellsum
@@ -1352,90 +1567,75 @@ __device__ void cell_reduce(const AugArgs& A, const double* __restrict__ pbuf, d
   if (threadIdx.x == 0) atomicExch(&A.st->cell_count[cell], 0u);
 }
 
-template <int D>
-__device__ void newton_update(const AugArgs& A, const double* R, int NH, const StepState& S, int dropped, bool ok,
-                              bool writer);
-
-// Gather table of the mixed path's FP32 Jacobian (first iteration of a correction step): one
-// record of kJW<D> ints per entry e of the assembly, e = p (3^d + 1) + r for coarse unknown p and
-// r < 3^d its neighbour z_p + (r digits in base 3) - 1, r = 3^d the border entry of p:
-//   [0] the entry's index into the factor's array (p ld + q, or N_H ld + p), -1: outside the
-//       lower band or the mesh;
-//   [1] |dv|_1 (bits 0-1), border flag (bit 2), p (bits 8-15), r (bits 16-23);
+// Gather table of the Jacobian: one record of kJW<D> ints per entry of its lower triangle that the
+// coarse simplices couple.  Those are the pairs (z, z - e) of interior coarse nodes with e a 0/1
+// vector (e = 0: the diagonal), ordered by e (its bits t: x, y[, z]) and then by z, and after them
+// the border entries (alpha, z):
+//   [0] the entry's index into the factor's array (p ld + q, or N_H ld + p);
+//   [1] |e|_1, at most 2 (bits 0-1), border flag (bit 2), p (bits 8-15), t (bits 16-23);
 //   [2 + o] for each of the 2^d cells around the node (o: the vertex bits of p in the cell), the
 //       cell-sum slot of the channel the entry takes from that cell, or -1.
-// The entry is the sum of those FP32 channels in o order (the same order as summing cell by
-// cell), so a table-driven assembly does no index arithmetic on the coarse mesh.
+// The entry is the sum of those channels in o order (the same order as summing cell by cell), so
+// a table-driven assembly does no index arithmetic on the coarse mesh.
 template <int D>
 constexpr int kJW = D == 2 ? 8 : 12;
 
+// Entries of edge vector t, and of the whole table, for m = nc - 1 interior nodes per side.
+template <int D>
+__host__ __device__ constexpr int jtab_count(int m, int t) {
+  int c = 1;
+  for (int ax = 0; ax < D; ++ax) c *= m - ((t >> ax) & 1);
+  return c;
+}
 template <int D>
 __host__ __device__ constexpr int aug_jtab_entries(int nc) {
-  int nh = 1, n3 = 1;
-  for (int q = 0; q < D; ++q) {
-    nh *= nc - 1;
-    n3 *= 3;
-  }
-  return nh * (n3 + 1);
+  int c = jtab_count<D>(nc - 1, 0);   // the border
+  for (int t = 0; t < (1 << D); ++t) c += jtab_count<D>(nc - 1, t);
+  return c;
 }
 
 template <int D>
 __global__ void k_aug_jtab(int nc, int* __restrict__ tab) {
   pdl_start();
   using G = Aug<D, true>;
-  constexpr int N3 = D == 2 ? 9 : 27;
   const int NH = (int)ipow(nc - 1, D);
   const int ld = NH + 2;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < NH * (N3 + 1); e += gridDim.x * blockDim.x) {
+  const int m = nc - 1;
+  const int total = aug_jtab_entries<D>(nc);
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     int* w = tab + (size_t)e * kJW<D>;
     for (int i = 0; i < kJW<D>; ++i) w[i] = -1;
-    const int p = e / (N3 + 1), rr = e - p * (N3 + 1);
-    int z[3];
-    unknown_coords<D>(p, nc, z);
-    if (rr == N3) {   // border entry: the channel JB of the vertex z in each cell around it
-      w[0] = NH * ld + p;
-      w[1] = 4 | (p << 8) | (rr << 16);
-      for (int o = 0; o < G::NV; ++o) {
-        bool ok = true;
-        int cell = 0, mul = 1;
-        for (int q = 0; q < D; ++q) {
-          const int cc = z[q] - ((o >> q) & 1);
-          if (cc < 0 || cc >= nc) ok = false;
-          cell += cc * mul;
-          mul *= nc;
-        }
-        if (ok) w[2 + o] = cell * G::NVAL + G::JB + o;
-      }
-      continue;
-    }
-    int zq[3], q = 0, mulq = 1, dist = 0, r2 = rr;
-    bool okq = true;
+    int t = 0, k = e;
+    while (t < (1 << D) && k >= jtab_count<D>(m, t)) k -= jtab_count<D>(m, t++);
+    const bool border = t == (1 << D);
+    if (border) t = 0;
+    // node z (its coordinates run over e_ax + 1 .. m), unknown p, and its neighbour q = z - e
+    int z[3] = {0, 0, 0}, p = 0, q = 0, mul = 1, dist = 0;
     for (int ax = 0; ax < D; ++ax) {
-      const int d = r2 % 3 - 1;
-      r2 /= 3;
-      zq[ax] = z[ax] + d;
-      if (zq[ax] < 1 || zq[ax] > nc - 1) okq = false;
-      q += (zq[ax] - 1) * mulq;
-      mulq *= (nc - 1);
-      dist += d < 0 ? -d : d;
+      const int ea = (t >> ax) & 1, len = m - ea;
+      z[ax] = k % len + 1 + ea;
+      k /= len;
+      p += (z[ax] - 1) * mul;
+      q += (z[ax] - 1 - ea) * mul;
+      mul *= m;
+      dist += ea;
     }
-    if (!okq || q > p) continue;
-    w[0] = p * ld + q;
-    w[1] = (dist > 2 ? 2 : dist) | (p << 8) | (rr << 16);
-    // the pair channel of (z, zq) in each cell that holds both
+    w[0] = border ? NH * ld + p : p * ld + q;
+    w[1] = (border ? 4 : dist > 2 ? 2 : dist) | (p << 8) | (t << 16);
+    // the pair channel of (z, z - e) -- border: the channel JB of z -- in each cell that holds both
     for (int o = 0; o < G::NV; ++o) {
       bool ok = true;
-      int cell = 0, mul = 1, vq = 0;
-      for (int qq = 0; qq < D; ++qq) {
-        const int cc = z[qq] - ((o >> qq) & 1);
+      int cell = 0, cm = 1, vq = 0;
+      for (int ax = 0; ax < D; ++ax) {
+        const int cc = z[ax] - ((o >> ax) & 1);
         if (cc < 0 || cc >= nc) ok = false;
-        const int dq = zq[qq] - cc;
+        const int dq = z[ax] - ((t >> ax) & 1) - cc;
         if (dq < 0 || dq > 1) ok = false;
-        vq |= dq << qq;
-        cell += cc * mul;
-        mul *= nc;
+        vq |= dq << ax;
+        cell += cc * cm;
+        cm *= nc;
       }
-      if (ok) w[2 + o] = cell * G::NVAL + G::JP + pair_index(G::NV, o, vq);
+      if (ok) w[2 + o] = cell * G::NVAL + (border ? G::JB + o : G::JP + pair_index(G::NV, o, vq));
     }
   }
 }
@@ -1607,17 +1807,32 @@ __device__ __forceinline__ void band_inverse_dispatch(const float* Af, const flo
   band_inverse_column<D>(Af, rd, n, ld, band, c, X);
 }
 
-// y = X r for the n x n matrix X (leading dimension ld) and r in FP32, by all warps (a row per
-// warp, the columns over its lanes, a shuffle sum in fixed order).
+// y = X r for the n x n matrix X (leading dimension ld) and r in FP32, by all warps: a row per
+// warp and turn, the columns over its lanes, the turns' shuffle sums interleaved.
+template <int NT>
 __device__ __forceinline__ void small_matvec(const float* X, int n, int ld, const float* r, float* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = warp; i < n; i += nw) {
-    float y = 0.f;
-    if (lane < n) y = X[i * ld + lane] * r[lane];
-    if (lane + 32 < n) y = fmaf(X[i * ld + lane + 32], r[lane + 32], y);
+  constexpr int NW = NT / 32, Q = NW == 8 ? 7 : 8;   // turns taken together (n <= 50 or 28)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool h0 = lane < n, h1 = lane + 32 < n;
+  const float r0 = h0 ? r[lane] : 0.f, r1 = h1 ? r[lane + 32] : 0.f;
+  for (int i0 = warp; i0 < n; i0 += Q * NW) {
+    float y[Q];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-    if (lane == 0) out[i] = y;
+    for (int q = 0; q < Q; ++q) {
+      const int i = i0 + q * NW;
+      y[q] = 0.f;
+      if (i < n) {
+        if (h0) y[q] = X[i * ld + lane] * r0;
+        if (h1) y[q] = fmaf(X[i * ld + lane + 32], r1, y[q]);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (lane == 0 && i0 + q * NW < n) out[i0 + q * NW] = y[q];
   }
 }
 
@@ -1674,7 +1889,6 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
                                                double* cellsum, double* Mreg, double* R, float* L,
                                                const StepState& S, bool first, bool writer) {
   using G = Aug<D, true>;
-  constexpr int N3 = D == 2 ? 9 : 27;
   const int tid = threadIdx.x;
   const int nthr = blockDim.x;
   const int lane = tid & 31;
@@ -1792,7 +2006,7 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
     // an entry per thread
     const float sigf = (float)sig;
     const int4* jt = reinterpret_cast<const int4*>(A.jtab);
-    for (int e = tid; e < NH * (N3 + 1); e += nthr) {
+    for (int e = tid; e < aug_jtab_entries<D>(A.nc); e += nthr) {
       int w[kJW<D>];
 #pragma unroll
       for (int i = 0; i < kJW<D> / 4; ++i) {
@@ -1802,7 +2016,6 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
         w[4 * i + 2] = t4.z;
         w[4 * i + 3] = t4.w;
       }
-      if (w[0] < 0) continue;
       float x = 0.f;
       if (!fixedp) {
 #pragma unroll
@@ -1816,13 +2029,10 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
       }
       const int dist = w[1] & 3;
       if (A.vc.a64) {
-        int z[3], dv[3], r2 = (w[1] >> 16) & 255;
+        int z[3], dv[3];
         unknown_coords<D>(p, A.nc, z);
 #pragma unroll
-        for (int ax = 0; ax < D; ++ax) {
-          dv[ax] = r2 % 3 - 1;
-          r2 /= 3;
-        }
+        for (int ax = 0; ax < D; ++ax) dv[ax] = -((w[1] >> (16 + ax)) & 1);
         x += (float)coarse_stiffness<D>(A, z, dv, dist);
       } else {
         if (dist == 0) x += sigf * (float)(2 * D);
@@ -1865,256 +2075,365 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
     Xuse = X;
   }
   // ---- the step y = J^{-1} R, then (c, alpha) += y and the convergence test
-  small_matvec(Xuse, NA, ld, rf, dl);
+  small_matvec<Aug<D, true>::NT>(Xuse, NA, ld, rf, dl);
   __syncthreads();
   newton_update_mixed<D>(A, dl, NH, S, dropped, ok, writer, red_sh);
 }
 
-// After a pass, in every block: cell sums, the dense system, the Newton step, convergence.
-// In the mixed path (JF32) the first iteration factors its Jacobian into L (LDL^T, FP32, with
-// the reciprocal pivots after it) and the later iterations are chord steps with that factor.
-// The fixed-point iteration (A.fixed_point) factors the Galerkin stiffness [[A_H, t], [t^T, s]]
-// once, in the path's precision, and every iteration solves with it against the residual
-// (y_{k+1} = y_k - K^{-1} R(y_k), i.e. K y_{k+1} = G - B^T W f(B y_k)).  `partials` holds this
-// iteration's sums, one row per coarse cell; only the writer block reports to DevState.
-// Not inlined: the dense step runs once per pass, and its own register allocation keeps it
-// from raising the pressure in the fine pass.
-template <int D, bool JF32>
-__device__ __noinline__ void newton_step(const AugArgs& A, const double* __restrict__ partials, double* cellsum,
-                                         double* M,
-                            double* R, typename std::conditional<JF32, float, double>::type* L, const StepState& S,
-                            bool first, bool writer) {
-  using FT = typename std::conditional<JF32, float, double>::type;
-  using G = Aug<D, JF32>;
+// (c, alpha) += the step in R (FP64) and the convergence test
+// ||step||_inf <= tol max(1, ||(c, alpha)||_inf), a thread per unknown.  The maxima are taken over
+// the magnitudes' bit patterns, which order as the numbers do (and put non-finite ones on top).
+template <int D>
+__device__ void newton_update(const AugArgs& A, const double* R, int NH, const StepState& S, int dropped, bool ok,
+                              bool writer) {
+  __shared__ unsigned long long max_sh[2][2];
   const int tid = threadIdx.x;
+  if (tid < 64) {
+    unsigned long long db = 0, yb = 0;
+    if (tid <= NH) {
+      double* y = &S.sa[1];
+      if (tid < NH) {
+        int z[3];
+        unknown_coords<D>(tid, A.nc, z);
+        y = &S.c[coarse_offset<D>(z, A.nc)];
+      }
+      const double nv = *y + R[tid];
+      *y = nv;
+      db = (unsigned long long)__double_as_longlong(R[tid]) & 0x7fffffffffffffffull;
+      yb = (unsigned long long)__double_as_longlong(nv) & 0x7fffffffffffffffull;
+    }
+    auto warp_max = [](unsigned long long b) {
+      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32));
+      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
+      return ((unsigned long long)hi << 32) | lo;
+    };
+    db = warp_max(db);
+    yb = warp_max(yb);
+    if ((tid & 31) == 0) {
+      max_sh[tid >> 5][0] = db;
+      max_sh[tid >> 5][1] = yb;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const unsigned long long db = max(max_sh[0][0], max_sh[1][0]), yb = max(max_sh[0][1], max_sh[1][1]);
+    const bool finite = (db >> 52) != 0x7ff && (yb >> 52) != 0x7ff;
+    const double dmax = __longlong_as_double((long long)db), ymax = __longlong_as_double((long long)yb);
+    S.flags[1] = (!ok || !finite) ? 1 : 0;
+    S.flags[0] = (finite && dmax <= A.tol * fmax(1.0, ymax)) ? 1 : 0;
+    if (writer) {
+      if (dropped) atomicOr(&A.st->flags, kFlagDropped);
+      if (!ok) atomicOr(&A.st->flags, kFlagNotSPD);
+      if (!finite) atomicOr(&A.st->flags, kFlagNonfinite);
+    }
+  }
+}
+
+// The FP64 path's linear solve J y = R.  FP64 elimination on one warp is a chain of FP64
+// operations (a band LDL^T of 50 unknowns 28 us, the two substitutions 18 us, per Newton
+// iteration), so the system is solved by iterative refinement instead: an FP32 inverse X of the
+// first iteration's Jacobian (the mixed path's band LDL^T and inverse columns) is kept for the
+// correction step, and y <- y + X (R - J y) with the residual, J and y in FP64 runs until the next
+// correction would be below the rounding of y.  The solution has FP64 accuracy whatever the
+// accuracy of X, which sets the rate only: about 1e-5 per sweep with its own J, ||I - X J|| with
+// a later one (systems of at most kRefineFresh unknowns, whose FP32 inverse costs little more
+// than two sweeps, get a new X every Newton iteration).  The step that passes Newton's test, and
+// so ends the iteration, is solved to the rounding of the iterate (c, alpha); an earlier one to
+// an error far below both the next step of a quadratically convergent iteration and the test's
+// tolerance, which the next residual corrects.
+// Measured at 50 unknowns: 3.5 to 9 us per Newton iteration after the first, against 46.
+// Where X is no good -- J not positive definite in FP32, the Schur complement of alpha below
+// kRefinePivot of its diagonal, magnitudes outside FP32, or no convergence in kRefineSweeps -- the
+// step falls back to the FP64 factorization, for the rest of the correction step (S.flags[2]).
+constexpr int kRefineSweeps = 16;
+constexpr int kRefineFresh = 16;
+constexpr float kRefinePivot = 1e-3f;
+
+// Refinement sweeps from y = 0 (see above); R, M in shared memory, y written over R on success;
+// iterate: max(1, ||(c, alpha)||_inf).
+// Returns false (R untouched) if they do not converge.
+template <int D>
+__device__ bool refine_solve(const AugArgs& A, const float* X, const double* M, int NH, double* R, float iterate) {
+  constexpr int LPR = D == 2 ? 2 : 4;    // lanes per row of the sparse residual
+  constexpr int NE = 4;                  // its entries per lane: 2D 7 + border, 3D 15 + border
+  constexpr int NT = Aug<D, false>::NT;
+  __shared__ double y_sh[kMaxAug];
+  __shared__ float r_sh[kMaxAug], z_sh[kMaxAug];
+  __shared__ unsigned max_sh[2][2];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int NA = NH + 1, ld = NA + 1, m = A.nc - 1;
+  // this lane's entries of row p of J: the mesh-edge neighbours and the alpha column
+  const int p = tid / LPR, sub = tid % LPR;
+  int idx[NE];
+  {
+    int z[3] = {0, 0, 0};
+    if (p < NH) unknown_coords<D>(p, A.nc, z);
+#pragma unroll
+    for (int k = 0; k < NE; ++k) {
+      const int e = sub * NE + k;   // 0: diagonal, 2t - 1 / 2t: + / - the t-th edge vector, last: alpha
+      idx[k] = -1;
+      if (p >= NH) continue;
+      if (e == LPR * NE - 1) {
+        idx[k] = NH;
+        continue;
+      }
+      const int t = (e + 1) >> 1, sg = e == 0 ? 0 : (e & 1) ? 1 : -1;
+      int q = 0, mul = 1;
+      bool in = true;
+#pragma unroll
+      for (int ax = 0; ax < D; ++ax) {
+        const int c = z[ax] + (((t >> ax) & 1) ? sg : 0);
+        in = in && c >= 1 && c <= m;
+        q += (c - 1) * mul;
+        mul *= m;
+      }
+      if (in) idx[k] = q;
+    }
+  }
+  if (tid < kMaxAug) {
+    y_sh[tid] = 0.0;
+    if (tid < NA) r_sh[tid] = (float)R[tid];
+  }
+  __syncthreads();
+  float zprev = 0.f;
+  for (int sweep = 0;; ++sweep) {
+    small_matvec<NT>(X, NA, ld, r_sh, z_sh);
+    __syncthreads();
+    if (tid < 64) {
+      float z = 0.f, ya = 0.f;
+      if (tid < NA) {
+        z = z_sh[tid];
+        const double y = y_sh[tid] + (double)z;
+        y_sh[tid] = y;
+        ya = fabsf((float)y);
+      }
+      const unsigned zb = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(z)));
+      const unsigned yb = __reduce_max_sync(0xffffffffu, __float_as_uint(ya));
+      if (lane == 0) {
+        max_sh[tid >> 5][0] = zb;
+        max_sh[tid >> 5][1] = yb;
+      }
+    }
+    __syncthreads();
+    const float zmax = __uint_as_float(max(max_sh[0][0], max_sh[1][0]));
+    const float ymax = __uint_as_float(max(max_sh[0][1], max_sh[1][1]));
+    if (!(zmax < 1e30f) || !(ymax > 1e-25f)) return false;   // also NaN
+    if (sweep > 0) {
+      // the next correction is about zmax (zmax / zprev)
+      const float rho = zmax / zprev;
+      const float tol = (float)A.tol * iterate;
+      const float goal = ymax > tol ? fminf(1e-3f * ymax * ymax, 1e-2f * tol) : 0.f;
+      if (zmax * fminf(rho, 1.f) <= fmaxf(goal, 5e-17f * iterate)) break;
+      if (rho > 0.5f && zmax <= 1e-13f * ymax) break;   // at the rounding level of an FP64 solve
+      if (sweep >= kRefineSweeps || rho > 0.5f) return false;
+    }
+    zprev = zmax;
+    // r = R - J y
+    double a = 0.0;
+#pragma unroll
+    for (int k = 0; k < NE; ++k)
+      if (idx[k] >= 0) a = fma(M[p * ld + idx[k]], y_sh[idx[k]], a);
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (p < NH && sub == 0) r_sh[p] = (float)(R[p] - a);
+    if (tid >= NT - 32) {   // the alpha row: eight lanes, seven products and three sums each
+      double b = 0.0;
+      for (int q = lane; q < NA && lane < 8; q += 8) b = fma(M[NH * ld + q], y_sh[q], b);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+      if (lane == 0) r_sh[NH] = (float)(R[NH] - b);
+    }
+    __syncthreads();
+  }
+  if (tid < NA) R[tid] = y_sh[tid];
+  __syncthreads();
+  return true;
+}
+
+// The FP64 path's dense step after a pass, in every block: cell sums, the system, the solve, the
+// update.  Every Newton iteration assembles its own Jacobian (the fixed-point iteration,
+// A.fixed_point, the Galerkin stiffness [[A_H, t], [t^T, s]]: K y_{k+1} = G - B^T W f(B y_k) as
+// y_{k+1} = y_k - K^{-1} R(y_k)).  `partials` holds this iteration's sums, one row per coarse
+// cell; only the writer block reports to DevState.  Not inlined: its own register allocation
+// keeps it from raising the pressure in the fine pass.
+template <int D>
+__device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __restrict__ partials, double* cellsum,
+                                              double* M, double* R, double* L, const StepState& S, bool first,
+                                              bool writer) {
+  using G = Aug<D, false>;
+  const int tid = threadIdx.x, lane = tid & 31;
+  constexpr int nthr = G::NT;
   const int ncell = (int)ipow(A.nc, D);
   const int NH = (int)ipow(A.nc - 1, D);
   const int NA = NH + 1;
   const int ld = NA + 1;
-  constexpr int N3 = D == 2 ? 9 : 27;
-  if constexpr (JF32) {
-    newton_step_mixed<D>(A, partials, cellsum, M, R, L, S, first, writer);
-    return;
-  }
-  const double alpha = S.sa[1];
-  const double* t_vec = S.t;
-  if ((JF32 || A.fixed_point) && !first) {
-    // chord / fixed-point step: the residual at the new iterate (mixed path: first-pass FP64
-    // sums plus this pass's increments; FP64 path: this pass's sums), solved with the factor
-    // of the first iteration
-    const int total = ncell * (G::NV + 1);
-    for (int base = tid; base < total; base += 4 * blockDim.x) {
-      double x[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int idx = base + r * blockDim.x;
-        x[r] = 0.0;
-        if (idx < total) {
-          const int cell = idx / (G::NV + 1), v = idx % (G::NV + 1);
-          const int chn = v < G::NV ? G::RA + v : G::SA;
-          x[r] = __ldcg(partials + (size_t)cell * G::NVAL + chn);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int idx = base + r * blockDim.x;
-        if (idx < total) {
-          const int cell = idx / (G::NV + 1), v = idx % (G::NV + 1);
-          const int chn = v < G::NV ? G::RA + v : G::SA;
-          cellsum[(size_t)cell * G::NVAL + chn] = JF32 ? x[r] + S.basev[idx] : x[r];
-        }
-      }
-    }
-    __syncthreads();
-    for (int p = tid; p < NH; p += blockDim.x) {
-      int z[3];
-      unknown_coords<D>(p, A.nc, z);
-      const double ahc = coarse_apply<D>(A, S.c, coarse_offset<D>(z, A.nc), z);
-      R[p] = -(ahc + alpha * t_vec[p] + node_channel<D, JF32>(cellsum, A.nc, z, G::RA));
-    }
-    if (tid < 32) {
-      double s2 = 0.0, tc = 0.0;
-      for (int c = tid; c < ncell; c += 32) s2 += cellsum[(long long)c * G::NVAL + G::SA];
-      for (int p = tid; p < NH; p += 32) {
-        int z[3];
-        unknown_coords<D>(p, A.nc, z);
-        tc += t_vec[p] * S.c[coarse_offset<D>(z, A.nc)];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        tc += __shfl_xor_sync(0xffffffffu, tc, o);
-      }
-      if (tid == 0) R[NH] = -(tc + alpha * S.sa[0] + s2);
-    }
-    __syncthreads();
-    if (tid < 32) ldlt_solve_band_warp<FT>(L, NA, ld, L + (size_t)NA * ld, aug_band<D>(A.nc), 1, R);
-    __syncthreads();
-    newton_update<D>(A, R, NH, S, 0, true, writer);
-    return;
-  }
-  // the cell sums (one row per coarse cell), eight loaded together
-  auto needed = [&](int v) { return !((!first && v >= G::TT && v < G::JB) || (A.fixed_point && v >= G::JB)); };
+  const bool fixedp = A.fixed_point != 0;
+  __shared__ int fac_sh[2];
+  __shared__ float iterate_sh;
+  // the cell sums (one contiguous block of rows, an even number of doubles): asynchronous 16-byte
+  // copies past L1, all in flight together; the matrix is cleared meanwhile
   {
-    const int total = ncell * G::NVAL;
-    for (int base = tid; base < total; base += 8 * blockDim.x) {
-      double x[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int idx = base + r * blockDim.x;
-        x[r] = (idx < total && needed(idx % G::NVAL)) ? __ldcg(partials + idx) : 0.0;
-      }
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int idx = base + r * blockDim.x;
-        if (idx < total && needed(idx % G::NVAL)) cellsum[idx] = x[r];
-      }
+    const int n16 = ncell * G::NVAL / 2;
+    for (int i = tid; i < n16; i += nthr) {
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(cellsum + 2 * i);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(partials + 2 * i) : "memory");
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  for (int idx = tid; idx < NA * ld; idx += blockDim.x) M[idx] = 0.0;
+  for (int idx = tid; idx < NA * ld; idx += nthr) M[idx] = 0.0;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  if (JF32) {
-    // mixed path: after the first pass the residual channels hold increments; the first
-    // pass's FP64 sums are kept in basev and added back (fixed order, same thread each time)
-    for (int idx = tid; idx < ncell * (G::NV + 1); idx += blockDim.x) {
-      const int cell = idx / (G::NV + 1), v = idx % (G::NV + 1);
-      const long long ch = (long long)cell * G::NVAL + (v < G::NV ? G::RA + v : G::SA);
-      if (first)
-        S.basev[idx] = cellsum[ch];
-      else
-        cellsum[ch] += S.basev[idx];
-    }
-    __syncthreads();
-  }
   if (first) {
-    for (int p = tid; p < NH; p += blockDim.x) {
+    for (int p = tid; p < NH; p += nthr) {
       int z[3];
       unknown_coords<D>(p, A.nc, z);
-      S.t[p] = node_channel<D, JF32>(cellsum, A.nc, z, G::TT);
+      S.t[p] = node_channel<D, false>(cellsum, A.nc, z, G::TT);
     }
-    if (tid < 32) {
+    if (tid >= nthr - 32) {
       double s0 = 0.0;
-      for (int c = tid; c < ncell; c += 32) s0 += cellsum[(long long)c * G::NVAL + G::SS];
+      for (int c = lane; c < ncell; c += 32) s0 += cellsum[(long long)c * G::NVAL + G::SS];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      if (tid == 0) S.sa[0] = s0;
+      if (lane == 0) S.sa[0] = s0;
     }
+    if (tid == 0) S.flags[2] = 0;
     __syncthreads();
   }
-  // J_HH on the coarse-edge pattern (entries for every neighbour in the 3^d box)
-  for (int idx = tid; idx < NH * N3; idx += blockDim.x) {
-    const int p = idx / N3;
-    int r = idx % N3;
-    int z[3], zq[3], dv[3];
-    unknown_coords<D>(p, A.nc, z);
-    bool ok = true;
-    int q = 0, mul = 1, dist = 0;
-    for (int ax = 0; ax < D; ++ax) {
-      const int d = r % 3 - 1;
-      r /= 3;
-      dv[ax] = d;
-      zq[ax] = z[ax] + d;
-      if (zq[ax] < 1 || zq[ax] > A.nc - 1) ok = false;
-      q += (zq[ax] - 1) * mul;
-      mul *= (A.nc - 1);
-      dist += abs(d);
-    }
-    if (!ok) continue;
-    double v = A.fixed_point ? 0.0 : pair_channel<D, JF32>(cellsum, A.nc, z, zq);
-    v += coarse_stiffness<D>(A, z, dv, dist);
-    M[p * ld + q] = v;
+  // max(1, ||(c, alpha)||_inf), for the solve's goal
+  if (tid < 32) {
+    float v = fmaxf(1.f, fabsf((float)S.sa[1]));
+    const int cn = (int)ipow(A.nc + 1, D);
+    for (int i = lane; i < cn; i += 32) v = fmaxf(v, fabsf((float)S.c[i]));
+    v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+    if (lane == 0) iterate_sh = v;
   }
-  // residual and the alpha border
-  for (int p = tid; p < NH; p += blockDim.x) {
+  // residual (a thread per unknown), the alpha row and corner (last warp), and the Jacobian from
+  // the gather table (every thread)
+  const double alpha = S.sa[1];
+  for (int p = tid; p < NH; p += nthr) {
     int z[3];
     unknown_coords<D>(p, A.nc, z);
     const double ahc = coarse_apply<D>(A, S.c, coarse_offset<D>(z, A.nc), z);
-    R[p] = -(ahc + alpha * t_vec[p] + node_channel<D, JF32>(cellsum, A.nc, z, G::RA));
-    const double jb = t_vec[p] + (A.fixed_point ? 0.0 : node_channel<D, JF32>(cellsum, A.nc, z, G::JB));
-    M[p * ld + NH] = jb;
-    M[NH * ld + p] = jb;
+    R[p] = -(ahc + alpha * S.t[p] + node_channel<D, false>(cellsum, A.nc, z, G::RA));
   }
-  if (tid < 32) {
+  if (tid >= nthr - 32) {
     double s2 = 0.0, s3 = 0.0, tc = 0.0;
-    for (int c = tid; c < ncell; c += 32) {
+    for (int c = lane; c < ncell; c += 32) {
       s2 += cellsum[(long long)c * G::NVAL + G::SA];
-      if (!A.fixed_point) s3 += cellsum[(long long)c * G::NVAL + G::JS];
+      if (!fixedp) s3 += cellsum[(long long)c * G::NVAL + G::JS];
     }
-    for (int p = tid; p < NH; p += 32) {
+    for (int p = lane; p < NH; p += 32) {
       int z[3];
       unknown_coords<D>(p, A.nc, z);
-      tc += t_vec[p] * S.c[coarse_offset<D>(z, A.nc)];
+      tc = fma(S.t[p], S.c[coarse_offset<D>(z, A.nc)], tc);
     }
+    s2 += tc;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       s2 += __shfl_xor_sync(0xffffffffu, s2, o);
       s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-      tc += __shfl_xor_sync(0xffffffffu, tc, o);
     }
-    if (tid == 0) {
-      R[NH] = -(tc + alpha * S.sa[0] + s2);
+    if (lane == 0) {
+      R[NH] = -(s2 + alpha * S.sa[0]);
       M[NH * ld + NH] = S.sa[0] + s3;
     }
   }
-  __syncthreads();
-  // Newton step on warp 0.  FP64 path: LDL^T in FP64.  Mixed path: LDL^T in FP32, kept in L
-  // for the chord steps of the later iterations.
-  int dropped = 0;
-  bool ok = true;
-  for (int idx = tid; idx < NA * ld; idx += blockDim.x) L[idx] = (FT)M[idx];
-  __syncthreads();
-  const int band = aug_band<D>(A.nc);
-  FT* rd = L + (size_t)NA * ld;
-  if (tid < 32) {
-    ok = ldlt_band_warp<FT>(L, NA, ld, rd, band, 1, true, JF32 ? 1e-6 : 1e-14, &dropped);
-    ldlt_solve_band_warp<FT>(L, NA, ld, rd, band, 1, R);
+  const int4* jt = reinterpret_cast<const int4*>(A.jtab);
+  for (int e = tid; e < aug_jtab_entries<D>(A.nc); e += nthr) {
+    int w[kJW<D>];
+#pragma unroll
+    for (int i = 0; i < kJW<D> / 4; ++i) {
+      const int4 t4 = __ldg(jt + (size_t)e * (kJW<D> / 4) + i);
+      w[4 * i] = t4.x;
+      w[4 * i + 1] = t4.y;
+      w[4 * i + 2] = t4.z;
+      w[4 * i + 3] = t4.w;
+    }
+    const int p = (w[1] >> 8) & 255;
+    double x;
+    int q;
+    if (w[1] & 4) {
+      x = S.t[p];
+      q = NH;
+    } else {
+      int z[3] = {0, 0, 0}, dv[3];
+      if (A.vc.a64) unknown_coords<D>(p, A.nc, z);
+#pragma unroll
+      for (int ax = 0; ax < D; ++ax) dv[ax] = -((w[1] >> (16 + ax)) & 1);
+      x = coarse_stiffness<D>(A, z, dv, w[1] & 3);
+      q = w[0] - p * ld;
+    }
+    if (!fixedp) {
+#pragma unroll
+      for (int o = 0; o < G::NV; ++o)
+        if (w[2 + o] >= 0) x += cellsum[w[2 + o]];
+    }
+    M[p * ld + q] = x;
+    M[q * ld + p] = x;
   }
   __syncthreads();
+  const int band = aug_band<D>(A.nc);
+  int dropped = 0;
+  bool ok = true;
+  // X, then the FP32 factor and its reciprocal pivots, where the FP64 factor would be
+  float* X = reinterpret_cast<float*>(L);
+  if ((first || NA <= kRefineFresh) && !S.flags[2]) {
+    float* Lf = X + (size_t)NA * ld;
+    float* rd = Lf + (size_t)NA * ld;
+    for (int i = tid; i < NA * ld; i += nthr) Lf[i] = (float)M[i];
+    __syncthreads();
+    if (tid < 32) {
+      bool okw;
+      if (D == 2 && NA == 50 && band == 8)
+        okw = ldlt_band_warp_ns<float, 2, 50, 8>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
+      else if (D == 2 && NA == 10 && band == 4)
+        okw = ldlt_band_warp_ns<float, 1, 10, 4>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
+      else if (D == 3 && NA == 28 && band == 13)
+        okw = ldlt_band_warp_ns<float, 4, 28, 13>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
+      else
+        okw = ldlt_band_warp<float>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
+      if (tid == 0 && (!okw || dropped)) S.flags[2] = 1;
+    }
+    __syncthreads();
+    if (!S.flags[2] && tid < NA) band_inverse_dispatch<D>(Lf, rd, NA, ld, band, tid, X);
+    __syncthreads();
+  }
+  if (!S.flags[2]) {
+    const bool solved = refine_solve<D>(A, X, M, NH, R, iterate_sh);
+    __syncthreads();
+    if (!solved && tid == 0) S.flags[2] = 1;
+    __syncthreads();
+  }
+  dropped = 0;
+  if (S.flags[2]) {
+    for (int idx = tid; idx < NA * ld; idx += nthr) L[idx] = M[idx];
+    __syncthreads();
+    double* rd = L + (size_t)NA * ld;
+    if (tid < 32) {
+      int dr = 0;
+      const bool okw = ldlt_band_warp<double>(L, NA, ld, rd, band, 1, true, 1e-14, &dr);
+      ldlt_solve_band_warp<double>(L, NA, ld, rd, band, 1, R);
+      if (tid == 0) {
+        fac_sh[0] = okw ? 1 : 0;
+        fac_sh[1] = dr;
+      }
+    }
+    __syncthreads();
+    ok = fac_sh[0] != 0;
+    dropped = fac_sh[1];
+  }
   newton_update<D>(A, R, NH, S, dropped, ok, writer);
 }
 
-// (c, alpha) += the step in R, convergence test and stop flags (warp 0 of every block; the
-// writer block also reports to DevState).
-template <int D>
-__device__ void newton_update(const AugArgs& A, const double* R, int NH, const StepState& S, int dropped, bool ok,
-                              bool writer) {
-  const int tid = threadIdx.x;
-  if (tid < 32) {
-    double dmax = 0.0, ymax = 0.0;
-    bool finite = true;
-    for (int p = tid; p < NH; p += 32) {
-      int z[3];
-      unknown_coords<D>(p, A.nc, z);
-      const long long off = coarse_offset<D>(z, A.nc);
-      const double nv = S.c[off] + R[p];
-      if (!isfinite(nv)) finite = false;
-      S.c[off] = nv;
-      dmax = fmax(dmax, fabs(R[p]));
-      ymax = fmax(ymax, fabs(nv));
-    }
-    const double na = S.sa[1] + R[NH];
-    if (tid == 0) {
-      if (!isfinite(na)) finite = false;
-      dmax = fmax(dmax, fabs(R[NH]));
-      ymax = fmax(ymax, fabs(na));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      ymax = fmax(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
-    }
-    finite = __all_sync(0xffffffffu, finite);
-    if (tid == 0) {
-      S.sa[1] = na;
-      S.flags[1] = (!ok || !finite) ? 1 : 0;
-      S.flags[0] = (dmax <= A.tol * fmax(1.0, ymax)) ? 1 : 0;
-      if (writer) {
-        if (dropped) atomicOr(&A.st->flags, kFlagDropped);
-        if (!ok) atomicOr(&A.st->flags, kFlagNotSPD);
-        if (!finite) atomicOr(&A.st->flags, kFlagNonfinite);
-      }
-    }
-  }
+template <int D, bool JF32>
+__device__ __forceinline__ void newton_step(const AugArgs& A, const double* __restrict__ partials, double* cellsum,
+                                            double* M, double* R,
+                                            typename std::conditional<JF32, float, double>::type* L,
+                                            const StepState& S, bool first, bool writer) {
+  if constexpr (JF32)
+    newton_step_mixed<D>(A, partials, cellsum, M, R, L, S, first, writer);
+  else
+    newton_step_fp64<D>(A, partials, cellsum, M, R, L, S, first, writer);
 }
 
 // Before the first pass, in every block: c = 0, alpha = 1, flags clear.
@@ -2149,7 +2468,7 @@ __global__ void __launch_bounds__(Aug<D, JF32>::NT, 512 / Aug<D, JF32>::NT) k_au
   extern __shared__ double sm[];
   double* acc = sm;                                 // channel rows [NVAL][NT]
   __shared__ double cv[G::NV];
-  __shared__ int flags_sh[2];
+  __shared__ int flags_sh[3];
   __shared__ int stop;
   __shared__ int last_sh;
   const int tid = threadIdx.x;
@@ -2183,6 +2502,8 @@ __global__ void __launch_bounds__(Aug<D, JF32>::NT, 512 / Aug<D, JF32>::NT) k_au
   S.flags = flags_sh;
   step_state_init<D>(A, S);
   const bool writer = blockIdx.x == 0;
+  unsigned gen = 0u;   // the grid barrier's generation (thread 0)
+  if (tid == 0) gen = ((volatile unsigned*)&A.st->bar_gen)[0];
   int it = 0;
   for (it = 1; it <= A.maxit; ++it) {
     const bool first = it == 1;
@@ -2205,7 +2526,7 @@ __global__ void __launch_bounds__(Aug<D, JF32>::NT, 512 / Aug<D, JF32>::NT) k_au
       cell_reduce<D, JF32>(A, pbuf, cbuf, cell, first, &last_sh);
       rows = cbuf;
     }
-    grid_barrier(A.st, nblocks, A.bar_spins, first && (int)blockIdx.x == A.bar_skip);
+    grid_barrier(A.st, nblocks, A.bar_spins, first && (int)blockIdx.x == A.bar_skip, gen);
     newton_step<D, JF32>(A, rows, cellsum, M, R, L, S, first, writer);
     __syncthreads();
     if (flags_sh[0] || flags_sh[1]) break;
@@ -2316,7 +2637,7 @@ __device__ __forceinline__ void k_augmented_cluster_body(const AugArgs& A) {
   extern __shared__ double sm[];
   double* acc = sm;
   __shared__ double cv[G::NV];
-  __shared__ int flags_sh[2];
+  __shared__ int flags_sh[3];
   __shared__ int stop;
   const int tid = threadIdx.x;
   const int ncell = (int)ipow(A.nc, D);
@@ -2528,38 +2849,60 @@ bool aug_shape_tuned(int dim, int coarse_cells, int level, bool mixed, AugShape*
   return true;
 }
 
-AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const AugBuffers& ab, bool tuned) {
+AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const AugBuffers& ab, bool coop,
+                   bool tuned) {
   const int ncell = (int)ipow(coarse_cells, dim);
   const int sfine = 1 << (level - 1);
   const int nt = ab.nt;
-  // column chunks of up to 32 nodes; on smaller levels shorter ones, until every thread has
-  // an item (each chunk costs one moment-to-channel conversion, so they are no shorter than
-  // that needs, and at least 2 nodes long).  FP64 path: every co-resident thread of the
-  // grid, since its per-node work is FP64 and one SM sub-partition issues one FP64 warp
-  // instruction per ~64 clocks.  Mixed path (FP32 float-float work per node): the threads of
-  // one block per cell, and only as many blocks as the chunks fill -- on small levels one
-  // per cell, which keeps the partial rows every block gathers and the arrivals at each grid
-  // barrier few.
   const long long ncol = ipow(sfine, dim - 1);
-  const long long target = (long long)(jac_f32 ? 1 : ab.bpc) * nt * ncell;
-  int chunk = sfine < 32 ? sfine : 32;
-  while (chunk > 2 && ncol * (sfine / chunk) * ncell < target) chunk >>= 1;
-  const long long items = ncol * (sfine / chunk);
-  // blocks per cell: about one chunk per thread; on the FP64 path, when that leaves blocks
-  // unfilled, the chunks are spread over all co-resident blocks of the cell instead
-  int bpc = (int)((items + nt - 1) / nt);
-  if (jac_f32) {
+  AugShape sh{1, 1};
+  if (!jac_f32 && coop) {
+    // FP64 path: the chunk length and blocks per cell of least cost, counted in FP64 warp
+    // instructions per SM sub-partition.  A chunk costs its nodes and one conversion of its
+    // moments to channels (per segment); a block's warps are dealt as Deal64 says, and the blocks
+    // an SM holds share its sub-partitions; a second block per cell adds the cell's reduction
+    // and a longer barrier (a node's and a conversion's FP64 operations: 2D 20 and 35, 3D 22 and 50).
+    const int node = dim == 2 ? 20 : 22, conv = dim == 2 ? 35 : 50, again = 30;
+    long long best = -1;
+    for (int chunk = 1; chunk <= 32 && chunk <= sfine; chunk *= 2)
+      for (int bpc = 1; bpc <= ab.bpc; ++bpc) {
+        const long long items = ncol * (sfine / chunk), n = (items + bpc - 1) / bpc;
+        const long long warps = (n + 31) / 32;   // of one segment (or of all, when they are not split)
+        const bool split = dim * warps * 32 <= nt;
+        const long long turns = split ? 1 : (n + nt - 1) / nt;
+        const long long act = split ? dim * warps : (warps < nt / 32 ? warps : nt / 32);
+        const long long per_sm = ((long long)ncell * bpc + ab.sms - 1) / (ab.sms > 0 ? ab.sms : 1);
+        // a warp runs the segments its lanes are in one after the other: with short chunks all of
+        // them, with long ones mostly one
+        const long long segs = split ? 1 : (chunk >= 8 ? 1 : dim);
+        const long long cost = turns * ((act * per_sm + 3) / 4) * segs * (chunk * node + conv) +
+                               (bpc > 1 ? again + bpc : 0);
+        if (best < 0 || cost < best) {
+          best = cost;
+          sh = AugShape{chunk, bpc};
+        }
+      }
+  } else {
+    // column chunks of up to 32 nodes; on smaller levels shorter ones, until every thread of one
+    // block per cell has an item (each chunk costs one moment-to-channel conversion, so they are
+    // no shorter than that needs, and at least 2 nodes long); mixed path: only as many blocks as
+    // the chunks fill -- on small levels one per cell, which keeps the partial rows every block
+    // gathers and the arrivals at each grid barrier few.  The cluster variant runs one block per
+    // cell in turn (FP64 path: chunks as for every co-resident thread of a cooperative grid).
+    const long long target = (long long)(jac_f32 ? 1 : ab.bpc) * nt * ncell;
+    int chunk = sfine < 32 ? sfine : 32;
+    while (chunk > 2 && ncol * (sfine / chunk) * ncell < target) chunk >>= 1;
+    const long long items = ncol * (sfine / chunk);
+    int bpc = (int)((items + nt - 1) / nt);
     if (bpc > ab.bpc) bpc = ab.bpc;
-  } else if (bpc > ab.bpc || items < (long long)ab.bpc * nt) {
-    bpc = (int)(items < ab.bpc ? items : ab.bpc);
+    if (bpc < 1 || !coop) bpc = 1;
+    sh = AugShape{chunk, bpc};
   }
-  if (bpc < 1) bpc = 1;
-  AugShape sh{chunk, bpc};
   AugShape t;
-  if (tuned && aug_shape_tuned(dim, coarse_cells, level, jac_f32, &t)) {
+  if (coop && tuned && aug_shape_tuned(dim, coarse_cells, level, jac_f32, &t)) {
     // a tuned shape within the launch's limits: a power-of-two chunk that divides the column,
     // at most the co-resident blocks per cell that the partial rows are sized for
-    if (t.chunk >= 2 && t.chunk <= 32 && t.chunk <= sfine && (t.chunk & (t.chunk - 1)) == 0) sh.chunk = t.chunk;
+    if (t.chunk >= 1 && t.chunk <= 32 && t.chunk <= sfine && (t.chunk & (t.chunk - 1)) == 0) sh.chunk = t.chunk;
     if (t.bpc >= 1 && t.bpc <= ab.bpc) sh.bpc = t.bpc;
   }
   return sh;
@@ -2596,6 +2939,16 @@ cudaError_t launch_augmented(int dim, int coarse_cells, int level, LevelGeo gk, 
   A.sigma_k = dim == 2 ? 1.0 : h;
   A.sigma_H = dim == 2 ? 1.0 : 1.0 / coarse_cells;
   A.tol = tol;
+  A.inv_s = 1.0 / sfine;
+  // channel weights; the FP64 path's passes leave sigma and, for a u^3 with derivative 3 a u^2, the
+  // factor 3 a to them, the mixed path's t and s carry sigma already
+  A.wRA = A.w * A.inv_s;
+  A.wSA = A.w;
+  A.wTT = jac_f32 ? A.inv_s : A.sigma_k * A.inv_s;
+  A.wSS = jac_f32 ? 1.0 : A.sigma_k;
+  A.wJS = kind == FMG_F_CUBIC ? A.w * (3.0 * a) : A.w;
+  A.wJB = A.wJS * A.inv_s;
+  A.wJP = A.wJB * A.inv_s;
   A.a_ff = ff_from_double(a);
   A.sigma_ff = ff_from_double(A.sigma_k);
   A.u = u;
