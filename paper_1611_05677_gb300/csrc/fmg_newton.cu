@@ -25,7 +25,12 @@
 // lambda_t = (P_t + R_t z)/s, and every sum the system needs is a combination of the
 // segment's moments sum X, sum X z, sum X z^2.  The thread accumulates those moments in
 // registers (FP64 for the residual; FP32 or FP64 for the Jacobian) and converts them to the
-// cell's vertex channels once per segment.  The residual sums carry f(U) - g, so G_H and gamma
+// cell's vertex channels once per segment.  The lanes of a warp walk neighbouring columns, whose
+// segments end at different z, so all walk the same z range (a chunk) with running moments, and a
+// lane keeps a copy of them where its segment ends: the segments' moments are differences of the
+// copies.  (A loop per segment runs as long as the longest lane's in each: up to twice the chunk in
+// 2D, three times in 3D.  Measured, loop per segment against this: mixed first pass at 257^3 719
+// and 496 us, at 2049^2 75 and 61; FP64 first pass at 129^3 380 and 239 us.)  The residual sums carry f(U) - g, so G_H and gamma
 // are never formed apart; the first pass also gathers t and s
 // (at (c, alpha) = (0, 1), U = u~), so no separate precompute pass is needed.
 //
@@ -842,8 +847,9 @@ __device__ __forceinline__ void first_node(const AugArgs& A, FirstMoments& m, ff
 // costs one memory latency; loads past the run (cnt < B) repeat its last valid node and their
 // nodes are not summed.
 template <int D, bool CUBIC, int B, bool VC>
-__device__ __forceinline__ void first_batch(const AugArgs& A, FirstMoments& m, long long off, int z, int cnt,
-                                            long long zstride, long long np, int x, int y, int zc) {
+__device__ __forceinline__ void first_batch(const AugArgs& A, FirstMoments& m, FirstMoments* snap, const int* zb,
+                                            long long off, int z, int cnt, long long zstride, long long np, int x,
+                                            int y, int zc) {
   constexpr int NI = D - 1;                  // in-plane axes: x (and y in 3D); the column is the last
   const long long io[2] = {1, np};
   ff uz[B + 2], gv[B], um[NI > 0 ? NI : 1][B], up[NI > 0 ? NI : 1][B];
@@ -871,22 +877,27 @@ __device__ __forceinline__ void first_batch(const AugArgs& A, FirstMoments& m, l
     nm[D - 1] = uz[q];
     nq[D - 1] = uz[q + 2];
     first_node<D, CUBIC, VC>(A, m, uz[q + 1], gv[q], nm, nq, z + q, x, y, zc);
+#pragma unroll
+    for (int t = 0; t < D - 1; ++t)
+      if (z + q == zb[t]) snap[t] = m;
   }
 }
 
 // The mixed first pass over the column nodes z0..z1 (offset `off` at z0), in register batches
 // of B nodes (B smaller in 3D, whose nodes have two more in-plane neighbours to hold).  x, y:
 // the column's fine in-plane coordinates; zc: the fine z of local z = 0 (the coefficient's
-// edge weights need the node's position).
+// edge weights need the node's position); zb: where the column's segments end (snap: the moments
+// up to there).
 template <int D, bool CUBIC, bool VC>
-__device__ __forceinline__ void first_pass_segment(const AugArgs& A, long long off, int z0, int z1,
-                                                   long long zstride, FirstMoments& m, int x, int y, int zc) {
+__device__ __forceinline__ void first_pass_run(const AugArgs& A, long long off, int z0, int z1, long long zstride,
+                                               FirstMoments& m, FirstMoments* snap, const int* zb, int x, int y,
+                                               int zc) {
   constexpr int B = D == 2 ? 8 : 4;
   const long long np = A.n + 1;
   m.q0 = m.q1 = m.sa = m.t0 = m.t1 = m.ss = ff{0.f, 0.f};
   m.d0 = m.d1 = m.d2 = m.e0 = m.e1 = m.js = 0.f;
   for (int z = z0; z <= z1; z += B, off += B * zstride)
-    first_batch<D, CUBIC, B, VC>(A, m, off, z, min(B, z1 - z + 1), zstride, np, x, y, zc);
+    first_batch<D, CUBIC, B, VC>(A, m, snap, zb, off, z, min(B, z1 - z + 1), zstride, np, x, y, zc);
 }
 
 // How the FP64 path deals a cell's items (column chunks) to its blocks and their threads.  An
@@ -912,24 +923,28 @@ __device__ __forceinline__ Deal64 deal64(const AugArgs& A) {
   return d;
 }
 
-// The FP64 path's moments of one column segment, summed over the nodes in order of z with the
-// weights m = z1 + 1 - z (m = number of nodes from z on) instead of z: sum f, sum f m and
-// sum f m (m + 1) / 2 are prefix sums, one FP64 add each per node.
+// The FP64 path's running moments of a column chunk, summed over the nodes in order of z with the
+// weights m = number of nodes from z to the last one summed: sum f, sum f m and sum f m (m + 1) / 2
+// are prefix sums, one FP64 add each per node.
 struct Moments64 {
-  double q0, q1, sa, d0, d1, d2, e0, e1, js, t0, t1, ss;
+  double q0, q1, d0, d1, d2, e0, e1, t0, t1;
+};
+struct Totals64 {
+  double sa, js, ss;   // the sums over the chunk that need no vertex weights
 };
 
 // The nodes z0..z1 (offset `off` at z0) of a column in FP64.  What bounds the FP64 pass is the
 // FP64 unit (one warp instruction per 64 clocks and SM sub-partition), so the node's work is
 // written for its operation count: with a u^3 (CUBIC) the derivative enters as u^2 (its factor
 // 3a is part of the channel weights) and a u^3 - g is one product and one fused multiply-add;
-// P c advances along z by one add.  2D: 20 operations in the first pass and 15 in the others,
-// against 26 and 20 for the plain form (2049^2: first pass 303 -> 217 us, others 217 -> 173).
-// Values are loaded B nodes at a time into registers, one memory latency per batch.
+// P c (pc at z0) advances along z by one add of the segment's slope.  2D: 20 operations in the first
+// pass and 15 in the others, against 26 and 20 for the plain form (2049^2: first pass 303 -> 193
+// us, others 217 -> 153, the running moments included).  Values are loaded B nodes at a time into registers, one memory latency
+// per batch.  zb: where the column's segments end (snap: the moments up to there).
 template <int D, bool CUBIC, bool FIRST, bool VC>
-__device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long long off, int z0, int z1,
-                                          long long zstride, long long np, double alpha, double pc, double pc1, int x,
-                                          int y, int zc) {
+__device__ __forceinline__ void run64(const AugArgs& A, Moments64& m, Totals64& tot, Moments64* snap, const int* zb,
+                                      long long off, int z0, int z1, long long zstride, long long np, double alpha,
+                                      double pc, const double* slope, int x, int y, int zc) {
   constexpr int B = FIRST ? 4 : 8;
   constexpr int NI = D - 1;
   const long long io[2] = {1, np};
@@ -960,7 +975,13 @@ __device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long l
       if (q >= cnt) break;
       const double ut = uv[q + 1];
       const double U = FIRST ? ut : fma(alpha, ut, pc);
-      if (!FIRST) pc += pc1;
+      if (!FIRST) {
+        double sl = slope[0];
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t)
+          if (z + q >= zb[t]) sl = slope[t + 1];
+        pc += sl;
+      }
       double fm, dj;
       if (CUBIC) {
         dj = U * U;
@@ -972,7 +993,7 @@ __device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long l
       }
       m.q0 += fm;
       m.q1 += m.q0;
-      m.sa = fma(fm, ut, m.sa);
+      tot.sa = fma(fm, ut, tot.sa);
       if (!A.fixed_point) {
         const double ej = dj * ut;
         m.d0 += dj;
@@ -980,7 +1001,7 @@ __device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long l
         m.d2 += m.d1;
         m.e0 += ej;
         m.e1 += m.e0;
-        m.js = fma(ej, ut, m.js);
+        tot.js = fma(ej, ut, tot.js);
       }
       if (FIRST) {
         // A u~ without its factor sigma (part of the channel weights)
@@ -1002,13 +1023,16 @@ __device__ __forceinline__ void segment64(const AugArgs& A, Moments64& m, long l
         }
         m.t0 += au;
         m.t1 += m.t0;
-        m.ss = fma(au, ut, m.ss);
+        tot.ss = fma(au, ut, tot.ss);
       }
+#pragma unroll
+      for (int t = 0; t < D - 1; ++t)
+        if (z + q == zb[t]) snap[t] = m;
     }
   }
 }
 
-// The fine pass of one block on the FP64 path: as fine_pass, the moments of a segment converted
+// The fine pass of one block on the FP64 path: as fine_pass32, the moments of a segment converted
 // to the cell's vertex channels through the segment's weight forms (SegW): with X_p = sum (p - z)
 // f and X_q = sum (z - q) f a channel costs one or two operations.
 template <int D, bool VC>
@@ -1047,80 +1071,113 @@ __device__ void fine_pass64(const AugArgs& A, int phase, double* acc, const doub
     if (x == 0 || (D == 3 && y == 0)) continue;
     const int zc = cellc[D - 1] * s;
     const long long base = D == 2 ? (long long)x : (long long)y * np + x;
-    const int zlo_chunk = ch * A.chunk;
-    const int zhi_chunk = zlo_chunk + A.chunk - 1;
-    const int zmin = (zc == 0) ? 1 : 0;
+    int za = max(ch * A.chunk, zc == 0 ? 1 : 0);   // z = 0 is the boundary face
+    int ze = ch * A.chunk + A.chunk - 1;
     SegW<D> sg[D];
     column_segments_w<D>(o, s, sg);
-#pragma unroll 1
-    for (int si = seg < 0 ? 0 : seg; si < (seg < 0 ? D : seg + 1); ++si) {
-      const SegW<D> S = sg[si];
-      const int z0 = max(max(S.z0, zlo_chunk), zmin);
-      const int z1 = min(S.z1, zhi_chunk);
-      if (z0 > z1) continue;
-      // P c at z0 and its step along z
-      double pc = 0.0, pc1 = 0.0;
-      if (phase != kFirst) {
-        pc1 = (cv[S.vq] - cv[S.vp]) * inv_s;
-        pc = fma(int_to_double(S.p - z0), cv[S.vp], int_to_double(z0 - S.q) * cv[S.vq]);
+    if (seg >= 0) {   // this thread's segment only
+      za = max(za, sg[seg].z0);
+      ze = min(ze, sg[seg].z1);
+    }
+    if (za > ze) continue;
+    int zb[D - 1];
 #pragma unroll
-        for (int t = 0; t < D - 1; ++t) pc = fma(int_to_double(S.c[t]), cv[S.vc[t]], pc);
-        pc *= inv_s;
+    for (int t = 0; t < D - 1; ++t) zb[t] = sg[t].z1;
+    // P c at za and its slopes
+    double pc = 0.0, slope[D];
+    if (phase != kFirst) {
+      SegW<D> S = sg[0];
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        slope[t] = (cv[sg[t].vq] - cv[sg[t].vp]) * inv_s;
+        if (t > 0 && za > zb[t - 1]) S = sg[t];
       }
-      long long off = base + (long long)(zc + z0) * zstride;
-      if (phase == kUpdate) {
-        constexpr int BU = 8;
-        for (int z = z0; z <= z1; z += BU, off += BU * zstride) {
-          const int cnt = min(BU, z1 - z + 1);
-          double v[BU];
+      pc = fma(int_to_double(S.p - za), cv[S.vp], int_to_double(za - S.q) * cv[S.vq]);
 #pragma unroll
-          for (int q = 0; q < BU; ++q) v[q] = A.u[off + (long long)min(q, cnt - 1) * zstride];
+      for (int t = 0; t < D - 1; ++t) pc = fma(int_to_double(S.c[t]), cv[S.vc[t]], pc);
+      pc *= inv_s;
+    }
+    long long off = base + (long long)(zc + za) * zstride;
+    if (phase == kUpdate) {
+      constexpr int BU = 8;
+      for (int z = za; z <= ze; z += BU, off += BU * zstride) {
+        const int cnt = min(BU, ze - z + 1);
+        double v[BU];
 #pragma unroll
-          for (int q = 0; q < BU; ++q) {
-            if (q >= cnt) break;
-            A.u[off + q * zstride] = fma(alpha, v[q], pc);
-            pc += pc1;
-          }
+        for (int q = 0; q < BU; ++q) v[q] = A.u[off + (long long)min(q, cnt - 1) * zstride];
+#pragma unroll
+        for (int q = 0; q < BU; ++q) {
+          if (q >= cnt) break;
+          A.u[off + q * zstride] = fma(alpha, v[q], pc);
+          double sl = slope[0];
+#pragma unroll
+          for (int t = 0; t < D - 1; ++t)
+            if (z + q >= zb[t]) sl = slope[t + 1];
+          pc += sl;
         }
-        continue;
       }
-      Moments64 m = {};
-      const bool cubic = A.kind == FMG_F_CUBIC;
-      if (phase == kFirst) {
-        if (cubic)
-          segment64<D, true, true, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
-        else
-          segment64<D, false, true, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
-      } else if (cubic) {
-        segment64<D, true, false, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
-      } else {
-        segment64<D, false, false, VC>(A, m, off, z0, z1, zstride, np, alpha, pc, pc1, x, y, zc);
+      continue;
+    }
+    Moments64 m = {}, snap[D - 1];
+    Totals64 tot = {};
+    const bool cubic = A.kind == FMG_F_CUBIC;
+    if (phase == kFirst) {
+      if (cubic)
+        run64<D, true, true, VC>(A, m, tot, snap, zb, off, za, ze, zstride, np, alpha, pc, slope, x, y, zc);
+      else
+        run64<D, false, true, VC>(A, m, tot, snap, zb, off, za, ze, zstride, np, alpha, pc, slope, x, y, zc);
+    } else if (cubic) {
+      run64<D, true, false, VC>(A, m, tot, snap, zb, off, za, ze, zstride, np, alpha, pc, slope, x, y, zc);
+    } else {
+      run64<D, false, false, VC>(A, m, tot, snap, zb, off, za, ze, zstride, np, alpha, pc, slope, x, y, zc);
+    }
+    double* row = acc + tid;
+    row[G::SA * G::NT] += tot.sa;
+    if (phase == kFirst) row[G::SS * G::NT] += tot.ss;
+    if (!A.fixed_point) row[G::JS * G::NT] += tot.js;
+#pragma unroll
+    for (int si = 0; si < D; ++si) {
+      const SegW<D> S = sg[si];
+      const int z0 = max(S.z0, za), z1 = min(S.z1, ze);
+      if (z0 > z1) continue;
+      // the segment's own moments: the running ones at z1 less the earlier segments' part
+      Moments64 g = (si < D - 1 && z1 < ze) ? snap[si < D - 1 ? si : 0] : m;
+      if (si > 0 && z0 > za) {
+        const Moments64& h = snap[si > 0 ? si - 1 : 0];
+        const double k = int_to_double(z1 - z0 + 1), k2 = int_to_double(((z1 - z0 + 1) * (z1 - z0 + 2)) >> 1);
+        g.q1 -= fma(k, h.q0, h.q1);
+        g.q0 -= h.q0;
+        if (phase == kFirst) {
+          g.t1 -= fma(k, h.t0, h.t1);
+          g.t0 -= h.t0;
+        }
+        if (!A.fixed_point) {
+          g.e1 -= fma(k, h.e0, h.e1);
+          g.e0 -= h.e0;
+          g.d2 -= fma(k2, h.d0, fma(k, h.d1, h.d2));
+          g.d1 -= fma(k, h.d0, h.d1);
+          g.d0 -= h.d0;
+        }
       }
       // weights in m = z1 + 1 - z: p - z = a + m, z - q = b - m
       const double a = int_to_double(S.p - z1 - 1), b = int_to_double(z1 + 1 - S.q);
       double c[D - 1];
 #pragma unroll
       for (int t = 0; t < D - 1; ++t) c[t] = int_to_double(S.c[t]);
-      double* row = acc + tid;
       auto linear = [&](int chn, double x0, double x1) {
         row[(chn + S.vp) * G::NT] += fma(a, x0, x1);
         row[(chn + S.vq) * G::NT] += fma(b, x0, -x1);
 #pragma unroll
         for (int t = 0; t < D - 1; ++t) row[(chn + S.vc[t]) * G::NT] = fma(c[t], x0, row[(chn + S.vc[t]) * G::NT]);
       };
-      linear(G::RA, m.q0, m.q1);
-      row[G::SA * G::NT] += m.sa;
-      if (phase == kFirst) {
-        linear(G::TT, m.t0, m.t1);
-        row[G::SS * G::NT] += m.ss;
-      }
+      linear(G::RA, g.q0, g.q1);
+      if (phase == kFirst) linear(G::TT, g.t0, g.t1);
       if (A.fixed_point) continue;   // the fixed-point iteration needs no Jacobian
-      linear(G::JB, m.e0, m.e1);
-      row[G::JS * G::NT] += m.js;
+      linear(G::JB, g.e0, g.e1);
       // sum f, sum f m, sum f m^2 = 2 sum f m (m + 1) / 2 - sum f m
-      const double m2 = fma(2.0, m.d2, -m.d1);
-      const double fp = fma(a, m.d0, m.d1), fq = fma(b, m.d0, -m.d1);   // sum f (p - z), sum f (z - q)
-      const double fpm = fma(a, m.d1, m2), fqm = fma(b, m.d1, -m2);     // the same times m
+      const double m2 = fma(2.0, g.d2, -g.d1);
+      const double fp = fma(a, g.d0, g.d1), fq = fma(b, g.d0, -g.d1);   // sum f (p - z), sum f (z - q)
+      const double fpm = fma(a, g.d1, m2), fqm = fma(b, g.d1, -m2);     // the same times m
       auto pair = [&](int v, int w) -> double& { return row[(G::JP + pair_index(G::NV, v, w)) * G::NT]; };
       pair(S.vp, S.vp) += fma(a, fp, fpm);
       pair(S.vp, S.vq) += fma(b, fp, -fpm);
@@ -1131,7 +1188,7 @@ __device__ void fine_pass64(const AugArgs& A, int phase, double* acc, const doub
         rp = fma(c[t], fp, rp);
         double& rq = pair(S.vq, S.vc[t]);
         rq = fma(c[t], fq, rq);
-        const double ct = c[t] * m.d0;
+        const double ct = c[t] * g.d0;
 #pragma unroll
         for (int r = t; r < D - 1; ++r) {
           double& rc = pair(S.vc[t], S.vc[r]);
@@ -1191,127 +1248,162 @@ __device__ void fine_pass32(const AugArgs& A, int phase, double* acc, const doub
     if (x == 0 || (D == 3 && y == 0)) continue;
     const int zc = cellc[D - 1] * s;                   // fine z of local offset 0
     const long long base = D == 2 ? (long long)x : (long long)y * np + x;
-    const int zlo_chunk = ch * A.chunk;
-    const int zhi_chunk = zlo_chunk + A.chunk - 1;
-    const int zmin = (zc == 0) ? 1 : 0;                // z = 0 is the boundary face
+    const int za = max(ch * A.chunk, zc == 0 ? 1 : 0);   // z = 0 is the boundary face
+    const int ze = ch * A.chunk + A.chunk - 1;
+    if (za > ze) continue;
     Seg<D> sg[D];
-    const int nseg = column_segments<D>(o, s, sg);
-    for (int si = 0; si < nseg; ++si) {
-      const Seg<D>& S = sg[si];
-      const int z0 = max(max(S.z0, zlo_chunk), zmin);
-      const int z1 = min(S.z1, zhi_chunk);
-      if (z0 > z1) continue;
-      // P c on the segment: pc0 + pc1 z (the mixed path forms it in FP32: it is the small
-      // Newton correction, and the passes after the first work in FP32 increments)
-      float pc0f = 0.f, pc1f = 0.f;
-      if (phase != kFirst) {
+    column_segments<D>(o, s, sg);
+    int zb[D - 1];   // the last z of each segment but the last one
+#pragma unroll
+    for (int t = 0; t < D - 1; ++t) zb[t] = sg[t].z1;
+    long long off = base + (long long)(zc + za) * zstride;
+    FirstMoments fm, fsnap[D - 1];                             // first pass
+    float cq0 = 0.f, cq1 = 0.f, csa = 0.f, cs0[D - 1], cs1[D - 1];   // chord pass
+    if (phase != kFirst) {
+      // P c on segment t: pc0 + pc1 z, in FP32 (it is the small Newton correction, and the passes
+      // after the first work in FP32 increments on top of the first pass's residual sums)
+      float pc0f[D], pc1f[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        pc0f[k] = pc1f[k] = 0.f;
 #pragma unroll
         for (int t = 0; t <= D; ++t) {
-          pc0f = fmaf((float)S.P[t], cvf[S.vid[t]], pc0f);
-          pc1f = fmaf((float)S.R[t], cvf[S.vid[t]], pc1f);
+          pc0f[k] = fmaf((float)sg[k].P[t], cvf[sg[k].vid[t]], pc0f[k]);
+          pc1f[k] = fmaf((float)sg[k].R[t], cvf[sg[k].vid[t]], pc1f[k]);
         }
-        pc0f *= inv_sf;
-        pc1f *= inv_sf;
+        pc0f[k] *= inv_sf;
+        pc1f[k] *= inv_sf;
       }
-      FirstMoments fm;                         // first pass
-      float cq0 = 0.f, cq1 = 0.f, csa = 0.f;   // chord pass
-      long long off = base + (long long)(zc + z0) * zstride;
-      if (phase != kFirst) {
-        // FP32 increments on top of the first pass's FP64 residual sums
-        const float af = a_f;
-        float q0 = 0.f, q1 = 0.f, sa = 0.f;
-        auto node = [&](ff ut, float zf, long long o) {
-          const float utf = ut.hi;
-          const float dl = fmaf(am1f, utf, fmaf(pc1f, zf, pc0f));
-          if (phase == kUpdate) {
-            const ff un = ff_add_f(ut, dl);
-            if (A.out_f64)
-              A.u[o] = ff_to_double_fast(un);
-            else
-              ff_store(A.u + o, un);
-            return;
-          }
-          // chord step: the Jacobian of the first pass is reused, so only the residual
-          // increments are summed here
-          float dF, fp;
-          delta_f(A.kind, A.a, ut, utf, dl, af, dF, fp);
-          q0 += dF;
-          q1 = fmaf(dF, zf, q1);
-          sa = fmaf(dF, utf, sa);
-        };
-        // sixteen independent loads in flight before the arithmetic, one memory latency per
-        // batch; loads past the run repeat its last node and are not processed
-        constexpr int BU = 16;
-        for (int z = z0; z <= z1; z += BU, off += BU * zstride) {
-          const int cnt = min(BU, z1 - z + 1);
-          ff v[BU];
+      const float af = a_f;
+      float q0 = 0.f, q1 = 0.f, sa = 0.f;
+      auto node = [&](ff ut, int z, long long o) {
+        const float utf = ut.hi, zf = (float)z;
+        float p0 = pc0f[0], p1 = pc1f[0];
 #pragma unroll
-          for (int q = 0; q < BU; ++q) v[q] = ff_load(A.u + off + (long long)min(q, cnt - 1) * zstride);
-#pragma unroll
-          for (int q = 0; q < BU; ++q) {
-            if (q >= cnt) break;
-            node(v[q], (float)(z + q), off + q * zstride);
+        for (int t = 0; t < D - 1; ++t)
+          if (z > zb[t]) {
+            p0 = pc0f[t + 1];
+            p1 = pc1f[t + 1];
           }
+        const float dl = fmaf(am1f, utf, fmaf(p1, zf, p0));
+        if (phase == kUpdate) {
+          const ff un = ff_add_f(ut, dl);
+          if (A.out_f64)
+            A.u[o] = ff_to_double_fast(un);
+          else
+            ff_store(A.u + o, un);
+          return;
         }
-        cq0 = q0;
-        cq1 = q1;
-        csa = sa;
-      } else {
-        // first pass: u~ and g are float-float, and f(u~) - g, A_k u~ and the
-        // residual and t/s moments are formed in float-float (FP32 error-free transformations,
-        // no FP64 arithmetic per node); the Jacobian moments in FP32 from the leading parts
-        if (A.kind == FMG_F_CUBIC)
-          first_pass_segment<D, true, VC>(A, off, z0, z1, zstride, fm, x, y, zc);
-        else
-          first_pass_segment<D, false, VC>(A, off, z0, z1, zstride, fm, x, y, zc);
+        // chord step: the Jacobian of the first pass is reused, so only the residual
+        // increments are summed here
+        float dF, fp;
+        delta_f(A.kind, A.a, ut, utf, dl, af, dF, fp);
+        q0 += dF;
+        q1 = fmaf(dF, zf, q1);
+        sa = fmaf(dF, utf, sa);
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t)
+          if (z == zb[t]) {
+            cs0[t] = q0;
+            cs1[t] = q1;
+          }
+      };
+      // sixteen independent loads in flight before the arithmetic, one memory latency per
+      // batch; loads past the run repeat its last node and are not processed
+      constexpr int BU = 16;
+      for (int z = za; z <= ze; z += BU, off += BU * zstride) {
+        const int cnt = min(BU, ze - z + 1);
+        ff v[BU];
+#pragma unroll
+        for (int q = 0; q < BU; ++q) v[q] = ff_load(A.u + off + (long long)min(q, cnt - 1) * zstride);
+#pragma unroll
+        for (int q = 0; q < BU; ++q) {
+          if (q >= cnt) break;
+          node(v[q], z + q, off + q * zstride);
+        }
       }
       if (phase == kUpdate) continue;
-      // moments -> vertex channels of this thread's row
-      {
-        // mixed path: the residual (and first-pass t, s) channels are float-float rows without
-        // their weights; the chord pass's moments are FP32 sums of increments
-        float2* fr = reinterpret_cast<float2*>(acc);
-        auto add = [&](int ch, ff x) {
-          const float2 o = fr[ch * G::NT + tid];
-          const ff r = ff_add_fast(ff{o.x, o.y}, x);
-          fr[ch * G::NT + tid] = make_float2(r.hi, r.lo);
-        };
-        if (phase != kFirst) {
+      cq0 = q0;
+      cq1 = q1;
+      csa = sa;
+    } else {
+      // first pass: u~ and g are float-float, and f(u~) - g, A_k u~ and the
+      // residual and t/s moments are formed in float-float (FP32 error-free transformations,
+      // no FP64 arithmetic per node); the Jacobian moments in FP32 from the leading parts
+      if (A.kind == FMG_F_CUBIC)
+        first_pass_run<D, true, VC>(A, off, za, ze, zstride, fm, fsnap, zb, x, y, zc);
+      else
+        first_pass_run<D, false, VC>(A, off, za, ze, zstride, fm, fsnap, zb, x, y, zc);
+    }
+    // moments -> vertex channels of this thread's row.  The residual (and first-pass t, s)
+    // channels are float-float rows without their weights; the chord pass's moments are FP32 sums
+    // of increments
+    float2* fr = reinterpret_cast<float2*>(acc);
+    auto add = [&](int ch, ff x) {
+      const float2 o = fr[ch * G::NT + tid];
+      const ff r = ff_add_fast(ff{o.x, o.y}, x);
+      fr[ch * G::NT + tid] = make_float2(r.hi, r.lo);
+    };
+    float* fj = Rows<D, true>::jac(acc);
+    if (phase == kFirst) {
+      add(G::SA, fm.sa);
+      add(G::SS, fm.ss);
+      if (!A.fixed_point) fj[(G::JS - G::JB) * G::NT + tid] += jw0 * fm.js;
+    } else {
+      add(G::SA, ff{csa, 0.f});
+    }
 #pragma unroll
-          for (int t = 0; t <= D; ++t)
-            add(G::RA + S.vid[t], ff{fmaf((float)S.P[t], cq0, (float)S.R[t] * cq1), 0.f});
-          add(G::SA, ff{csa, 0.f});
-          continue;
+    for (int si = 0; si < D; ++si) {
+      const Seg<D>& S = sg[si];
+      const int z0 = max(S.z0, za), z1 = min(S.z1, ze);
+      if (z0 > z1) continue;
+      const bool cut = si < D - 1 && z1 < ze;   // the segment ends inside the chunk
+      const bool cont = si > 0 && z0 > za;      // and begins inside it
+      constexpr int L1 = D - 2;
+      if (phase != kFirst) {
+        float q0 = cut ? cs0[si < L1 ? si : L1] : cq0, q1 = cut ? cs1[si < L1 ? si : L1] : cq1;
+        if (cont) {
+          q0 -= cs0[si > 0 ? si - 1 : 0];
+          q1 -= cs1[si > 0 ? si - 1 : 0];
         }
 #pragma unroll
-        for (int t = 0; t <= D; ++t) {
-          const float Pt = (float)S.P[t], Rt = (float)S.R[t];
-          const int v = S.vid[t];
-          add(G::RA + v, ff_add(ff_mul_f(fm.q0, Pt), ff_mul_f(fm.q1, Rt)));
-          add(G::TT + v, ff_add(ff_mul_f(fm.t0, Pt), ff_mul_f(fm.t1, Rt)));
-        }
-        add(G::SA, fm.sa);
-        add(G::SS, fm.ss);
+        for (int t = 0; t <= D; ++t)
+          add(G::RA + S.vid[t], ff{fmaf((float)S.P[t], q0, (float)S.R[t] * q1), 0.f});
+        continue;
+      }
+      FirstMoments g = cut ? fsnap[si < L1 ? si : L1] : fm;
+      if (cont) {
+        const FirstMoments& h = fsnap[si > 0 ? si - 1 : 0];
+        g.q0 = ff_sub(g.q0, h.q0);
+        g.q1 = ff_sub(g.q1, h.q1);
+        g.t0 = ff_sub(g.t0, h.t0);
+        g.t1 = ff_sub(g.t1, h.t1);
+        g.d0 -= h.d0;
+        g.d1 -= h.d1;
+        g.d2 -= h.d2;
+        g.e0 -= h.e0;
+        g.e1 -= h.e1;
+      }
+#pragma unroll
+      for (int t = 0; t <= D; ++t) {
+        const float Pt = (float)S.P[t], Rt = (float)S.R[t];
+        const int v = S.vid[t];
+        add(G::RA + v, ff_add(ff_mul_f(g.q0, Pt), ff_mul_f(g.q1, Rt)));
+        add(G::TT + v, ff_add(ff_mul_f(g.t0, Pt), ff_mul_f(g.t1, Rt)));
       }
       if (A.fixed_point) continue;   // the fixed-point iteration needs no Jacobian
-      {
-        // FP32 Jacobian channels, converted in FP32 into the FP32 rows
-        float* fj = Rows<D, true>::jac(acc);
-        const float wf = jw1, wf2 = jw2;
-        const float d0 = fm.d0, d1 = fm.d1, d2 = fm.d2, e0 = fm.e0, e1 = fm.e1;
+      // FP32 Jacobian channels, converted in FP32 into the FP32 rows
 #pragma unroll
-        for (int t = 0; t <= D; ++t) {
-          const float Pt = (float)S.P[t], Rt = (float)S.R[t];
-          const int v = S.vid[t];
-          fj[(G::JB - G::JB + v) * G::NT + tid] += wf * fmaf(Pt, e0, Rt * e1);
+      for (int t = 0; t <= D; ++t) {
+        const float Pt = (float)S.P[t], Rt = (float)S.R[t];
+        const int v = S.vid[t];
+        fj[(G::JB - G::JB + v) * G::NT + tid] += jw1 * fmaf(Pt, g.e0, Rt * g.e1);
 #pragma unroll
-          for (int r = t; r <= D; ++r) {
-            const float Pr = (float)S.P[r], Rr = (float)S.R[r];
-            fj[(G::JP - G::JB + pair_index(G::NV, v, S.vid[r])) * G::NT + tid] +=
-                wf2 * fmaf(Pt * Pr, d0, fmaf(fmaf(Pt, Rr, Rt * Pr), d1, Rt * Rr * d2));
-          }
+        for (int r = t; r <= D; ++r) {
+          const float Pr = (float)S.P[r], Rr = (float)S.R[r];
+          fj[(G::JP - G::JB + pair_index(G::NV, v, S.vid[r])) * G::NT + tid] +=
+              jw2 * fmaf(Pt * Pr, g.d0, fmaf(fmaf(Pt, Rr, Rt * Pr), g.d1, Rt * Rr * g.d2));
         }
-        fj[(G::JS - G::JB) * G::NT + tid] += jw0 * fm.js;
       }
     }
   }
@@ -2872,10 +2964,8 @@ AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const Aug
         const long long turns = split ? 1 : (n + nt - 1) / nt;
         const long long act = split ? dim * warps : (warps < nt / 32 ? warps : nt / 32);
         const long long per_sm = ((long long)ncell * bpc + ab.sms - 1) / (ab.sms > 0 ? ab.sms : 1);
-        // a warp runs the segments its lanes are in one after the other: with short chunks all of
-        // them, with long ones mostly one
-        const long long segs = split ? 1 : (chunk >= 8 ? 1 : dim);
-        const long long cost = turns * ((act * per_sm + 3) / 4) * segs * (chunk * node + conv) +
+        // (a warp whose lanes' chunks hold parts of several segments converts each)
+        const long long cost = turns * ((act * per_sm + 3) / 4) * (chunk * node + (split ? 1 : 2) * conv) +
                                (bpc > 1 ? again + bpc : 0);
         if (best < 0 || cost < best) {
           best = cost;
