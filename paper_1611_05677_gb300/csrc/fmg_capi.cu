@@ -33,7 +33,8 @@ struct fmg_ctx {
   float* u32b[kMaxLevels] = {};   // second FP32 buffer: output of the fused pre-smoothing kernel,
                                   // or the Chebyshev smoother's second iterate (mixed path)
   float* d32[kMaxLevels] = {};    // Chebyshev step direction (mixed path)
-  double* ua[kMaxLevels] = {};    // Chebyshev second iterate and direction (FP64 path and ops)
+  double* ua[kMaxLevels] = {};    // Chebyshev second iterate and direction (FP64 path and ops); ua also
+                                  // the second iterate of the FP64 red-black tile kernels
   double* dd[kMaxLevels] = {};
   ChebCoef cheb = {};
   double* Ainv = nullptr;
@@ -167,6 +168,9 @@ size_t layout(fmg_ctx* c, const fmg_params* p, char* base) {
     if (cheb) {
       ua = (double*)take(nodes * 8);
       dd = (double*)take(nodes * 8);
+    } else if (p->precision == FMG_PREC_FP64 && !p->coefficient && n > coarse_cycle_cells(p->dim) &&
+               fused_rb64_supported(p->dim, n, p->nu_pre, p->nu_post)) {
+      ua = (double*)take(nodes * 8);   // the tile kernels' second iterate
     }
     if (c && base) {
       c->u[k] = u;
@@ -335,6 +339,8 @@ bool fused_cycle_used(const fmg_ctx* c, int k) {
   return c->u32b[k - 1] && c->p.smoother == FMG_SMOOTHER_RBGS && !c->vc.a64;
 }
 
+// started: the level's first step from zero (Chebyshev step 0, or the red half of the first
+// red-black sweep) was taken by the restriction that produced b.
 cudaError_t vcycle(fmg_ctx* c, int j, double* u, const double* b, bool top = false, bool started = false) {
   const int dim = c->p.dim;
   cudaStream_t s = c->stream;
@@ -343,27 +349,50 @@ cudaError_t vcycle(fmg_ctx* c, int j, double* u, const double* b, bool top = fal
     return cudaSuccess;
   }
   if (j <= coarse_cycle_top(c)) {
-    // below the top level the restriction has zeroed u
+    // below the top level the cycle starts from zero
     TRY(launch_coarse_cycle<double>(dim, c->p.coarse_cells, j, u, b, c->p.nu_pre, c->p.nu_post, c->Ainv, nullptr,
                                     cheb_coef(c), !top, s, vcp(c)));
     return cudaSuccess;
   }
   const LevelGeo gf = c->geo[j - 1], gc = c->geo[j - 2];
   const bool cheb = c->p.smoother == FMG_SMOOTHER_CHEBYSHEV;
+  // the next level from zero in one launch of its own: its start buffer is not read
+  auto own_start = [&](int k) { return k <= coarse_cycle_top(c) || (!cheb && c->ua[k - 1]); };
+  if (!cheb && c->ua[j - 1]) {
+    int slot = -1;
+    if (top) TRY(tbegin(c, FMG_KT_PRE_TOP, j, &slot));
+    TRY(launch_pre_rb64(gf, c->p.nu_pre, top ? u : nullptr, b, c->ua[j - 1], c->b[j - 2], s));
+    TRY(tend(c, slot));
+    TRY(vcycle(c, j - 1, c->u[j - 2], c->b[j - 2]));
+    slot = -1;
+    if (top) TRY(tbegin(c, FMG_KT_POST_TOP, j, &slot));
+    TRY(launch_post_rb64(gf, c->p.nu_post, c->ua[j - 1], c->u[j - 2], b, u, s));
+    return tend(c, slot);
+  }
   if (cheb) TRY(cheb_steps<double>(c, j, u, c->ua[j - 1], c->dd[j - 1], b, c->p.nu_pre, top, started ? 1 : 0));
   for (int it = 0; !cheb && it < c->p.nu_pre; ++it) {
     int slot = -1;
     if (top) TRY(tbegin(c, FMG_KT_SMOOTH_TOP, j, &slot));
-    TRY(launch_rbgs<double>(dim, gf, u, b, 0, s, vcp(c)));
+    if (it > 0 || !started) TRY(launch_rbgs<double>(dim, gf, u, b, 0, s, vcp(c)));
     TRY(launch_rbgs<double>(dim, gf, u, b, 1, s, vcp(c)));
     TRY(tend(c, slot));
   }
-  const bool fuse = fuse_first_step(c, j - 1);
-  double* uc0 = fuse ? cheb_start(c->u[j - 2], c->ua[j - 2], c->p.nu_pre) : c->u[j - 2];
-  TRY(launch_residual_restrict<double, double>(dim, gf, u, b, gc, c->b[j - 2], uc0, s,
-                                               fuse ? c->dd[j - 2] : nullptr, fuse ? cheb_e0(c, j - 1) : 0.0, vcp(c)));
+  bool fuse = false;
+  if (!cheb && !vcp(c) && c->p.nu_pre >= 1) {
+    fuse = !own_start(j - 1);
+    TRY(launch_restrict_rb64(dim, gf, u, b, gc, c->b[j - 2], c->u[j - 2], fuse, s));
+  } else {
+    fuse = fuse_first_step(c, j - 1);
+    double* uc0 = fuse ? cheb_start(c->u[j - 2], c->ua[j - 2], c->p.nu_pre) : c->u[j - 2];
+    TRY(launch_residual_restrict<double, double>(dim, gf, u, b, gc, c->b[j - 2], uc0, s,
+                                                 fuse ? c->dd[j - 2] : nullptr, fuse ? cheb_e0(c, j - 1) : 0.0,
+                                                 vcp(c)));
+  }
   TRY(vcycle(c, j - 1, c->u[j - 2], c->b[j - 2], false, fuse));
-  TRY(launch_prolong<double, double>(dim, gc, c->u[j - 2], gf, u, 1, s));
+  if (!cheb && c->p.nu_post >= 1)
+    TRY(launch_prolong_rb64(dim, gc, c->u[j - 2], gf, u, s));
+  else
+    TRY(launch_prolong<double, double>(dim, gc, c->u[j - 2], gf, u, 1, s));
   if (cheb) TRY(cheb_steps<double>(c, j, u, c->ua[j - 1], c->dd[j - 1], b, c->p.nu_post, top));
   for (int it = 0; !cheb && it < c->p.nu_post; ++it) {
     int slot = -1;
@@ -491,13 +520,18 @@ cudaError_t top_cycle_ff(fmg_ctx* c, int k, double* u, const double* b, bool res
 }
 
 // Algorithm 3.1 at level k >= 2 on the level-k array u (FP64 contexts).
-cudaError_t correction_step(fmg_ctx* c, int k, double* u) {
+// from_coarse: u starts as the FMG interpolation of level k-1, formed here together with b.
+cudaError_t correction_step(fmg_ctx* c, int k, double* u, bool from_coarse = false) {
   if (c->p.precision == FMG_PREC_MIXED) return cudaErrorInvalidValue;
   const LevelGeo g = c->geo[k - 1];
   int slot_step = -1, slot_aug = -1;
   TRY(tbegin(c, FMG_KT_CORRECTION, k, &slot_step));
   // step 1: b = (g, v) - (f(x, u^{(l)}), v)   (eq. 3.4)
-  TRY(launch_nonlinear_rhs(c->p.dim, g, u, c->g[k - 1], c->b[k - 1], c->p.f, c->p.f_scale, c->stream));
+  if (from_coarse)
+    TRY(launch_level_start64(c->p.dim, c->geo[k - 2], c->u[k - 2], g, u, c->g[k - 1], c->b[k - 1], c->p.f,
+                             c->p.f_scale, c->stream));
+  else
+    TRY(launch_nonlinear_rhs(c->p.dim, g, u, c->g[k - 1], c->b[k - 1], c->p.f, c->p.f_scale, c->stream));
   for (int i = 0; i < c->p.m_vcycles; ++i) TRY(top_cycle(c, k, u, c->b[k - 1]));
   // step 2: semilinear problem on V_H + span{u~}  (eq. 3.6)
   TRY(tbegin(c, FMG_KT_AUGMENTED, k, &slot_aug));
@@ -548,16 +582,13 @@ cudaError_t run_fmg(fmg_ctx* c) {
   TRY(launch_level1_newton(c->p.dim, c->geo[0], c->g[0], c->u[0], c->p.f, c->p.f_scale, c->p.level1_tol,
                            c->p.level1_maxit, mixed, c->st, c->stream, mixed && c->nlev > 1, vcp(c)));
   for (int k = 2; k <= c->nlev; ++k) {
-    // u^{(0)}_{h_k} = u_{h_{k-1}}: the natural inclusion (the mixed path forms it in the pass
-    // that starts its first correction step)
-    if (!mixed)
-      TRY(launch_prolong<double, double>(c->p.dim, c->geo[k - 2], c->u[k - 2], c->geo[k - 1], c->u[k - 1], 0,
-                                         c->stream));
+    // u^{(0)}_{h_k} = u_{h_{k-1}}: the natural inclusion, formed in the pass that starts the level's
+    // first correction step
     for (int l = 0; l < c->p.p_corrections; ++l) {
       if (mixed)
         TRY(correction_step_ff(c, k, k == c->nlev && l == c->p.p_corrections - 1, l == 0));
       else
-        TRY(correction_step(c, k, c->u[k - 1]));
+        TRY(correction_step(c, k, c->u[k - 1], l == 0));
     }
   }
   return cudaSuccess;
@@ -672,6 +703,7 @@ const std::vector<PhaseKernel>& phase_registry() {
     phase_kernels_ff(r);
     phase_kernels_fused(r);
     phase_kernels_coarse(r);
+    phase_kernels_rb64(r);
     phase_kernels_newton(r);
     return r;
   }();

@@ -72,25 +72,6 @@ struct CLevel {
   unsigned magic;       // 2^20 / (n / 2), rounded up
 };
 
-// x / 4 without the FP64 multiplier (it issues at 1/64 of the FP32 rate): the exponent lowered
-// by two where that is exact, the product otherwise.
-__device__ __forceinline__ double quarter(double x) {
-  const int hi = __double2hiint(x);
-  const int e = hi & 0x7ff00000;
-  if (e > 0x00200000 && e != 0x7ff00000) return __hiloint2double(hi - 0x00200000, __double2loint(x));
-  return x * 0.25;
-}
-__device__ __forceinline__ float quarter(float x) { return x * 0.25f; }
-
-// x 2^k (|k| < 64), the FP64 form the same way.
-__device__ __forceinline__ double times_pow2(double x, int k) {
-  const int hi = __double2hiint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  if (e > 64 && e < 0x7ff - 64) return __hiloint2double(hi + (k << 20), __double2loint(x));
-  return scalbn(x, k);
-}
-__device__ __forceinline__ float times_pow2(float x, int k) { return x * __int_as_float((127 + k) << 23); }
-
 template <typename T, int D, bool CHEB, bool VC>
 __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
   cg::cluster_group cluster = cg::this_cluster();

@@ -104,6 +104,25 @@ struct DevState {
   double pad[3];
 };
 
+// x / 4 without the FP64 multiplier (it issues at 1/64 of the FP32 rate): the exponent lowered
+// by two where that is exact, the product otherwise.
+__device__ __forceinline__ double quarter(double x) {
+  const int hi = __double2hiint(x);
+  const int e = hi & 0x7ff00000;
+  if (e > 0x00200000 && e != 0x7ff00000) return __hiloint2double(hi - 0x00200000, __double2loint(x));
+  return x * 0.25;
+}
+__device__ __forceinline__ float quarter(float x) { return x * 0.25f; }
+
+// x 2^k (|k| < 64), the FP64 form the same way.
+__device__ __forceinline__ double times_pow2(double x, int k) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  if (e > 64 && e < 0x7ff - 64) return __hiloint2double(hi + (k << 20), __double2loint(x));
+  return scalbn(x, k);
+}
+__device__ __forceinline__ float times_pow2(float x, int k) { return x * __int_as_float((127 + k) << 23); }
+
 struct LevelGeo {
   int n;          // cells per side
   int np;         // n + 1
@@ -419,6 +438,24 @@ cudaError_t launch_pre_fused(int dim, LevelGeo g, int nu, const float* b, float*
 // u = u_in + P e_c, nu black-red sweeps; stored in u_out, or added to u64_top when non-NULL
 cudaError_t launch_post_fused(int dim, LevelGeo g, int nu, const float* u_in, const float* ec, const float* b,
                               float* u_out, double* u64_top, cudaStream_t s, bool u_ff = false);
+
+// FP64 red-black cycle kernels with A = I (fmg_rb64.cu).
+// b_c = P^T (b - A u) after a red-black sweep (the black residuals taken as zero); start: u_c gets the
+// coarse level's first red half sweep from zero, else it is not written
+cudaError_t launch_restrict_rb64(int dim, LevelGeo gf, const double* u_f, const double* b_f, LevelGeo gc, double* b_c,
+                                 double* u_c, bool start, cudaStream_t s);
+// u_f += P e_c on the red nodes (before a black-red sweep)
+cudaError_t launch_prolong_rb64(int dim, LevelGeo gc, const double* e_c, LevelGeo gf, double* u_f, cudaStream_t s);
+// the start of level g: u = P u_c and b = w (g - a f(u))
+cudaError_t launch_level_start64(int dim, LevelGeo gc, const double* uc, LevelGeo g, double* u, const double* gn,
+                                 double* b, int kind, double a, cudaStream_t s);
+// 2D tile kernels: nu sweeps from u_in (NULL: zero) into u_out and the restriction; nu sweeps from
+// u_in + P e_c into u_out.  u_in and u_out differ.
+bool fused_rb64_supported(int dim, int n, int nu_pre, int nu_post);
+cudaError_t launch_pre_rb64(LevelGeo g, int nu, const double* u_in, const double* b, double* u_out, double* bc,
+                            cudaStream_t s);
+cudaError_t launch_post_rb64(LevelGeo g, int nu, const double* u_in, const double* ec, const double* b, double* u_out,
+                             cudaStream_t s);
 
 // Sets the calling thread's error message (what fmg_last_error(NULL) returns).
 // Context services for the request server (fmg_capi.cu).

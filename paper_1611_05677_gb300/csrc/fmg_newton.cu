@@ -362,133 +362,6 @@ __global__ void k_coarse_inverse(int dim, int n1, double* __restrict__ Ainv, Dev
   }
 }
 
-// Algorithm 3.2 step 1: Newton on A_1 U + w f(U) = w g, from U = 0 (one CTA).  The residual,
-// the iterate and the convergence test are FP64; the Jacobian A_1 + diag(w f'(U)) is factored
-// in precision T (T = float in the mixed path: an inexact Newton step whose error the next
-// FP64 residual corrects, so the iteration converges to the same FP64 solution).
-template <typename T>
-__device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
-                                double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) {
-  extern __shared__ double sm[];
-  const int m = n1 - 1;
-  const int N = dim == 2 ? m * m : m * m * m;
-  const int ld = N + 1;
-  double* U = sm;
-  double* rhs = U + N;
-  double* Fp = rhs + N;
-  T* L = reinterpret_cast<T*>(Fp + N);
-  T* work = L + (size_t)N * ld;
-  T* invd = work + N;
-  __shared__ int done, ok_sh;
-  const double h = 1.0 / n1;
-  const double sigma = dim == 2 ? 1.0 : h;
-  const double w = dim == 2 ? h * h : h * h * h;
-  const int band = dim == 2 ? m : m * m;   // lexicographic half-bandwidth of the 2d+1-point stencil
-  for (int i = threadIdx.x; i < N; i += blockDim.x) U[i] = 0.0;
-  // entries outside the band are zero and the factorization never writes them
-  for (int i = threadIdx.x; i < N * ld; i += blockDim.x) L[i] = T(0);
-  if (threadIdx.x == 0) done = 0;
-  __syncthreads();
-  int it = 0;
-  for (it = 1; it <= maxit; ++it) {
-    for (int p = threadIdx.x; p < N; p += blockDim.x) {
-      double F, D;
-      f_eval<double>(kind, a, U[p], F, D);
-      // (A U)_p from the stencil: sigma (2d U_p - sum of interior axis neighbours), or with
-      // the coefficient sigma sum_e w_e (U_p - U_e) (boundary neighbours are zero)
-      double au;
-      if (vc.a64) {
-        double wt[6];
-        level1_weights(vc, p, m, dim, wt);
-        double acc = 0.0;
-        int rem = p, mul = 1;
-        for (int ax = 0; ax < dim; ++ax) {
-          const int c = rem % m;
-          rem /= m;
-          acc += wt[2 * ax] * (U[p] - (c > 0 ? U[p - mul] : 0.0));
-          acc += wt[2 * ax + 1] * (U[p] - (c < m - 1 ? U[p + mul] : 0.0));
-          mul *= m;
-        }
-        au = sigma * acc;
-      } else {
-        double nb = 0.0;
-        int rem = p, mul = 1;
-        for (int ax = 0; ax < dim; ++ax) {
-          const int c = rem % m;
-          rem /= m;
-          if (c > 0) nb += U[p - mul];
-          if (c < m - 1) nb += U[p + mul];
-          mul *= m;
-        }
-        au = sigma * (2.0 * dim * U[p] - nb);
-      }
-      rhs[p] = -(au + w * F - w * g[node_of(p, m, dim)]);
-      Fp[p] = w * D;
-    }
-    __syncthreads();
-    // the lower band of the Jacobian A_1 + diag(w f'(U)) (the factor of the previous
-    // iteration overwrote it)
-    for (int idx = threadIdx.x; idx < N * (band + 1); idx += blockDim.x) {
-      const int p = idx / (band + 1), q = p - idx % (band + 1);
-      if (q < 0) continue;
-      const double v = level1_entry(p, q, m, dim, sigma, vc) + (p == q ? Fp[p] : 0.0);
-      L[p * ld + q] = (T)v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      // the benchmark shapes (2D 1/H = 8, 3D 1/H = 4) with their size and band fixed at compile time
-      const bool okw = (dim == 2 && N == 49 && band == 7)
-                           ? ldlt_band_warp_ns<T, 1, 49, 7>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
-                       : (dim == 3 && N == 27 && band == 9)
-                           ? ldlt_band_warp_ns<T, 2, 27, 9>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
-                           : ldlt_band_warp<T>(L, N, ld, invd, band, 0, false, 0.0, nullptr);
-      ldlt_solve_band_warp<T>(L, N, ld, invd, band, 0, rhs);
-      if (threadIdx.x == 0) ok_sh = okw ? 1 : 0;
-    }
-    __syncthreads();
-    const bool ok = ok_sh != 0;
-    if (threadIdx.x < 32) {
-      double dmax = 0.0, umax = 0.0;
-      bool finite = true;
-      for (int p = threadIdx.x; p < N; p += 32) {
-        const double v = U[p] + rhs[p];
-        if (!isfinite(v)) finite = false;
-        dmax = fmax(dmax, fabs(rhs[p]));
-        umax = fmax(umax, fabs(v));
-        U[p] = v;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-        umax = fmax(umax, __shfl_xor_sync(0xffffffffu, umax, o));
-      }
-      finite = __all_sync(0xffffffffu, finite);
-      if (threadIdx.x == 0) {
-        if (!ok) atomicOr(&st->flags, kFlagNotSPD);
-        if (!finite) atomicOr(&st->flags, kFlagNonfinite);
-        if (!ok || !finite) done = 2;
-        else if (dmax <= tol * fmax(1.0, umax)) done = 1;
-      }
-    }
-    __syncthreads();
-    if (done) break;
-  }
-  if (threadIdx.x == 0) {
-    if (done != 1) atomicOr(&st->flags, kFlagNewtonCap);
-    st->level1_iters = it > maxit ? maxit : it;
-  }
-  for (int p = threadIdx.x; p < N; p += blockDim.x) {
-    if (out_ff)
-      ff_store(u + node_of(p, m, dim), ff_from_double(U[p]));
-    else
-      u[node_of(p, m, dim)] = U[p];
-  }
-}
-
-template <typename T>
-__global__ void k_level1_newton(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
-                                double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) { pdl_start(); k_level1_newton_body<T>(dim, n1, g, u, kind, a, tol, maxit, st, out_ff, vc); }
-
 // ------------------------------------------------------------------ augmented problem
 template <int D, bool JF32>
 struct Aug {
@@ -2172,6 +2045,13 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
   newton_update_mixed<D>(A, dl, NH, S, dropped, ok, writer, red_sh);
 }
 
+// Maximum over a warp's lanes.
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long b) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+
 // (c, alpha) += the step in R (FP64) and the convergence test
 // ||step||_inf <= tol max(1, ||(c, alpha)||_inf), a thread per unknown.  The maxima are taken over
 // the magnitudes' bit patterns, which order as the numbers do (and put non-finite ones on top).
@@ -2194,13 +2074,8 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
       db = (unsigned long long)__double_as_longlong(R[tid]) & 0x7fffffffffffffffull;
       yb = (unsigned long long)__double_as_longlong(nv) & 0x7fffffffffffffffull;
     }
-    auto warp_max = [](unsigned long long b) {
-      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32));
-      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0u);
-      return ((unsigned long long)hi << 32) | lo;
-    };
-    db = warp_max(db);
-    yb = warp_max(yb);
+    db = warp_max_bits(db);
+    yb = warp_max_bits(yb);
     if ((tid & 31) == 0) {
       max_sh[tid >> 5][0] = db;
       max_sh[tid >> 5][1] = yb;
@@ -2244,22 +2119,22 @@ constexpr float kRefinePivot = 1e-3f;
 // Refinement sweeps from y = 0 (see above); R, M in shared memory, y written over R on success;
 // iterate: max(1, ||(c, alpha)||_inf).
 // Returns false (R untouched) if they do not converge.
-template <int D>
-__device__ bool refine_solve(const AugArgs& A, const float* X, const double* M, int NH, double* R, float iterate) {
+template <int D, int NT>
+__device__ bool refine_solve(int nc, double newton_tol, const float* X, const double* M, int NH, double* R,
+                             float iterate) {
   constexpr int LPR = D == 2 ? 2 : 4;    // lanes per row of the sparse residual
   constexpr int NE = 4;                  // its entries per lane: 2D 7 + border, 3D 15 + border
-  constexpr int NT = Aug<D, false>::NT;
   __shared__ double y_sh[kMaxAug];
   __shared__ float r_sh[kMaxAug], z_sh[kMaxAug];
   __shared__ unsigned max_sh[2][2];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int NA = NH + 1, ld = NA + 1, m = A.nc - 1;
+  const int NA = NH + 1, ld = NA + 1, m = nc - 1;
   // this lane's entries of row p of J: the mesh-edge neighbours and the alpha column
   const int p = tid / LPR, sub = tid % LPR;
   int idx[NE];
   {
     int z[3] = {0, 0, 0};
-    if (p < NH) unknown_coords<D>(p, A.nc, z);
+    if (p < NH) unknown_coords<D>(p, nc, z);
 #pragma unroll
     for (int k = 0; k < NE; ++k) {
       const int e = sub * NE + k;   // 0: diagonal, 2t - 1 / 2t: + / - the t-th edge vector, last: alpha
@@ -2313,7 +2188,7 @@ __device__ bool refine_solve(const AugArgs& A, const float* X, const double* M, 
     if (sweep > 0) {
       // the next correction is about zmax (zmax / zprev)
       const float rho = zmax / zprev;
-      const float tol = (float)A.tol * iterate;
+      const float tol = (float)newton_tol * iterate;
       const float goal = ymax > tol ? fminf(1e-3f * ymax * ymax, 1e-2f * tol) : 0.f;
       if (zmax * fminf(rho, 1.f) <= fmaxf(goal, 5e-17f * iterate)) break;
       if (rho > 0.5f && zmax <= 1e-13f * ymax) break;   // at the rounding level of an FP64 solve
@@ -2491,7 +2366,7 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
     __syncthreads();
   }
   if (!S.flags[2]) {
-    const bool solved = refine_solve<D>(A, X, M, NH, R, iterate_sh);
+    const bool solved = refine_solve<D, nthr>(A.nc, A.tol, X, M, NH, R, iterate_sh);
     __syncthreads();
     if (!solved && tid == 0) S.flags[2] = 1;
     __syncthreads();
@@ -2549,6 +2424,246 @@ __device__ void step_report(const AugArgs& A, const StepState& S, int it, bool w
     A.st->alpha[A.level_index] = S.sa[1];
   }
 }
+
+// Algorithm 3.2 step 1: Newton on A_1 U + w f(U) = w g, from U = 0 (one CTA).  The residual,
+// the iterate and the convergence test are FP64.  Mixed path: the Jacobian A_1 + diag(w f'(U)) is
+// factored in FP32 (an inexact Newton step whose error the next FP64 residual corrects, so the
+// iteration converges to the same FP64 solution).  FP64 path: each step is solved to FP64 accuracy
+// by refinement on an FP32 inverse of its own Jacobian, as the augmented step's (the system is
+// bordered by an idle unknown, so that it has the augmented system's shape; the FP64 factor and
+// substitutions of 49 unknowns took 40 us per iteration on one warp, this takes LEVEL1).
+template <typename T>
+__device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
+                                double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) {
+  extern __shared__ double sm[];
+  const int m = n1 - 1;
+  const int N = dim == 2 ? m * m : m * m * m;
+  const int ld = N + 1;
+  double* U = sm;
+  double* rhs = U + N;
+  double* Fp = rhs + N + 1;   // (rhs: the FP64 path borders the system)
+  T* L = reinterpret_cast<T*>(Fp + N);
+  T* work = L + (size_t)N * ld;
+  T* invd = work + N;
+  // FP64 path, bordered: the Jacobian M, the FP64 factor's place F (X, then the FP32 factor and its
+  // reciprocal pivots, until it is needed), an FP32 copy of A_1 and A_1's diagonal
+  constexpr bool kRefine = sizeof(T) == 8;
+  const int NA = N + 1, lda = NA + 1;
+  double* M = Fp + N;
+  double* F = M + (size_t)NA * lda;
+  double* dg = F + (size_t)NA * lda + NA;
+  float* A32 = reinterpret_cast<float*>(dg + N);
+  __shared__ int use64;
+  __shared__ float iterate_sh;
+  __shared__ unsigned long long max_sh[2][2];
+  const int tid = threadIdx.x, lane = tid & 31;
+  __shared__ int done, ok_sh;
+  const double h = 1.0 / n1;
+  const double sigma = dim == 2 ? 1.0 : h;
+  const double w = dim == 2 ? h * h : h * h * h;
+  const int band = dim == 2 ? m : m * m;   // lexicographic half-bandwidth of the 2d+1-point stencil
+  for (int i = threadIdx.x; i < N; i += blockDim.x) U[i] = 0.0;
+  // entries outside the band are zero and the factorization never writes them
+  if constexpr (kRefine) {
+    for (int i = tid; i < NA * lda; i += blockDim.x) {
+      const int p = i / lda, q = i - p * lda;
+      const double v = p < N && q < N ? level1_entry(p, q, m, dim, sigma, vc) : p == N && q == N ? 1.0 : 0.0;
+      M[i] = v;
+      A32[i] = (float)v;
+      if (p == q && p < N) dg[p] = v;
+    }
+    if (tid == 0) use64 = 0;
+  } else {
+    for (int i = tid; i < N * ld; i += blockDim.x) L[i] = T(0);
+  }
+  if (tid == 0) done = 0;
+  __syncthreads();
+  int it = 0;
+  for (it = 1; it <= maxit; ++it) {
+    for (int p = threadIdx.x; p < N; p += blockDim.x) {
+      double F, D;
+      f_eval<double>(kind, a, U[p], F, D);
+      // (A U)_p from the stencil: sigma (2d U_p - sum of interior axis neighbours), or with
+      // the coefficient sigma sum_e w_e (U_p - U_e) (boundary neighbours are zero)
+      double au;
+      if (vc.a64) {
+        double wt[6];
+        level1_weights(vc, p, m, dim, wt);
+        double acc = 0.0;
+        int rem = p, mul = 1;
+        for (int ax = 0; ax < dim; ++ax) {
+          const int c = rem % m;
+          rem /= m;
+          acc += wt[2 * ax] * (U[p] - (c > 0 ? U[p - mul] : 0.0));
+          acc += wt[2 * ax + 1] * (U[p] - (c < m - 1 ? U[p + mul] : 0.0));
+          mul *= m;
+        }
+        au = sigma * acc;
+      } else {
+        double nb = 0.0;
+        int rem = p, mul = 1;
+        for (int ax = 0; ax < dim; ++ax) {
+          const int c = rem % m;
+          rem /= m;
+          if (c > 0) nb += U[p - mul];
+          if (c < m - 1) nb += U[p + mul];
+          mul *= m;
+        }
+        au = sigma * (2.0 * dim * U[p] - nb);
+      }
+      rhs[p] = -(au + w * F - w * g[node_of(p, m, dim)]);
+      Fp[p] = w * D;
+    }
+    __syncthreads();
+    if constexpr (kRefine) {
+      float* X = reinterpret_cast<float*>(F);
+      float* Lf = X + (size_t)NA * lda;
+      float* rd = Lf + (size_t)NA * lda;
+      if (!use64) {
+        for (int i = tid; i < NA * lda; i += blockDim.x) Lf[i] = A32[i];
+        __syncthreads();
+      }
+      if (tid < N) {
+        const double v = dg[tid] + Fp[tid];
+        M[tid * lda + tid] = v;
+        if (!use64) Lf[tid * lda + tid] = (float)v;
+      }
+      if (tid == N) rhs[N] = 0.0;
+      if (tid >= 64 && tid < 96) {   // max(1, ||U||_inf), for the solve's goal
+        float v = 1.f;
+        for (int p = lane; p < N; p += 32) v = fmaxf(v, fabsf((float)U[p]));
+        v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+        if (lane == 0) iterate_sh = v;
+      }
+      __syncthreads();
+      if (!use64) {
+        if (tid < 32) {
+          const bool okw = (dim == 2 && NA == 50)   ? ldlt_band_warp_ns<float, 2, 50, 8>(Lf, NA, lda, rd, 8, 1, false, 0.0, nullptr)
+                           : (dim == 2 && NA == 10) ? ldlt_band_warp_ns<float, 1, 10, 4>(Lf, NA, lda, rd, 4, 1, false, 0.0, nullptr)
+                           : (dim == 3 && NA == 28) ? ldlt_band_warp_ns<float, 4, 28, 13>(Lf, NA, lda, rd, 13, 1, false, 0.0, nullptr)
+                                                    : ldlt_band_warp<float>(Lf, NA, lda, rd, band, 1, false, 0.0, nullptr);
+          if (tid == 0 && !okw) use64 = 1;
+        }
+        __syncthreads();
+        if (!use64 && tid < NA) {
+          if (dim == 2)
+            band_inverse_dispatch<2>(Lf, rd, NA, lda, NA == 50 ? 8 : NA == 10 ? 4 : band, tid, X);
+          else
+            band_inverse_dispatch<3>(Lf, rd, NA, lda, NA == 28 ? 13 : band, tid, X);
+        }
+        __syncthreads();
+      }
+      if (!use64) {
+        const bool solved = dim == 2 ? refine_solve<2, 256>(n1, tol, X, M, N, rhs, iterate_sh)
+                                     : refine_solve<3, 256>(n1, tol, X, M, N, rhs, iterate_sh);
+        __syncthreads();
+        if (!solved && tid == 0) use64 = 1;
+        __syncthreads();
+      }
+      if (use64) {
+        for (int i = tid; i < NA * lda; i += blockDim.x) F[i] = M[i];
+        __syncthreads();
+        if (tid < 32) {
+          const bool okw = ldlt_band_warp<double>(F, NA, lda, F + (size_t)NA * lda, band, 1, false, 0.0, nullptr);
+          ldlt_solve_band_warp<double>(F, NA, lda, F + (size_t)NA * lda, band, 1, rhs);
+          if (tid == 0) ok_sh = okw ? 1 : 0;
+        }
+        __syncthreads();
+      } else if (tid == 0) {
+        ok_sh = 1;
+      }
+      if (tid < 64) {
+        unsigned long long db = 0, ub = 0;
+        if (tid < N) {
+          const double v = U[tid] + rhs[tid];
+          U[tid] = v;
+          db = (unsigned long long)__double_as_longlong(rhs[tid]) & 0x7fffffffffffffffull;
+          ub = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+        }
+        db = warp_max_bits(db);
+        ub = warp_max_bits(ub);
+        if (lane == 0) {
+          max_sh[tid >> 5][0] = db;
+          max_sh[tid >> 5][1] = ub;
+        }
+      }
+      __syncthreads();
+      if (tid == 0) {
+        const unsigned long long db = max(max_sh[0][0], max_sh[1][0]), ub = max(max_sh[0][1], max_sh[1][1]);
+        const bool finite = (db >> 52) != 0x7ff && (ub >> 52) != 0x7ff;
+        if (!ok_sh) atomicOr(&st->flags, kFlagNotSPD);
+        if (!finite) atomicOr(&st->flags, kFlagNonfinite);
+        if (!ok_sh || !finite)
+          done = 2;
+        else if (__longlong_as_double((long long)db) <= tol * fmax(1.0, __longlong_as_double((long long)ub)))
+          done = 1;
+      }
+      __syncthreads();
+      if (done) break;
+      continue;
+    }
+    // the lower band of the Jacobian A_1 + diag(w f'(U)) (the factor of the previous
+    // iteration overwrote it)
+    for (int idx = threadIdx.x; idx < N * (band + 1); idx += blockDim.x) {
+      const int p = idx / (band + 1), q = p - idx % (band + 1);
+      if (q < 0) continue;
+      const double v = level1_entry(p, q, m, dim, sigma, vc) + (p == q ? Fp[p] : 0.0);
+      L[p * ld + q] = (T)v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      // the benchmark shapes (2D 1/H = 8, 3D 1/H = 4) with their size and band fixed at compile time
+      const bool okw = (dim == 2 && N == 49 && band == 7)
+                           ? ldlt_band_warp_ns<T, 1, 49, 7>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
+                       : (dim == 3 && N == 27 && band == 9)
+                           ? ldlt_band_warp_ns<T, 2, 27, 9>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
+                           : ldlt_band_warp<T>(L, N, ld, invd, band, 0, false, 0.0, nullptr);
+      ldlt_solve_band_warp<T>(L, N, ld, invd, band, 0, rhs);
+      if (threadIdx.x == 0) ok_sh = okw ? 1 : 0;
+    }
+    __syncthreads();
+    const bool ok = ok_sh != 0;
+    if (threadIdx.x < 32) {
+      double dmax = 0.0, umax = 0.0;
+      bool finite = true;
+      for (int p = threadIdx.x; p < N; p += 32) {
+        const double v = U[p] + rhs[p];
+        if (!isfinite(v)) finite = false;
+        dmax = fmax(dmax, fabs(rhs[p]));
+        umax = fmax(umax, fabs(v));
+        U[p] = v;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+        umax = fmax(umax, __shfl_xor_sync(0xffffffffu, umax, o));
+      }
+      finite = __all_sync(0xffffffffu, finite);
+      if (threadIdx.x == 0) {
+        if (!ok) atomicOr(&st->flags, kFlagNotSPD);
+        if (!finite) atomicOr(&st->flags, kFlagNonfinite);
+        if (!ok || !finite) done = 2;
+        else if (dmax <= tol * fmax(1.0, umax)) done = 1;
+      }
+    }
+    __syncthreads();
+    if (done) break;
+  }
+  if (threadIdx.x == 0) {
+    if (done != 1) atomicOr(&st->flags, kFlagNewtonCap);
+    st->level1_iters = it > maxit ? maxit : it;
+  }
+  for (int p = threadIdx.x; p < N; p += blockDim.x) {
+    if (out_ff)
+      ff_store(u + node_of(p, m, dim), ff_from_double(U[p]));
+    else
+      u[node_of(p, m, dim)] = U[p];
+  }
+}
+
+template <typename T>
+__global__ void k_level1_newton(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
+                                double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) { pdl_start(); k_level1_newton_body<T>(dim, n1, g, u, kind, a, tol, maxit, st, out_ff, vc); }
 
 // VC: the first pass forms A_k u~ with the coefficient's edge weights (a variant of its own, so
 // that the constant-coefficient kernels keep their register allocation).
@@ -2832,7 +2947,8 @@ cudaError_t launch_level1_newton(int dim, LevelGeo g1, const double* gn, double*
     if ((e = raise_dyn_smem((const void*)k_level1_newton<float>, smem)) != cudaSuccess) return e;
     launch_k(k_level1_newton<float>, 1, 256, smem, s, dim, g1.n, gn, u, kind, a, tol, maxit, st, out_ff ? 1 : 0, v);
   } else {
-    const size_t smem = sizeof(double) * (3 * N + 2 + N * (N + 1) + 2 * N + 4);
+    const size_t na = N + 1, sq = na * (na + 1);
+    const size_t smem = sizeof(double) * (3 * N + 2 + 2 * sq + na + N) + sizeof(float) * sq;
     if ((e = raise_dyn_smem((const void*)k_level1_newton<double>, smem)) != cudaSuccess) return e;
     launch_k(k_level1_newton<double>, 1, 256, smem, s, dim, g1.n, gn, u, kind, a, tol, maxit, st, out_ff ? 1 : 0, v);
   }

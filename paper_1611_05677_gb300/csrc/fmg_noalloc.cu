@@ -24,12 +24,13 @@ int g_ainv_key[kMaxDevices] = {};                  // (dim, coarse_cells) whose 
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Layout inside the scratch: DevState | A_1^{-1} | u_1, b_1 | ... | u_{k-1}, b_{k-1}.
+// Layout inside the scratch: DevState | A_1^{-1} | u_1, b_1 | ... | u_{k-1}, b_{k-1}, then, as far as
+// they fit, the tile kernels' second iterates of levels 2..k (tmp_off 0: none).
 struct Layout {
-  size_t state, ainv, levels, level_off[kMaxLevels], end;
+  size_t state, ainv, levels, level_off[kMaxLevels], end, tmp_off[kMaxLevels];
 };
 
-Layout make_layout(int dim, int coarse_cells, int level) {
+Layout make_layout(int dim, int coarse_cells, int level, int nu_pre, int nu_post) {
   Layout L{};
   size_t off = 0;
   L.state = off;
@@ -45,6 +46,14 @@ Layout make_layout(int dim, int coarse_cells, int level) {
     off += align256(2 * (size_t)nodes * sizeof(double));
   }
   L.end = off;
+  for (int j = 2; j <= level; ++j) {
+    const int n = coarse_cells << (j - 1);
+    if (n <= coarse_cycle_cells(dim) || !fused_rb64_supported(dim, n, nu_pre, nu_post)) continue;
+    const size_t bytes = align256((size_t)ipow(n + 1, dim) * sizeof(double));
+    if (off + bytes > kNoAllocBytes) continue;
+    L.tmp_off[j - 1] = off;
+    off += bytes;
+  }
   return L;
 }
 
@@ -63,6 +72,7 @@ struct Ctx {
   }
   double* u(int j) const { return reinterpret_cast<double*>(base + lay.level_off[j - 1]); }
   double* b(int j) const { return u(j) + geo(j).nodes; }
+  double* tmp(int j) const { return lay.tmp_off[j - 1] ? reinterpret_cast<double*>(base + lay.tmp_off[j - 1]) : nullptr; }
 };
 
 // Largest level the cluster coarse cycle takes (same rule as the context's schedule).
@@ -72,22 +82,37 @@ int coarse_top(const Ctx& c, int level) {
   return j;
 }
 
-cudaError_t vcycle(const Ctx& c, int j, int level, double* u, const double* b) {
+// The cycle of fmg_op_vcycle's FP64 red-black path.  started: the red half of the level's first sweep
+// was taken by the restriction.
+cudaError_t vcycle(const Ctx& c, int j, int level, double* u, const double* b, bool started = false) {
   cudaError_t e;
   if (j == 1) return launch_coarse_solve_f64(c.dim, c.geo(1), c.ainv, b, u, c.s);
   if (j <= coarse_top(c, level))
-    return launch_coarse_cycle<double>(c.dim, c.nc, j, u, b, c.nu_pre, c.nu_post, c.ainv, nullptr, nullptr, false,
-                                       c.s);
+    return launch_coarse_cycle<double>(c.dim, c.nc, j, u, b, c.nu_pre, c.nu_post, c.ainv, nullptr, nullptr,
+                                       j < level, c.s);
   const LevelGeo gf = c.geo(j), gc = c.geo(j - 1);
+  if (double* t = c.tmp(j)) {
+    if ((e = launch_pre_rb64(gf, c.nu_pre, j == level ? u : nullptr, b, t, c.b(j - 1), c.s)) != cudaSuccess) return e;
+    if ((e = vcycle(c, j - 1, level, c.u(j - 1), c.b(j - 1))) != cudaSuccess) return e;
+    return launch_post_rb64(gf, c.nu_post, t, c.u(j - 1), b, u, c.s);
+  }
   for (int it = 0; it < c.nu_pre; ++it) {
-    if ((e = launch_rbgs<double>(c.dim, gf, u, b, 0, c.s)) != cudaSuccess) return e;
+    if ((it > 0 || !started) && (e = launch_rbgs<double>(c.dim, gf, u, b, 0, c.s)) != cudaSuccess) return e;
     if ((e = launch_rbgs<double>(c.dim, gf, u, b, 1, c.s)) != cudaSuccess) return e;
   }
-  if ((e = launch_residual_restrict<double, double>(c.dim, gf, u, b, gc, c.b(j - 1), c.u(j - 1), c.s)) !=
-      cudaSuccess)
-    return e;
-  if ((e = vcycle(c, j - 1, level, c.u(j - 1), c.b(j - 1))) != cudaSuccess) return e;
-  if ((e = launch_prolong<double, double>(c.dim, gc, c.u(j - 1), gf, u, 1, c.s)) != cudaSuccess) return e;
+  const bool own_start = j - 1 <= coarse_top(c, level) || c.tmp(j - 1);
+  const bool fuse = c.nu_pre >= 1 && !own_start;
+  if (c.nu_pre >= 1)
+    e = launch_restrict_rb64(c.dim, gf, u, b, gc, c.b(j - 1), c.u(j - 1), fuse, c.s);
+  else
+    e = launch_residual_restrict<double, double>(c.dim, gf, u, b, gc, c.b(j - 1), c.u(j - 1), c.s);
+  if (e != cudaSuccess) return e;
+  if ((e = vcycle(c, j - 1, level, c.u(j - 1), c.b(j - 1), fuse)) != cudaSuccess) return e;
+  if (c.nu_post >= 1)
+    e = launch_prolong_rb64(c.dim, gc, c.u(j - 1), gf, u, c.s);
+  else
+    e = launch_prolong<double, double>(c.dim, gc, c.u(j - 1), gf, u, 1, c.s);
+  if (e != cudaSuccess) return e;
   for (int it = 0; it < c.nu_post; ++it) {
     if ((e = launch_rbgs<double>(c.dim, gf, u, b, 1, c.s)) != cudaSuccess) return e;
     if ((e = launch_rbgs<double>(c.dim, gf, u, b, 0, c.s)) != cudaSuccess) return e;
@@ -113,7 +138,7 @@ extern "C" fmg_status fmg_vcycle_noalloc(int dim, int coarse_cells, int level, c
   if (level < 1 || level > kMaxLevels - 1) return fail(FMG_ERR_INVALID, "level out of range");
   if (!b || !u || cycles < 0 || nu_pre < 0 || nu_post < 0 || nu_pre > 64 || nu_post > 64)
     return fail(FMG_ERR_INVALID, "bad arguments");
-  const Layout lay = make_layout(dim, coarse_cells, level);
+  const Layout lay = make_layout(dim, coarse_cells, level, nu_pre, nu_post);
   if (lay.end > kNoAllocBytes)
     return fail(FMG_ERR_INVALID, "level " + std::to_string(level) + " needs " + std::to_string(lay.end) +
                                      " bytes of scratch; the no-allocation V-cycle holds at most " +

@@ -67,6 +67,7 @@ void phase_kernels_stencil(std::vector<PhaseKernel>& out);
 void phase_kernels_ff(std::vector<PhaseKernel>& out);
 void phase_kernels_fused(std::vector<PhaseKernel>& out);
 void phase_kernels_coarse(std::vector<PhaseKernel>& out);
+void phase_kernels_rb64(std::vector<PhaseKernel>& out);
 void phase_kernels_newton(std::vector<PhaseKernel>& out);
 
 }  // namespace fmg

@@ -40,14 +40,14 @@ __device__ __forceinline__ void k_rbgs2_body(T* __restrict__ u, const T* __restr
   const long long np = n + 1;
   const long long c = (long long)j * np + i;
   const T s = (u[c - 1] + u[c + 1]) + (u[c - np] + u[c + np]);
-  u[c] = (b[c] + s) * T(0.25);
+  u[c] = quarter(b[c] + s);
 }
 
 template <typename T>
 __global__ void k_rbgs2(T* __restrict__ u, const T* __restrict__ b, int n, int colour) { pdl_start(); k_rbgs2_body<T>(u, b, n, colour); }
 
 template <typename T>
-__global__ void k_rbgs3(T* __restrict__ u, const T* __restrict__ b, int n, int colour, T bscale, T inv6) {
+__global__ void k_rbgs3(T* __restrict__ u, const T* __restrict__ b, int n, int colour, int lg, T inv6) {
   pdl_start();
   const int j = blockIdx.y + 1;
   const int l = blockIdx.z + 1;
@@ -59,7 +59,7 @@ __global__ void k_rbgs3(T* __restrict__ u, const T* __restrict__ b, int n, int c
   const long long pl = np * np;
   const long long c = ((long long)l * np + j) * np + i;
   const T s = ((u[c - 1] + u[c + 1]) + (u[c - np] + u[c + np])) + (u[c - pl] + u[c + pl]);
-  u[c] = (b[c] * bscale + s) * inv6;
+  u[c] = (times_pow2(b[c], lg) + s) * inv6;   // n = 2^lg
 }
 
 // ------------------------------------------------------------------ Chebyshev-Jacobi step
@@ -589,7 +589,10 @@ cudaError_t launch_rbgs(int dim, LevelGeo g, T* u, const T* b, int colour, cudaS
   if (dim == 2) {
     launch_k(k_rbgs2<T>, dim3(gx, n - 1), kBlock, 0, s, u, b, n, colour);
   } else {
-    launch_k(k_rbgs3<T>, dim3(gx, n - 1, n - 1), kBlock, 0, s, u, b, n, colour, T(n), T(1.0 / 6.0));
+    int lg = 0;
+    while ((1 << lg) < n) ++lg;
+    if ((1 << lg) != n) return cudaErrorInvalidValue;   // (3D meshes are 2^k cells per side)
+    launch_k(k_rbgs3<T>, dim3(gx, n - 1, n - 1), kBlock, 0, s, u, b, n, colour, lg, T(1.0 / 6.0));
   }
   return cudaGetLastError();
 }
