@@ -626,10 +626,20 @@ fmg_status read_state(fmg_ctx* c, fmg_stats* st, bool accumulate_pending) {
 fmg_status load_rhs(fmg_ctx* c, const double* g_fine, int on_device) {
   if (!g_fine) return fail(c, FMG_ERR_INVALID, "g is NULL");
   const int top = c->nlev - 1;
-  CK(c, cudaMemcpyAsync(c->g[top], g_fine, c->geo[top].nodes * sizeof(double),
-                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+  const double* src = g_fine;
+  // device memory of this device is read in place by the launch below; anything else is copied first
+  cudaPointerAttributes at = {};
+  const bool direct = on_device && (reinterpret_cast<size_t>(g_fine) & 7) == 0 &&
+                      cudaPointerGetAttributes(&at, g_fine) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                      at.device == c->device;
+  if (!direct) {
+    cudaGetLastError();
+    CK(c, cudaMemcpyAsync(c->g[top], g_fine, c->geo[top].nodes * sizeof(double),
+                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    src = c->g[top];
+  }
   // the boundary ring, every coarser level by injection and the float-float copies: one launch
-  CK(c, launch_rhs_levels(c->p.dim, c->nlev, c->geo, c->g, c->gf, c->p.precision == FMG_PREC_MIXED, c->stream));
+  CK(c, launch_rhs_levels(c->p.dim, c->nlev, c->geo, src, c->g, c->gf, c->p.precision == FMG_PREC_MIXED, c->stream));
   return FMG_OK;
 }
 

@@ -313,7 +313,7 @@ __global__ void k_add_f32_ff(double* __restrict__ uff, const float* __restrict__
 __global__ void k_ff_from_f64(const double* __restrict__ s, double* __restrict__ d, long long n) {
   pdl_start();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) ff_store(d + i, ff_from_double(s[i]));
+  if (i < n) ff_store(d + i, ff_from_double_int(s[i]));
 }
 
 __global__ void k_ff_to_f64(const double* __restrict__ s, double* __restrict__ d, long long n) {
@@ -398,65 +398,80 @@ cudaError_t launch_add_f32_ff(LevelGeo g, double* u_ff, const float* e32, cudaSt
 
 namespace {
 
-// The right-hand side of every level from the fine g just copied in, in one launch: the fine
-// g's boundary ring set to zero in place; each coarser level's g the fine values at its nodes (the
-// nodal injection of the nested hierarchy: node (i, j[, l]) of level k is fine node
-// (i, j[, l]) n_L / n_k), zero on its boundary; and with ff the float-float copy of every level.
-// Blocks boff[k] .. boff[k+1]-1 take level k.  The fine level's blocks write only its boundary
-// ring and the coarser levels' blocks read only fine interior nodes, so they do not race.
+// The right-hand side of every level from the fine g at `src`, in one launch: every level's g is the
+// fine values at its nodes (the nodal injection of the nested hierarchy: node (i, j[, l]) of level k
+// is fine node (i, j[, l]) n_L / n_k), zero on its boundary, stored as FP64 where g[k] is given and
+// as float-float where gf[k] is.  src may be the fine level's own array (then only its boundary
+// ring is written).  Bound by HBM: the fine level reads 8 bytes and writes 8 per node and array.
+// Blocks boff[k] .. boff[k+1]-1 take level k, a block a row of nodes at a time (no index division
+// per node).  No block reads what another writes.
 struct RhsLevels {
+  const double* src;
   double* g[kMaxLevels];
   double* gf[kMaxLevels];
   int n[kMaxLevels];
-  long long nodes[kMaxLevels];
-  long long boff[kMaxLevels + 1];
-  int nlev, dim, ff;
+  unsigned boff[kMaxLevels + 1];
+  int nlev, dim, rows;   // rows per block
 };
 
-__global__ void k_rhs_levels(const __grid_constant__ RhsLevels R) {
+__global__ void __launch_bounds__(256) k_rhs_levels(const __grid_constant__ RhsLevels R) {
   pdl_start();
-  const long long bid = blockIdx.x;
   int k = 0;
-  while (k + 1 < R.nlev && bid >= R.boff[k + 1]) ++k;
-  const long long idx = (bid - R.boff[k]) * blockDim.x + threadIdx.x;
-  if (idx >= R.nodes[k]) return;
+  while (k + 1 < R.nlev && blockIdx.x >= R.boff[k + 1]) ++k;
   const int top = R.nlev - 1;
-  const int n = R.n[k];
-  const long long cp = n + 1;
-  const int i = (int)(idx % cp), j = (int)((idx / cp) % cp), l = R.dim == 3 ? (int)(idx / (cp * cp)) : 0;
-  const bool bnd = i == 0 || i == n || j == 0 || j == n || (R.dim == 3 && (l == 0 || l == n));
-  double v;
-  if (k == top) {
-    v = bnd ? 0.0 : R.g[top][idx];
-    if (bnd) R.g[top][idx] = 0.0;
-  } else {
-    const long long st = R.n[top] / n, fp = R.n[top] + 1;
-    v = bnd ? 0.0 : R.g[top][((l * st) * fp + j * st) * fp + i * st];
-    R.g[k][idx] = v;
+  const int n = R.n[k], np = n + 1, nt = R.n[top];
+  const int st = nt / n;
+  const long long fp = nt + 1;
+  const int nrows = R.dim == 2 ? np : np * np;
+  double* g = R.g[k];
+  double* gf = R.gf[k];
+  const bool self = g == R.src;
+  const int r0 = (int)(blockIdx.x - R.boff[k]) * R.rows;
+  for (int r = r0; r < min(r0 + R.rows, nrows); ++r) {
+    const int l = R.dim == 3 ? r / np : 0, j = r - l * np;
+    const bool edge = j == 0 || j == n || (R.dim == 3 && (l == 0 || l == n));
+    const double* in = R.src + ((long long)l * st * fp + (long long)j * st) * fp;
+    const long long o = (long long)r * np;
+    for (int i0 = threadIdx.x; i0 < np; i0 += 4 * 256) {
+      double v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = i0 + q * 256;
+        v[q] = i > 0 && i < n && !edge ? in[(long long)i * st] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = i0 + q * 256;
+        if (i >= np) break;
+        if (g && (!self || edge || i == 0 || i == n)) g[o + i] = v[q];
+        if (gf) ff_store(gf + o + i, ff_from_double_int(v[q]));
+      }
+    }
   }
-  if (R.ff) ff_store(R.gf[k] + idx, ff_from_double(v));
 }
 
 }  // namespace
 
-cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, double* const* g, double* const* gf, bool ff,
-                              cudaStream_t s) {
+cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, const double* src, double* const* g,
+                              double* const* gf, bool ff, cudaStream_t s) {
   if (nlev < 1 || nlev > kMaxLevels) return cudaErrorInvalidValue;
   RhsLevels R = {};
+  R.src = src;
+  R.rows = dim == 2 ? 1 : 4;
   long long off = 0;
   for (int k = 0; k < nlev; ++k) {
-    R.g[k] = g[k];
+    // with float-float copies only level 1 (the exact semilinear solve) reads the FP64 ones, and the
+    // fine one may be the source
+    R.g[k] = !ff || k == 0 || g[k] == src ? g[k] : nullptr;
     R.gf[k] = ff ? gf[k] : nullptr;
     R.n[k] = geo[k].n;
-    R.nodes[k] = geo[k].nodes;
-    R.boff[k] = off;
-    off += (geo[k].nodes + 255) / 256;
+    R.boff[k] = (unsigned)off;
+    off += (ipow(geo[k].np, dim - 1) + R.rows - 1) / R.rows;
   }
-  R.boff[nlev] = off;
+  if (off < 1 || off > 0x7fffffffll) return cudaErrorInvalidValue;
+  R.boff[nlev] = (unsigned)off;
   R.nlev = nlev;
   R.dim = dim;
-  R.ff = ff ? 1 : 0;
-  if (off < 1 || off > 0x7fffffffll) return cudaErrorInvalidValue;
   launch_k(k_rhs_levels, dim3((unsigned)off), 256, 0, s, R);
   return cudaGetLastError();
 }

@@ -113,6 +113,40 @@ __host__ __device__ __forceinline__ ff ff_from_double(double x) {
   r.lo = (float)(x - (double)r.hi);
   return r;
 }
+// The same pair with integer operations for the split (FP64 instructions, conversions included,
+// issue at 1/64 of the FP32 rate here; four of them per node bound the pass that converts g): hi
+// takes the leading 24 of the 53 significand bits, rounded to nearest even, and the signed rest,
+// below 2^28 units of the last place, is an integer whose FP32 conversion rounds the same way.
+// Magnitudes outside 2^-70 .. 2^126 (zero excepted) take the FP64 form.
+__host__ __device__ __forceinline__ ff ff_from_double_int(double x) {
+#ifdef __CUDA_ARCH__
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+#else
+  unsigned long long b;
+  memcpy(&b, &x, sizeof b);
+#endif
+  const unsigned neg = (unsigned)(b >> 63);
+  const int e = (int)((b >> 52) & 0x7ff);
+  if ((b << 1) != 0 && (unsigned)(e - (1023 - 70)) >= 196u) return ff_from_double(x);
+  const unsigned top = (unsigned)((b >> 29) & 0x7fffffu) | 0x800000u, rest = (unsigned)(b & 0x1fffffffu);
+  const unsigned up = (rest > 0x10000000u || (rest == 0x10000000u && (top & 1u))) ? 1u : 0u;
+  const int r = (int)rest - (int)(up << 29);
+  const bool zero = (b << 1) == 0;
+  // 2^(e - 1023 - 52) as FP32 bits; (top + up) - 2^23 carries into the exponent when it rounds over
+  const unsigned hb = zero ? neg << 31 : (neg << 31) | (((unsigned)(e - 1023 + 127) << 23) + (top + up - 0x800000u));
+  const unsigned sb = (unsigned)(e - 1023 - 52 + 127) << 23;
+  ff o;
+#ifdef __CUDA_ARCH__
+  o.hi = __uint_as_float(hb);
+  o.lo = zero ? 0.f : (float)(neg ? -r : r) * __uint_as_float(sb);
+#else
+  float sc;
+  memcpy(&o.hi, &hb, 4);
+  memcpy(&sc, &sb, 4);
+  o.lo = zero ? 0.f : (float)(neg ? -r : r) * sc;
+#endif
+  return o;
+}
 __host__ __device__ __forceinline__ double ff_to_double(ff x) { return (double)x.hi + (double)x.lo; }
 
 __host__ __device__ __forceinline__ unsigned ff_bits(float f) {

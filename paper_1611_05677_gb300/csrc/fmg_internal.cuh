@@ -104,24 +104,21 @@ struct DevState {
   double pad[3];
 };
 
-// x / 4 without the FP64 multiplier (it issues at 1/64 of the FP32 rate): the exponent lowered
-// by two where that is exact, the product otherwise.
-__device__ __forceinline__ double quarter(double x) {
-  const int hi = __double2hiint(x);
-  const int e = hi & 0x7ff00000;
-  if (e > 0x00200000 && e != 0x7ff00000) return __hiloint2double(hi - 0x00200000, __double2loint(x));
-  return x * 0.25;
-}
-__device__ __forceinline__ float quarter(float x) { return x * 0.25f; }
-
-// x 2^k (|k| < 64), the FP64 form the same way.
+// x 2^k (|k| < 64) without the FP64 multiplier (it issues at 1/64 of the FP32 rate): k added to the
+// exponent where that is exact.  Zeros, and values within 64 binades of the format's ends, take the
+// library's scaling in a call of its own: inlined, it is evaluated for every lane and selected
+// (the FP64 level start at 2049^2 then took 11 FP64 instructions per node, 96 us).
+static __device__ __noinline__ double scale_pow2_edge(double x, int k) { return scalbn(x, k); }
 __device__ __forceinline__ double times_pow2(double x, int k) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) & 0x7ff;
   if (e > 64 && e < 0x7ff - 64) return __hiloint2double(hi + (k << 20), __double2loint(x));
-  return scalbn(x, k);
+  if (((hi << 1) | __double2loint(x)) == 0) return x;
+  return scale_pow2_edge(x, k);
 }
 __device__ __forceinline__ float times_pow2(float x, int k) { return x * __int_as_float((127 + k) << 23); }
+__device__ __forceinline__ double quarter(double x) { return times_pow2(x, -2); }
+__device__ __forceinline__ float quarter(float x) { return x * 0.25f; }
 
 struct LevelGeo {
   int n;          // cells per side
@@ -423,9 +420,10 @@ cudaError_t launch_add_f32_ff(LevelGeo g, double* u_ff, const float* e32, cudaSt
 cudaError_t launch_level_start_ff(int dim, LevelGeo gc, const double* uc_ff, LevelGeo g, double* u_ff,
                                   const double* g_ff, double* b_ff, int kind, double a, float* r32, float* e32,
                                   float* d32, double e0, cudaStream_t s, const VarCoef* vc = nullptr);
-// every level's g (and its float-float copy gf, with ff) from the fine g, its boundary zeroed
-cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, double* const* g, double* const* gf, bool ff,
-                              cudaStream_t s);
+// every level's g from the fine g at src (a device array, or the fine level's own g), boundaries zero;
+// with ff the float-float copies gf, and FP64 ones on level 1 only
+cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, const double* src, double* const* g,
+                              double* const* gf, bool ff, cudaStream_t s);
 // conversions (in place allowed)
 cudaError_t launch_ff_from_f64(const double* src, double* dst_ff, long long n, cudaStream_t s);
 cudaError_t launch_ff_to_f64(const double* src_ff, double* dst, long long n, cudaStream_t s);
@@ -444,6 +442,8 @@ cudaError_t launch_post_fused(int dim, LevelGeo g, int nu, const float* u_in, co
 // coarse level's first red half sweep from zero, else it is not written
 cudaError_t launch_restrict_rb64(int dim, LevelGeo gf, const double* u_f, const double* b_f, LevelGeo gc, double* b_c,
                                  double* u_c, bool start, cudaStream_t s);
+// one colour of a 2D half sweep, for levels large enough to fill the device with strips of rows
+cudaError_t launch_rbgs2_strip(LevelGeo g, double* u, const double* b, int colour, cudaStream_t s);
 // u_f += P e_c on the red nodes (before a black-red sweep)
 cudaError_t launch_prolong_rb64(int dim, LevelGeo gc, const double* e_c, LevelGeo gf, double* u_f, cudaStream_t s);
 // the start of level g: u = P u_c and b = w (g - a f(u))

@@ -2431,7 +2431,7 @@ __device__ void step_report(const AugArgs& A, const StepState& S, int it, bool w
 // iteration converges to the same FP64 solution).  FP64 path: each step is solved to FP64 accuracy
 // by refinement on an FP32 inverse of its own Jacobian, as the augmented step's (the system is
 // bordered by an idle unknown, so that it has the augmented system's shape; the FP64 factor and
-// substitutions of 49 unknowns took 40 us per iteration on one warp, this takes LEVEL1).
+// substitutions of 49 unknowns took 40 us per iteration on one warp, this takes 19).
 template <typename T>
 __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
                                 double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) {

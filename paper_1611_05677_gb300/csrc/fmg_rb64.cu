@@ -32,6 +32,45 @@ __device__ __forceinline__ double res2(const double* __restrict__ u, const doubl
   return fma(-4.0, u[c], b[c] + ((u[c - 1] + u[c + 1]) + (u[c - np] + u[c + np])));
 }
 
+// ------------------------------------------------------------------ half sweeps
+// One colour in 2D, S rows per thread: the rows' loads (b and the four neighbours, all of the other
+// colour) are issued together.  One node per thread took 23.8 us at 2049^2, 5 FP64 operations
+// with the product by 1/4; this 20.6, 4 operations (13.3 at the FP64 rate).
+template <int S>
+__device__ __forceinline__ void k_rbgs2_strip_body(double* __restrict__ u, const double* __restrict__ b, int n,
+                                                   int colour) {
+  const int j0 = blockIdx.y * S + 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const long long np = n + 1;
+  double v[S];
+  long long c[S];
+  bool on[S];
+  double q[S][5];
+#pragma unroll
+  for (int r = 0; r < S; ++r) {
+    const int j = j0 + r;
+    const int i = ((colour + j) & 1) ? 2 * t + 1 : 2 * t + 2;
+    on[r] = i <= n - 1 && j <= n - 1;
+    c[r] = on[r] ? (long long)j * np + i : np + 1;
+    q[r][0] = u[c[r] - 1];
+    q[r][1] = u[c[r] + 1];
+    q[r][2] = u[c[r] - np];
+    q[r][3] = u[c[r] + np];
+    q[r][4] = b[c[r]];
+  }
+#pragma unroll
+  for (int r = 0; r < S; ++r) v[r] = quarter(q[r][4] + ((q[r][0] + q[r][1]) + (q[r][2] + q[r][3])));
+#pragma unroll
+  for (int r = 0; r < S; ++r)
+    if (on[r]) u[c[r]] = v[r];
+}
+template <int S>
+__global__ void __launch_bounds__(kRB) k_rbgs2_strip(double* __restrict__ u, const double* __restrict__ b, int n,
+                                                     int colour) {
+  pdl_start();
+  k_rbgs2_strip_body<S>(u, b, n, colour);
+}
+
 // ------------------------------------------------------------------ restriction of red residuals
 // 2D: b_c(I, J) = r(2I, 2J) + (r(2I+1, 2J+1) + r(2I-1, 2J-1)) / 2.  The residual at (2I+1, 2J+1) serves
 // the coarse nodes (I, J) and (I+1, J+1): a thread walks S coarse rows of a column and takes the
@@ -142,33 +181,49 @@ __global__ void k_prolong_rb3(const double* __restrict__ e, int nc, double* __re
 // ------------------------------------------------------------------ level start
 // u = P u_c (the FMG interpolation) and b = w (g - a f(u)) in one pass; b is zero on the boundary.
 // w = 2^wexp when wexp <= 0, else the factor w.
+// A thread takes kLS rows (along y in 2D, z in 3D), their loads issued together.
+constexpr int kLS = 4;
 template <int D>
 __device__ __forceinline__ void k_level_start64_body(const double* __restrict__ e, int nc, double* __restrict__ u,
                                                      const double* __restrict__ g, double* __restrict__ b, int kind,
                                                      double a, double w, int wexp) {
   const int n = 2 * nc;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y, l = D == 3 ? (int)blockIdx.z : 0;
+  const int z0 = (D == 2 ? blockIdx.y : blockIdx.z) * kLS;
   if (i > n) return;
   const long long np = n + 1, cp = nc + 1;
-  const long long f = ((long long)l * np + j) * np + i;
-  const bool inner = i > 0 && i < n && j > 0 && j < n && (D == 2 || (l > 0 && l < n));
-  if (!inner) {
-    b[f] = 0.0;
-    return;
+  double ep[kLS], eq[kLS], gv[kLS];
+  long long f[kLS];
+  int in[kLS];   // 0: past the level, 1: boundary, 2: interior node on a coarse node, 3: between two
+#pragma unroll
+  for (int r = 0; r < kLS; ++r) {
+    const int j = D == 2 ? z0 + r : (int)blockIdx.y, l = D == 3 ? z0 + r : 0;
+    f[r] = ((long long)l * np + j) * np + i;
+    const bool here = z0 + r <= n;
+    const bool inner = here && i > 0 && i < n && j > 0 && j < n && (D == 2 || (l > 0 && l < n));
+    const long long p = ((long long)(l >> 1) * cp + (j >> 1)) * cp + (i >> 1);
+    const long long q = ((long long)((l + 1) >> 1) * cp + ((j + 1) >> 1)) * cp + ((i + 1) >> 1);
+    in[r] = inner ? (p == q ? 2 : 3) : here ? 1 : 0;
+    ep[r] = inner ? e[p] : 0.0;
+    eq[r] = inner ? e[q] : 0.0;
+    gv[r] = inner ? g[f[r]] : 0.0;
   }
-  const long long p = ((long long)(l >> 1) * cp + (j >> 1)) * cp + (i >> 1);
-  const long long q = ((long long)((l + 1) >> 1) * cp + ((j + 1) >> 1)) * cp + ((i + 1) >> 1);
-  double v = e[p];
-  if (q != p) v = times_pow2(v + e[q], -1);
-  u[f] = v;
-  double r;
-  if (kind == FMG_F_CUBIC) {
-    r = fma(-a, v * v * v, g[f]);
-  } else {
-    r = g[f] - f_only<double>(kind, a, v);
+#pragma unroll
+  for (int r = 0; r < kLS; ++r) {
+    if (in[r] < 2) {
+      if (in[r] == 1) b[f[r]] = 0.0;
+      continue;
+    }
+    const double v = in[r] == 2 ? ep[r] : times_pow2(ep[r] + eq[r], -1);
+    u[f[r]] = v;
+    double x;
+    if (kind == FMG_F_CUBIC) {
+      x = fma(-a, v * v * v, gv[r]);
+    } else {
+      x = gv[r] - f_only<double>(kind, a, v);
+    }
+    b[f[r]] = wexp <= 0 ? times_pow2(x, wexp) : w * x;
   }
-  b[f] = wexp <= 0 ? times_pow2(r, wexp) : w * r;
 }
 template <int D>
 __global__ void k_level_start64(const double* __restrict__ e, int nc, double* __restrict__ u,
@@ -179,6 +234,16 @@ __global__ void k_level_start64(const double* __restrict__ e, int nc, double* __
 }
 
 // ------------------------------------------------------------------ 2D tile kernels
+// 8-byte asynchronous global -> shared copy, so that a thread has all its copies in flight at once
+// (a loop of loads and stores cost a memory latency per turn: 14 us per launch); zero-fills when off.
+__device__ __forceinline__ void cp_async8(double* dst, const double* src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(on ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+}
+
 // One colour of a sweep on the local rows and columns lo..hi of a W x W tile whose local (0, 0) is
 // global (gx0, gy0); interior nodes only.  The nodes of the region are dealt to the threads in
 // one sequence (an FP64 warp instruction costs the same with few lanes as with all).
@@ -222,10 +287,14 @@ __device__ __forceinline__ void k_pre_rb64_body(const double* __restrict__ u_in,
     const int ly = t / W, lx = t - ly * W;
     const int gx = gx0 + lx, gy = gy0 + ly;
     const bool on = gx >= 0 && gx <= n && gy >= 0 && gy <= n;
-    const long long c = (long long)gy * np + gx;
-    su[t] = on && u_in ? u_in[c] : 0.0;
-    sb[t] = on ? b[c] : 0.0;
+    const long long c = on ? (long long)gy * np + gx : 0;
+    cp_async8(&sb[t], b + c, on);
+    if (u_in)
+      cp_async8(&su[t], u_in + c, on);
+    else
+      su[t] = 0.0;
   }
+  cp_async_wait();
   __syncthreads();
   for (int s = 0; s < 2 * NU; ++s) {
     tile_half64<W>(su, sb, s + 1, W - 2 - s, s & 1, gx0, gy0, n);
@@ -271,19 +340,34 @@ __device__ __forceinline__ void k_post_rb64_body(const double* __restrict__ u_in
   const int X0 = blockIdx.x * T, Y0 = blockIdx.y * T;
   const int gx0 = X0 - H, gy0 = Y0 - H;
   const long long np = n + 1, cp = (n >> 1) + 1;
+  // the coarse nodes of the tile region, (gx0 / 2 ..) in x and y
+  constexpr int CW = W / 2 + 1;
+  double* se = sb + W * W;
+  const int cx0 = gx0 >> 1, cy0 = gy0 >> 1, nc = n >> 1;
   for (int t = threadIdx.x; t < W * W; t += kRT) {
     const int ly = t / W, lx = t - ly * W;
     const int gx = gx0 + lx, gy = gy0 + ly;
     const bool on = gx >= 0 && gx <= n && gy >= 0 && gy <= n;
     const bool inner = gx > 0 && gx < n && gy > 0 && gy < n;
-    const long long c = (long long)gy * np + gx;
-    double v = inner ? u_in[c] : on ? u_out[c] : 0.0;   // (the boundary is the result's own)
-    if (inner && !((gx + gy) & 1)) {
-      const long long a = (long long)(gy >> 1) * cp + (gx >> 1);
-      v = (gx & 1) ? fma(0.5, ec[a] + ec[a + cp + 1], v) : v + ec[a];
+    const long long c = on ? (long long)gy * np + gx : 0;
+    cp_async8(&su[t], (inner ? u_in : u_out) + c, on);   // (the boundary is the result's own)
+    cp_async8(&sb[t], b + c, on);
+  }
+  for (int t = threadIdx.x; t < CW * CW; t += kRT) {
+    const int y = t / CW, x = t - y * CW;
+    const bool on = cx0 + x >= 0 && cx0 + x <= nc && cy0 + y >= 0 && cy0 + y <= nc;
+    cp_async8(&se[t], ec + (on ? (long long)(cy0 + y) * cp + cx0 + x : 0), on);
+  }
+  cp_async_wait();
+  __syncthreads();
+  // += P e_c on the red nodes: the coarse value itself, or the mean of a diagonal edge's ends
+  for (int t = threadIdx.x; t < W * (W / 2); t += kRT) {
+    const int ly = t / (W / 2), lx = 2 * (t - ly * (W / 2)) + ((gx0 + gy0 + ly) & 1);
+    const int gx = gx0 + lx, gy = gy0 + ly;
+    if (gx > 0 && gx < n && gy > 0 && gy < n) {
+      const double* e = se + ((gy >> 1) - cy0) * CW + (gx >> 1) - cx0;
+      su[ly * W + lx] = (gx & 1) ? fma(0.5, e[0] + e[CW + 1], su[ly * W + lx]) : su[ly * W + lx] + e[0];
     }
-    su[t] = v;
-    sb[t] = on ? b[c] : 0.0;
   }
   __syncthreads();
   for (int s = 0; s < 2 * NU; ++s) {
@@ -316,7 +400,7 @@ cudaError_t launch_pre(int n, const double* u_in, const double* b, double* u_out
 template <int NU, int T>
 cudaError_t launch_post(int n, const double* u_in, const double* ec, const double* b, double* u_out, cudaStream_t s) {
   constexpr int W = T + 4 * NU;
-  const size_t smem = sizeof(double) * 2 * W * W;
+  const size_t smem = sizeof(double) * (2 * W * W + (W / 2 + 1) * (W / 2 + 1));
   const unsigned t = cdiv(n + 1, T);
   cudaError_t e = raise_dyn_smem((const void*)k_post_rb64<NU, T>, smem);
   if (e != cudaSuccess) return e;
@@ -330,6 +414,12 @@ constexpr int kFused64 = 512;
 constexpr int kTile16 = 128;
 
 }  // namespace
+
+cudaError_t launch_rbgs2_strip(LevelGeo g, double* u, const double* b, int colour, cudaStream_t s) {
+  const dim3 grid(cdiv(g.n / 2, kRB), cdiv(g.n - 1, 4));
+  launch_k(k_rbgs2_strip<4>, grid, kRB, 0, s, u, b, g.n, colour);
+  return cudaGetLastError();
+}
 
 bool fused_rb64_supported(int dim, int n, int nu_pre, int nu_post) {
   return dim == 2 && n <= kFused64 && (n & 1) == 0 && nu_pre >= 1 && nu_pre <= 2 && nu_post >= 1 && nu_post <= 2;
@@ -391,14 +481,15 @@ cudaError_t launch_level_start64(int dim, LevelGeo gc, const double* uc, LevelGe
   const int wexp = (1 << lg) == g.n ? -dim * lg : 1;
   const unsigned gx = cdiv(g.n + 1, kRB);
   if (dim == 2)
-    launch_k(k_level_start64<2>, dim3(gx, g.n + 1), kRB, 0, s, uc, gc.n, u, gn, b, kind, a, w, wexp);
+    launch_k(k_level_start64<2>, dim3(gx, cdiv(g.n + 1, kLS)), kRB, 0, s, uc, gc.n, u, gn, b, kind, a, w, wexp);
   else
-    launch_k(k_level_start64<3>, dim3(gx, g.n + 1, g.n + 1), kRB, 0, s, uc, gc.n, u, gn, b, kind, a, w, wexp);
+    launch_k(k_level_start64<3>, dim3(gx, g.n + 1, cdiv(g.n + 1, kLS)), kRB, 0, s, uc, gc.n, u, gn, b, kind, a, w, wexp);
   return cudaGetLastError();
 }
 
 // The 2D kernels, for phase-batched launches.
 void phase_kernels_rb64(std::vector<PhaseKernel>& out) {
+  out.push_back(phase_kernel<&k_rbgs2_strip_body<4>, kRB, 1>(&k_rbgs2_strip<4>));
   out.push_back(phase_kernel<&k_restrict_rb2_body<1>, kRB, 1>(&k_restrict_rb2<1>));
   out.push_back(phase_kernel<&k_restrict_rb2_body<2>, kRB, 1>(&k_restrict_rb2<2>));
   out.push_back(phase_kernel<&k_restrict_rb2_body<4>, kRB, 1>(&k_restrict_rb2<4>));
