@@ -195,6 +195,7 @@ size_t layout(fmg_ctx* c, const fmg_params* p, char* base) {
   const size_t items = cfg.partial_items;
   double* partials = (double*)take(2 * (items + ipow(p->coarse_cells, p->dim)) * aug_nvals(p->dim) * 8);
   double* cfin = (double*)take((ipow(p->coarse_cells + 1, p->dim) + 1) * 8);
+  double* state = (double*)take(aug_state_bytes(p->dim, p->coarse_cells, p->precision == FMG_PREC_MIXED));
   int* jtab = (int*)take(aug_jtab_ints(p->dim, p->coarse_cells) * 4);
   // the coefficient table in FP64, FP32 and float-float (a row of d entries per cell of T_H)
   const long long ncoef = ipow(p->coarse_cells, p->dim) * p->dim;
@@ -213,6 +214,7 @@ size_t layout(fmg_ctx* c, const fmg_params* p, char* base) {
     c->ab.partials = partials;
     c->ab.Ainv = Ainv;
     c->ab.cfin = cfin;
+    c->ab.state = state;
     c->ab.jtab = jtab;
     c->ab.bar_spins = 0;
     c->ab.bar_skip = -1;

@@ -368,6 +368,7 @@ struct AugBuffers {
   int nt;             // threads per block
   size_t smem;        // dynamic shared memory per block
   int sms;            // multiprocessors of the device
+  double* state;      // a correction step's state between the launches of its wide form (aug_state_bytes)
   const int* jtab;     // the mixed path's Jacobian gather table (launch_aug_jtab, once per context)
   long long bar_spins; // grid-barrier polls before a timeout (0: the default, 2^25)
   int bar_skip;        // failure-detection test hook: block that skips its first arrival (-1: none)
@@ -387,6 +388,7 @@ bool aug_shape_tuned(int dim, int coarse_cells, int level, bool mixed, AugShape*
 // Fills bpc/nt/smem/partial_items for this device (occupancy-based), outside any capture.
 void aug_configure(int dim, int coarse_cells, bool mixed, AugBuffers* ab);
 int aug_nvals(int dim);
+size_t aug_state_bytes(int dim, int coarse_cells, bool mixed);
 // ints of the mixed path's Jacobian gather table, and the kernel that fills it
 size_t aug_jtab_ints(int dim, int coarse_cells);
 cudaError_t launch_aug_jtab(int dim, int coarse_cells, int* tab, cudaStream_t s);

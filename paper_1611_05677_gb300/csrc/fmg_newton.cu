@@ -438,6 +438,8 @@ struct AugArgs {
   int bar_skip;         // test hook: this block skips its first barrier arrival (-1: none)
   VarCoef vc;           // the coefficient A(x) (vc.a64 == nullptr: A = I)
   const int* jtab;      // the Jacobian gather table (k_aug_jtab)
+  double* state;        // wide passes: the step's state between launches (null: the whole step in one launch)
+  int pass;             // wide passes: this launch's Newton iteration
   // FP64 path: the quadrature weight of each channel kind (its rows carry none)
   double wRA, wSA, wTT, wSS, wJB, wJP, wJS;
 };
@@ -2833,6 +2835,159 @@ __global__ void __launch_bounds__(256) k_aug_update(double* __restrict__ u, int 
   }
 }
 
+// The correction step's state between the launches of the wide form: the StepState arrays and the
+// kept factor as they lie in shared memory, then [0] converged, [1] stop, [2] FP64 factor, [3] the
+// iterations done.
+template <int D, bool JF32>
+__host__ __device__ size_t step_words(int nc) {   // 8-byte words before the flags
+  return (AugSmem<D, JF32>::bytes(nc) - AugSmem<D, JF32>::region(nc) + 7) / 8;
+}
+template <int D, bool JF32>
+__device__ int* step_flags(const AugArgs& A) {
+  return reinterpret_cast<int*>(A.state + step_words<D, JF32>(A.nc));
+}
+template <int D, bool JF32>
+__device__ bool step_done(const AugArgs& A) {
+  const int* f = step_flags<D, JF32>(A);
+  return (__ldcg(f) | __ldcg(f + 1)) != 0;
+}
+template <int D, bool JF32>
+__device__ void step_store(const AugArgs& A, const StepState& S, int it) {
+  const int* src = reinterpret_cast<const int*>(S.c);
+  int* dst = reinterpret_cast<int*>(A.state);
+  const int n = (int)((AugSmem<D, JF32>::bytes(A.nc) - AugSmem<D, JF32>::region(A.nc)) / 4);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+  int* f = step_flags<D, JF32>(A);
+  if (threadIdx.x < 3) f[threadIdx.x] = S.flags[threadIdx.x];
+  if (threadIdx.x == 3) f[3] = it;
+}
+// The state into shared memory; returns the iterations done.
+template <int D, bool JF32>
+__device__ int step_load(const AugArgs& A, const StepState& S) {
+  int* dst = reinterpret_cast<int*>(S.c);
+  const int* src = reinterpret_cast<const int*>(A.state);
+  const int n = (int)((AugSmem<D, JF32>::bytes(A.nc) - AugSmem<D, JF32>::region(A.nc)) / 4);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldcg(src + i);
+  const int* f = step_flags<D, JF32>(A);
+  if (threadIdx.x < 3) S.flags[threadIdx.x] = __ldcg(f + threadIdx.x);
+  const int it = __ldcg(f + 3);
+  __syncthreads();
+  return it;
+}
+
+// The coarse offset of vertex v of a cell.
+template <int D>
+__device__ __forceinline__ long long cell_vertex(int nc, int cell, int v) {
+  long long off = 0, mul = 1;
+  for (int q = 0; q < D; ++q) {
+    off += (long long)(cell % nc + ((v >> q) & 1)) * mul;
+    cell /= nc;
+    mul *= (nc + 1);
+  }
+  return off;
+}
+
+// Contexts that run side by side (batches, the server) cannot use a grid barrier, since their
+// blocks need not be resident together, and one cluster is at most 16 CTAs: a pass over 129^3
+// nodes took it most of a millisecond.  On the larger levels the first kWidePasses Newton
+// iterations are therefore launches of their own over blocks that never wait: each does its part
+// of the fine pass, the last one of a cell sums the cell's rows, and the last one of the grid takes
+// the dense step and leaves the state in A.state.  The cluster kernel then carries on with
+// whatever iterations are left (most often none) and k_augmented_wide_update writes u.
+constexpr int kWidePasses = 2;
+
+template <int D, bool JF32>
+__device__ __forceinline__ void k_augmented_wide_body(const AugArgs& A) {
+  using G = Aug<D, JF32>;
+  using FT = typename std::conditional<JF32, float, double>::type;
+  extern __shared__ double sm[];
+  double* acc = sm;
+  __shared__ double cv[G::NV];
+  __shared__ double alpha_sh;
+  __shared__ int flags_sh[3];
+  __shared__ int go_sh;
+  __shared__ int last_sh;
+  const int tid = threadIdx.x;
+  const int cell = blockIdx.x / A.bpc, bic = blockIdx.x % A.bpc;
+  const int ncell = (int)ipow(A.nc, D);
+  const int NA = (int)ipow(A.nc - 1, D) + 1;
+  const bool first = A.pass == 1;
+  StepState S;
+  FT* L;
+  AugSmem<D, JF32>::carve(sm, A.nc, S, L);
+  S.flags = flags_sh;
+  const long long alpha_at = S.sa + 1 - S.c;
+  if (tid == 0) {
+    const int abort = ((volatile int*)&A.st->abort)[0];
+    go_sh = !abort && (first || !step_done<D, JF32>(A)) ? 1 : 0;
+    alpha_sh = first ? 1.0 : __ldcg(A.state + alpha_at);
+  }
+  if (tid < G::NV) cv[tid] = first ? 0.0 : __ldcg(A.state + cell_vertex<D>(A.nc, cell, tid));
+  Rows<D, JF32>::zero(acc, first, A.fixed_point != 0, tid);
+  __syncthreads();
+  if (!go_sh) {
+    // given up in an earlier launch: the later ones find no iteration done
+    if (first && blockIdx.x == 0) {
+      step_state_init<D>(A, S);
+      step_store<D, JF32>(A, S, 0);
+    }
+    return;
+  }
+  double* pbuf = A.partials + (size_t)(A.pass & 1) * A.pstride;
+  fine_pass<D, JF32>(A, first ? kFirst : kNewton, acc, cv, alpha_sh, cell, bic);
+  block_reduce_rows<D, JF32>(A, acc, pbuf + (size_t)blockIdx.x * G::NVAL, first, A.fixed_point != 0);
+  const double* rows = pbuf;
+  if (A.bpc > 1) {
+    double* cbuf = A.partials + 2 * A.pstride + (size_t)(A.pass & 1) * ncell * G::NVAL;
+    cell_reduce<D, JF32>(A, pbuf, cbuf, cell, first, &last_sh);
+    rows = cbuf;
+  }
+  __threadfence();   // this block's rows before its arrival
+  __syncthreads();
+  if (tid == 0) last_sh = atomicAdd(&A.st->bar_count, 1u) == gridDim.x - 1 ? 1 : 0;
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();   // the other blocks' rows, after their arrivals
+  if (tid == 0) A.st->bar_count = 0u;
+  if (first)
+    step_state_init<D>(A, S);
+  else
+    step_load<D, JF32>(A, S);
+  double* cellsum = acc;
+  double* M = cellsum + (size_t)ncell * G::NVAL;
+  double* R = M + (size_t)NA * (NA + 1);
+  newton_step<D, JF32>(A, rows, cellsum, M, R, L, S, first, true);
+  __syncthreads();
+  if (flags_sh[0] || flags_sh[1]) step_report(A, S, A.pass, true);
+  if (flags_sh[1] && tid == 0) A.st->abort = 1;
+  step_store<D, JF32>(A, S, A.pass);
+}
+template <int D, bool JF32>
+__global__ void __launch_bounds__(Aug<D, JF32>::NT, 512 / Aug<D, JF32>::NT) k_augmented_wide(const __grid_constant__ AugArgs A) {
+  pdl_start();
+  k_augmented_wide_body<D, JF32>(A);
+}
+
+// u = alpha u~ + P_{H->k} c over the grid, from the state the passes left.
+template <int D, bool JF32>
+__device__ __forceinline__ void k_augmented_wide_update_body(const AugArgs& A) {
+  using G = Aug<D, JF32>;
+  __shared__ double cv[G::NV];
+  __shared__ double alpha_sh;
+  const int tid = threadIdx.x;
+  const int cell = blockIdx.x / A.bpc, bic = blockIdx.x % A.bpc;
+  if (tid < G::NV) cv[tid] = A.state[cell_vertex<D>(A.nc, cell, tid)];
+  if (tid == 0) alpha_sh = A.state[ipow(A.nc + 1, D) + ipow(A.nc - 1, D) + 1];   // StepState: c, t, then s and alpha
+  __syncthreads();
+  fine_pass<D, JF32>(A, kUpdate, nullptr, cv, alpha_sh, cell, bic);
+}
+template <int D, bool JF32>
+__global__ void __launch_bounds__(Aug<D, JF32>::NT, 512 / Aug<D, JF32>::NT)
+    k_augmented_wide_update(const __grid_constant__ AugArgs A) {
+  pdl_start();
+  k_augmented_wide_update_body<D, JF32>(A);
+}
+
 template <int D, bool JF32>
 __device__ __forceinline__ void k_augmented_cluster_body(const AugArgs& A) {
   using G = Aug<D, JF32>;
@@ -2868,8 +3023,14 @@ __device__ __forceinline__ void k_augmented_cluster_body(const AugArgs& A) {
   };
   step_state_init<D>(A, S);
   const bool writer = rank == 0;
-  int it = 0;
-  for (it = 1; it <= A.maxit; ++it) {
+  int it = 1;
+  if (A.state) {
+    // the wide passes' iterations are done: carry on from their state, or leave what they finished
+    if (step_done<D, JF32>(A)) return;
+    it = step_load<D, JF32>(A, S) + 1;
+  }
+  bool iterated = false;
+  for (; it <= A.maxit; ++it) {
     const bool first = it == 1;
     double* pbuf = A.partials + (size_t)(it & 1) * A.pstride;
     if (tid == 0) stop = ((volatile int*)&A.st->abort)[0];
@@ -2883,12 +3044,19 @@ __device__ __forceinline__ void k_augmented_cluster_body(const AugArgs& A) {
       block_reduce_rows<D, JF32>(A, acc, pbuf + (size_t)cell * G::NVAL, first, A.fixed_point != 0);
     }
     cluster.sync();
+    iterated = true;
     newton_step<D, JF32>(A, pbuf, cellsum, M, R, L, S, first, writer);
     __syncthreads();
     if (flags_sh[0] || flags_sh[1]) break;
   }
   step_report(A, S, it, writer);
   if (flags_sh[1] && writer && tid == 0) A.st->abort = 1;
+  if (A.state) {
+    // the update is a launch of its own; without an iteration here the stored iterate stands (after
+    // one, every CTA has passed a cluster barrier since it read the state)
+    if (writer && iterated) step_store<D, JF32>(A, S, it);
+    return;
+  }
   for (int cell = rank; cell < ncell; cell += CS) {
     if (tid < G::NV) cv[tid] = S.c[vertex_offset(cell, tid)];
     __syncthreads();
@@ -3114,6 +3282,30 @@ AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const Aug
   return sh;
 }
 
+namespace {
+// Nodes per thread of the cluster from which the step's passes are launches over the whole device.
+// A burst of 24 mixed 2D and 3D requests: 4.37 ms with the cluster kernel alone, 3.67 from 32
+// nodes per thread, 3.65 from 8 and from 2; a batch of 32: 2.28, 2.17 and 2.15 ms (2.37 from 2
+// with chunks of 8 nodes).  Chunks of 16 or 8 nodes over more blocks gave 2.23 and 2.37 ms: the
+// blocks of the other instances fill the device.  The cluster kernel keeps the levels below; smaller
+// clusters for those were slower (4 nodes per thread: 2.49 and 5.08 ms).
+constexpr long long kWideNodes = 8;
+
+template <int D, bool JF32>
+cudaError_t launch_wide(const AugArgs& W, size_t smem, cudaStream_t s) {
+  cudaError_t e = raise_dyn_smem((const void*)k_augmented_wide<D, JF32>, smem);
+  if (e != cudaSuccess) return e;
+  launch_k(k_augmented_wide<D, JF32>, dim3((unsigned)(ipow(W.nc, D) * W.bpc)), Aug<D, JF32>::NT, smem, s, W);
+  return cudaGetLastError();
+}
+}  // namespace
+
+size_t aug_state_bytes(int dim, int coarse_cells, bool mixed) {
+  const size_t w = dim == 2 ? (mixed ? step_words<2, true>(coarse_cells) : step_words<2, false>(coarse_cells))
+                            : (mixed ? step_words<3, true>(coarse_cells) : step_words<3, false>(coarse_cells));
+  return w * 8 + 4 * sizeof(int);
+}
+
 cudaError_t launch_augmented(int dim, int coarse_cells, int level, LevelGeo gk, double* u, const double* gn,
                              int kind, double a, double tol, int maxit, bool jac_f32, const AugBuffers& ab,
                              DevState* st, int level_index, cudaStream_t s, int cluster_size, int fixed_point,
@@ -3175,9 +3367,25 @@ cudaError_t launch_augmented(int dim, int coarse_cells, int level, LevelGeo gk, 
   // the statistics; a completed barrier leaves its count at zero and generations only grow, so
   // the launches of one solve need no reset between them
   cudaError_t e = cudaSuccess;
+  A.state = nullptr;
+  A.pass = 0;
   if (cluster_size > 0) {
     if (A.vc.a64) return cudaErrorInvalidValue;   // batches and the server take A = I only
     A.bpc = 1;
+    const bool wide = ab.state && gk.nodes > kWideNodes * cluster_size * nt;
+    const AugShape ws = aug_shape(dim, coarse_cells, level, jac_f32, ab, true, false);
+    if (wide) {
+      AugArgs W = A;
+      W.state = ab.state;
+      W.chunk = ws.chunk;
+      W.bpc = ws.bpc;
+      for (W.pass = 1; W.pass <= kWidePasses && W.pass <= maxit; ++W.pass) {
+        e = dim == 2 ? (jac_f32 ? launch_wide<2, true>(W, smem, s) : launch_wide<2, false>(W, smem, s))
+                     : (jac_f32 ? launch_wide<3, true>(W, smem, s) : launch_wide<3, false>(W, smem, s));
+        if (e != cudaSuccess) return e;
+      }
+      A.state = ab.state;
+    }
     cudaLaunchConfig_t cc = {};
     cc.gridDim = dim3(cluster_size);
     cc.blockDim = dim3(nt);
@@ -3190,12 +3398,28 @@ cudaError_t launch_augmented(int dim, int coarse_cells, int level, LevelGeo gk, 
     ca[0].val.clusterDim.z = 1;
     cc.attrs = ca;
     cc.numAttrs = 1;
+    if (dim == 2)
+      e = jac_f32 ? cudaLaunchKernelEx(&cc, k_augmented_cluster<2, true>, A)
+                  : cudaLaunchKernelEx(&cc, k_augmented_cluster<2, false>, A);
+    else
+      e = jac_f32 ? cudaLaunchKernelEx(&cc, k_augmented_cluster<3, true>, A)
+                  : cudaLaunchKernelEx(&cc, k_augmented_cluster<3, false>, A);
+    if (e != cudaSuccess || !wide) return e;
+    A.chunk = ws.chunk;
+    A.bpc = ws.bpc;
+    const unsigned blocks = (unsigned)(ncell * ws.bpc);
     if (dim == 2) {
-      if (jac_f32) return cudaLaunchKernelEx(&cc, k_augmented_cluster<2, true>, A);
-      return cudaLaunchKernelEx(&cc, k_augmented_cluster<2, false>, A);
+      if (jac_f32)
+        launch_k(k_augmented_wide_update<2, true>, dim3(blocks), nt, 0, s, A);
+      else
+        launch_k(k_augmented_wide_update<2, false>, dim3(blocks), nt, 0, s, A);
+    } else {
+      if (jac_f32)
+        launch_k(k_augmented_wide_update<3, true>, dim3(blocks), nt, 0, s, A);
+      else
+        launch_k(k_augmented_wide_update<3, false>, dim3(blocks), nt, 0, s, A);
     }
-    if (jac_f32) return cudaLaunchKernelEx(&cc, k_augmented_cluster<3, true>, A);
-    return cudaLaunchKernelEx(&cc, k_augmented_cluster<3, false>, A);
+    return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ncell * bpc);
@@ -3248,6 +3472,14 @@ void phase_kernels_newton(std::vector<PhaseKernel>& out) {
       &k_augmented_cluster<2, true>));
   out.push_back(phase_kernel<&k_augmented_cluster_body<2, false>, Aug<2, false>::NT, 512 / Aug<2, false>::NT>(
       &k_augmented_cluster<2, false>));
+  out.push_back(phase_kernel<&k_augmented_wide_body<2, true>, Aug<2, true>::NT, 512 / Aug<2, true>::NT>(
+      &k_augmented_wide<2, true>));
+  out.push_back(phase_kernel<&k_augmented_wide_body<2, false>, Aug<2, false>::NT, 512 / Aug<2, false>::NT>(
+      &k_augmented_wide<2, false>));
+  out.push_back(phase_kernel<&k_augmented_wide_update_body<2, true>, Aug<2, true>::NT, 512 / Aug<2, true>::NT>(
+      &k_augmented_wide_update<2, true>));
+  out.push_back(phase_kernel<&k_augmented_wide_update_body<2, false>, Aug<2, false>::NT, 512 / Aug<2, false>::NT>(
+      &k_augmented_wide_update<2, false>));
 }
 
 }  // namespace fmg
