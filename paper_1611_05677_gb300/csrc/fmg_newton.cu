@@ -93,14 +93,9 @@ __device__ __forceinline__ double recip_pivot(double d) {
 // drop_last and the last pivot (the Schur complement of the last unknown) falls below drop_tol
 // times the original last diagonal entry, rd[n-1] = 0: that unknown is frozen (*dropped = 1).
 // Returns false if a pivot is not positive.
-template <typename T, int NS, int FN = 0, int FBAND = 0>
-__device__ bool ldlt_band_warp_ns(T* A, int n_arg, int ld_arg, T* rd, int band_arg, int border, bool drop_last,
-                                  double drop_tol, int* dropped) {
-  // FN, FBAND > 0: the size and band fixed at compile time (ld = FN + 1), which folds the
-  // offsets and strides into constants
-  const int n = FN > 0 ? FN : n_arg;
-  const int ld = FN > 0 ? FN + 1 : ld_arg;
-  const int band = FBAND > 0 ? FBAND : band_arg;
+template <typename T, int NS>
+__device__ bool ldlt_band_warp_ns(T* A, int n, int ld, T* rd, int band, int border, bool drop_last, double drop_tol,
+                                  int* dropped) {
   const int lane = threadIdx.x & 31;
   const int nb = n - border;
   const int q = band + border;
@@ -1607,171 +1602,126 @@ __global__ void k_aug_jtab(int nc, int* __restrict__ tab) {
   }
 }
 
-// Largest lexicographic half-bandwidth of J_HH (aug_band) of a dimension: 2D 1/H <= 8 gives
-// 8, 3D 1/H <= 4 gives 13.
-template <int D>
-__host__ __device__ constexpr int aug_band_max() {
-  return D == 2 ? 8 : 13;
-}
-
-// Column c of J^{-1} from the band LDL^T factor of ldlt_band_warp (A in place: A[i][k] =
-// L_ik d_k below the diagonal, rd[k] = 1/d_k; band rows 0..nb-1, dense border row nb = n - 1):
-// the forward substitution L w = e_c with y = D^{-1} w kept in X's column, then the backward
-// substitution L^T x = y over the band and the border entry.  The band window of the last KB
-// values is kept in registers; every thread walks the same rows, so the factor's entries are
-// shared-memory broadcasts.
-template <int D>
-__device__ __forceinline__ void band_inverse_column(const float* __restrict__ Af, const float* __restrict__ rd, int n,
-                                                    int ld, int band, int c, float* __restrict__ X) {
-  constexpr int KB = aug_band_max<D>();
-  const int nb = n - 1;
-  // win[t] holds the value of the row t + 1 steps back (forward) or ahead (backward); the
-  // newest one (t = 0) enters each sum last, so the rest of the sum does not wait for it
-  float win[KB];
+// The inverse of the n x n SPD matrix in A (FP32, row-major, leading dimension ld, lower triangle
+// read) by the symmetric sweep operator, two unknowns at a time, over a block of NT threads: a
+// thread keeps a tile of TR x 4 entries in registers, a step publishes the two pivot rows in shared
+// memory (one barrier) and subtracts their rank-2 update.  X (ld too, both triangles) may be A itself.
+// n <= 64 (NT = 256) or 32 (NT = 128); padding unknowns are uncoupled, with diagonal 1.  The last unknown is left out (its row
+// and column of X zero, *dropped = 1) if drop_last and its pivot, the Schur complement, is at most
+// drop_tol times its diagonal.  Returns false in every thread if a pivot is not positive.
+// Bound by the chain from one pair of pivots to the next (two reciprocals, a barrier, the loads) and
+// by the loads' shared-memory bandwidth, hence square tiles (14 rows of one column per thread: 16.9k
+// cycles at n = 50).  The band LDL^T on one warp and a column of the inverse per thread, which this
+// replaced, took 13.7k + 11.1k cycles at n = 50 and band 8 (256 threads) and 12.6k + 8.4k at n = 28
+// (128 threads); this 14.7k and 6.8k.
+template <int NT>
+__device__ bool sweep_inverse(const float* A, int n, int ld, float* X, bool drop_last, float drop_tol, int* dropped) {
+  constexpr int TC = 4, TXN = NT == 256 ? 16 : 8, TR = TXN * TC / (NT / TXN);   // 64^2 in 4 x 4, 32^2 in 2 x 4
+  static_assert(TR == 2 || TR == 4, "a pair of pivot rows lies in one tile");
+  __shared__ __align__(16) float v[2][2][TXN * TC];
+  const int tx = threadIdx.x % TXN, ty = threadIdx.x / TXN;
+  const bool active = ty * TR < n;
+  float a[TR][TC];
 #pragma unroll
-  for (int t = 0; t < KB; ++t) win[t] = 0.f;
-  for (int k = 0; k < nb; ++k) {
-    float s0 = 0.f, s1 = 0.f;
+  for (int r = 0; r < TR; ++r)
 #pragma unroll
-    for (int t = KB - 1; t >= 1; --t) {
-      const int j = k - 1 - t;
-      if (t < band && j >= 0) {
-        if (t & 1)
-          s1 = fmaf(Af[k * ld + j], win[t], s1);
-        else
-          s0 = fmaf(Af[k * ld + j], win[t], s0);
-      }
+    for (int c = 0; c < TC; ++c) {
+      const int i = ty * TR + r, k = tx * TC + c;
+      const int hi = max(i, k), lo = min(i, k);
+      a[r][c] = hi < n ? A[hi * ld + lo] : (i == k ? 1.f : 0.f);
     }
-    const float a0 = k >= 1 ? Af[k * ld + k - 1] : 0.f;
-    const float y = ((k == c ? 1.f : 0.f) - fmaf(a0, win[0], s0 + s1)) * rd[k];
-    X[k * ld + c] = y;
-#pragma unroll
-    for (int t = KB - 1; t > 0; --t) win[t] = win[t - 1];
-    win[0] = y;
-  }
-  {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    int j = 0;
-    for (; j + 3 < nb; j += 4) {
-      s0 = fmaf(Af[nb * ld + j], X[j * ld + c], s0);
-      s1 = fmaf(Af[nb * ld + j + 1], X[(j + 1) * ld + c], s1);
-      s2 = fmaf(Af[nb * ld + j + 2], X[(j + 2) * ld + c], s2);
-      s3 = fmaf(Af[nb * ld + j + 3], X[(j + 3) * ld + c], s3);
-    }
-    for (; j < nb; ++j) s0 = fmaf(Af[nb * ld + j], X[j * ld + c], s0);
-    X[nb * ld + c] = ((nb == c ? 1.f : 0.f) - ((s0 + s1) + (s2 + s3))) * rd[nb];
-  }
-  const float xb = X[nb * ld + c];
-#pragma unroll
-  for (int t = 0; t < KB; ++t) win[t] = 0.f;
-  for (int k = nb - 1; k >= 0; --k) {
-    float s0 = Af[nb * ld + k] * xb, s1 = 0.f;
-#pragma unroll
-    for (int t = KB - 1; t >= 1; --t) {
-      const int i = k + 1 + t;
-      if (t < band && i < nb) {
-        if (t & 1)
-          s1 = fmaf(Af[i * ld + k], win[t], s1);
-        else
-          s0 = fmaf(Af[i * ld + k], win[t], s0);
-      }
-    }
-    const float a0 = k + 1 < nb ? Af[(k + 1) * ld + k] : 0.f;
-    const float x = X[k * ld + c] - rd[k] * fmaf(a0, win[0], s0 + s1);
-    X[k * ld + c] = x;
-#pragma unroll
-    for (int t = KB - 1; t > 0; --t) win[t] = win[t - 1];
-    win[0] = x;
-  }
-}
-
-// The same column for a size and band fixed at compile time (the dense systems of the
-// benchmark shapes).  The band window lives in W = BAND + 1 registers addressed modulo W, and
-// the substitutions are unrolled W steps at a time, so every window slot and every offset into
-// the factor is a compile-time constant: the loads of a step are issued ahead and only the FMA
-// chain through the newest value stays on the critical path.
-template <int NA, int BAND>
-__device__ __forceinline__ void band_inverse_column_fixed(const float* __restrict__ Af, const float* __restrict__ rd,
-                                                          int c, float* __restrict__ X) {
-  constexpr int ld = NA + 1, nb = NA - 1, W = BAND + 1;
-  float win[W];
-#pragma unroll
-  for (int m = 0; m < W; ++m) win[m] = 0.f;
-  // one forward step: y_k = ([k == c] - sum_{t=1..BAND} A[k][k-t] y_{k-t}) / d_k; the older
-  // terms go into two partial sums, the newest (t = 1) is added last; `guard`: rows near the top,
-  // where k - t < 0 (decided at compile time in the peeled first block)
-  auto fwd = [&](int k, int kk, bool guard) {
-    float p0 = 0.f, p1 = 0.f;
-#pragma unroll
-    for (int t = BAND; t >= 2; --t) {
-      if (guard && k - t < 0) continue;
-      if (t & 1)
-        p1 = fmaf(Af[k * ld + k - t], win[(kk - t + W) % W], p1);
-      else
-        p0 = fmaf(Af[k * ld + k - t], win[(kk - t + W) % W], p0);
-    }
-    float sum = p0 + p1;
-    if (!guard || k >= 1) sum = fmaf(Af[k * ld + k - 1], win[(kk - 1 + W) % W], sum);
-    const float y = ((k == c ? 1.f : 0.f) - sum) * rd[k];
-    win[kk] = y;
-    X[k * ld + c] = y;
+  const float drop_at = drop_last ? drop_tol * A[(n - 1) * ld + n - 1] : 0.f;
+  auto publish = [&](int b, int r) {
+    *reinterpret_cast<float4*>(&v[b][0][tx * TC]) = make_float4(a[r][0], a[r][1], a[r][2], a[r][3]);
+    *reinterpret_cast<float4*>(&v[b][1][tx * TC]) = make_float4(a[r + 1][0], a[r + 1][1], a[r + 1][2], a[r + 1][3]);
   };
-#pragma unroll
-  for (int kk = 0; kk < W; ++kk)
-    if (kk < nb) fwd(kk, kk, true);
-  for (int k0 = W; k0 < nb; k0 += W) {
-#pragma unroll
-    for (int kk = 0; kk < W; ++kk)
-      if (k0 + kk < nb) fwd(k0 + kk, kk, false);
-  }
-  {
-    float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int j = 0; j < nb; ++j) s4[j & 3] = fmaf(Af[nb * ld + j], X[j * ld + c], s4[j & 3]);
-    X[nb * ld + c] = ((nb == c ? 1.f : 0.f) - ((s4[0] + s4[1]) + (s4[2] + s4[3]))) * rd[nb];
-  }
-  const float xb = X[nb * ld + c];
-  // one backward step: x_k = y_k - (sum_{t=1..BAND} A[k+t][k] x_{k+t} + A[nb][k] x_nb) / d_k,
-  // from the top (guard: rows where k + t >= nb)
-#pragma unroll
-  for (int m = 0; m < W; ++m) win[m] = 0.f;
-  auto bwd = [&](int k, int kk, bool guard) {
-    float p0 = Af[nb * ld + k] * xb, p1 = 0.f;
-#pragma unroll
-    for (int t = BAND; t >= 2; --t) {
-      if (guard && k + t >= nb) continue;
-      if (t & 1)
-        p1 = fmaf(Af[(k + t) * ld + k], win[(kk - t + W) % W], p1);
-      else
-        p0 = fmaf(Af[(k + t) * ld + k], win[(kk - t + W) % W], p0);
-    }
-    float sum = p0 + p1;
-    if (!guard || k + 1 < nb) sum = fmaf(Af[(k + 1) * ld + k], win[(kk - 1 + W) % W], sum);
-    const float x = X[k * ld + c] - rd[k] * sum;
-    win[kk] = x;
-    X[k * ld + c] = x;
+  if (ty == 0) publish(0, 0);
+  __syncthreads();
+  unsigned bad = 0u, drop = 0u;
+  const int last = drop_last ? n - 1 : -1;
+  auto recip = [&](int k, float d) {
+    const unsigned out = (unsigned)(k == last) & (unsigned)!(d > drop_at);
+    const unsigned neg = (out ^ 1u) & (unsigned)!(d > 0.f);
+    drop |= out;
+    bad |= neg;
+    const float y = recip_pivot(d);
+    return (out | neg) != 0u ? 0.f : y;
   };
+#pragma unroll 1
+  for (int k4 = 0; k4 < n; k4 += 4) {
 #pragma unroll
-  for (int kk = 0; kk < W; ++kk)
-    if (nb - 1 - kk >= 0) bwd(nb - 1 - kk, kk, true);
-  for (int k0 = nb - 1 - W; k0 >= 0; k0 -= W) {
+    for (int h = 0; h < 2; ++h) {
+      const int k = k4 + 2 * h;
+      if (k >= n) break;
+      const float* v0 = v[h][0];
+      const float* v1 = v[h][1];
+      // every load ahead of the reciprocals' chain
+      float y0[TR], y1[TR], x0[TC], x1[TC], s0[TC], s1[TC];
+      const float p = v0[k], c = v0[k + 1], d = v1[k + 1];
+      *reinterpret_cast<float4*>(x0) = *reinterpret_cast<const float4*>(&v0[tx * TC]);
+      *reinterpret_cast<float4*>(x1) = *reinterpret_cast<const float4*>(&v1[tx * TC]);
+      if constexpr (TR == 4) {
+        *reinterpret_cast<float4*>(y0) = *reinterpret_cast<const float4*>(&v0[ty * TR]);
+        *reinterpret_cast<float4*>(y1) = *reinterpret_cast<const float4*>(&v1[ty * TR]);
+      } else {
+        *reinterpret_cast<float2*>(y0) = *reinterpret_cast<const float2*>(&v0[ty * TR]);
+        *reinterpret_cast<float2*>(y1) = *reinterpret_cast<const float2*>(&v1[ty * TR]);
+      }
+      // the inverse of the 2 x 2 pivot block [p c; c d]: e00 e01; e01 e11 = d1
+      const float d0 = recip(k, p);
+      const float l = c * d0;
+      const float d1 = recip(k + 1, fmaf(-l, c, d));
+      const float e01 = -l * d1, e00 = fmaf(-l, e01, d0);
+      if (active) {
+        // the pivot rows become the block's inverse times themselves, negated at the block
 #pragma unroll
-    for (int kk = 0; kk < W; ++kk)
-      if (k0 - kk >= 0) bwd(k0 - kk, kk, false);
+        for (int q = 0; q < TC; ++q) {
+          s0[q] = fmaf(e00, x0[q], e01 * x1[q]);
+          s1[q] = fmaf(e01, x0[q], d1 * x1[q]);
+        }
+        const bool pc = tx == k4 / TC, pr = ty == k / TR;
+        s0[2 * h] = pc ? -e00 : s0[2 * h];
+        s1[2 * h] = pc ? -e01 : s1[2 * h];
+        s0[2 * h + 1] = pc ? -e01 : s0[2 * h + 1];
+        s1[2 * h + 1] = pc ? -d1 : s1[2 * h + 1];
+#pragma unroll
+        for (int r = 0; r < TR; ++r) {
+          a[r][2 * h] = pc ? 0.f : a[r][2 * h];
+          a[r][2 * h + 1] = pc ? 0.f : a[r][2 * h + 1];
+        }
+        // the next pivot rows first, so that they are on their way while the others are updated
+        constexpr int kLocal = TR == 4 ? 2 : 0;   // (a tile of two rows holds one pair)
+        const int next = (h ^ 1) * kLocal;
+        auto update = [&](int r) {
+#pragma unroll
+          for (int q = 0; q < TC; ++q) a[r][q] = fmaf(-y1[r], s1[q], fmaf(-y0[r], s0[q], a[r][q]));
+        };
+        update(next);
+        update(next + 1);
+        if (ty == (k + 2) / TR) publish(h ^ 1, next);
+        if constexpr (TR == 4) {
+          update(2 - next);
+          update(3 - next);
+        }
+#pragma unroll
+        for (int q = 0; q < TC; ++q) {
+          a[h * kLocal][q] = pr ? s0[q] : a[h * kLocal][q];
+          a[h * kLocal + 1][q] = pr ? s1[q] : a[h * kLocal + 1][q];
+        }
+      }
+      __syncthreads();
+    }
   }
-}
-
-// Column c of J^{-1}: the unrolled form for the sizes it is instantiated for, else the loop.
-template <int D>
-__device__ __forceinline__ void band_inverse_dispatch(const float* Af, const float* rd, int n, int ld, int band, int c,
-                                                      float* X) {
-  if constexpr (D == 2) {
-    if (n == 50 && band == 8) return band_inverse_column_fixed<50, 8>(Af, rd, c, X);
-    if (n == 10 && band == 4) return band_inverse_column_fixed<10, 4>(Af, rd, c, X);
-  } else {
-    if (n == 28 && band == 13) return band_inverse_column_fixed<28, 13>(Af, rd, c, X);
-  }
-  band_inverse_column<D>(Af, rd, n, ld, band, c, X);
+  if (dropped) *dropped = (int)drop;
+#pragma unroll
+  for (int r = 0; r < TR; ++r)
+#pragma unroll
+    for (int c = 0; c < TC; ++c) {
+      const int i = ty * TR + r, k = tx * TC + c;
+      if (i < n && k < n) X[i * ld + k] = -a[r][c];
+    }
+  __syncthreads();
+  return bad == 0u;
 }
 
 // y = X r for the n x n matrix X (leading dimension ld) and r in FP32, by all warps: a row per
@@ -1845,9 +1795,8 @@ __device__ void newton_update_mixed(const AugArgs& A, const float* y, int NH, co
 // (N_H+1)-dimensional system of eq. 3.6 on V_H + span{u~} is formed in FP64 from the cell
 // sums (the first pass's sums are kept and the later passes' increments added to them).  The
 // first iteration also assembles the Jacobian (fixed point: the Galerkin stiffness) in FP32
-// from the FP32 channels directly into the band-plus-border pattern, factors it by the band
-// LDL^T on one warp and forms its inverse from the factor (a column per thread), which is
-// kept in shared memory: every iteration's step is then y = J^{-1} R, a block-wide
+// from the FP32 channels directly into the band-plus-border pattern and forms its inverse
+// (sweep_inverse), which is kept in shared memory: every iteration's step is then y = J^{-1} R, a block-wide
 // matrix-vector product, so the later iterations are chord steps at the cost of one product.
 // If the last pivot (the Schur complement of alpha) falls below 1e-6 of its original
 // diagonal entry, alpha is frozen (its row and column of the inverse are zero).
@@ -1864,11 +1813,9 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
   const int NA = NH + 1;
   const int ld = NA + 1;
   const bool fixedp = A.fixed_point != 0;
-  float* X = reinterpret_cast<float*>(Mreg);   // J^{-1} as it is formed [NA][ld]
-  float* rf = X + (size_t)NA * ld;             // R in FP32 [NA]
+  float* rf = reinterpret_cast<float*>(Mreg);   // R in FP32 [NA]
   float* dl = rf + NA;                         // the step y = J^{-1} R [NA]
   __shared__ float s3_sh;
-  __shared__ int fac_sh[2];
   __shared__ unsigned red_sh[3];
   if (tid == 0) red_sh[0] = red_sh[1] = red_sh[2] = 0u;
   // ---- cell sums (one row per coarse cell): the residual channels in FP64, in the first
@@ -1963,7 +1910,6 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
   };
   int dropped = 0;
   bool ok = true;
-  const float* Xuse = L;   // the kept inverse (chord steps)
   if (!first) {
     form_residual(tid, nthr);
     __syncthreads();
@@ -2009,40 +1955,12 @@ __device__ __noinline__ void newton_step_mixed(const AugArgs& A, const double* _
     }
     if (tid == 0) L[NH * ld + NH] = (float)S.sa[0] + (fixedp ? 0.f : s3_sh);
     __syncthreads();
-    // ---- band LDL^T of J on warp 0 while the other warps form the residual, then the inverse,
-    // a column per thread
-    const int band = aug_band<D>(A.nc);
-    float* rd = L + (size_t)NA * ld;
-    if (tid < 32) {
-      int dr = 0;
-      bool okw;
-      // the benchmark shapes with their size and band fixed at compile time
-      if (D == 2 && NA == 50 && band == 8)
-        okw = ldlt_band_warp_ns<float, 2, 50, 8>(L, NA, ld, rd, band, 1, true, 1e-6, &dr);
-      else if (D == 2 && NA == 10 && band == 4)
-        okw = ldlt_band_warp_ns<float, 1, 10, 4>(L, NA, ld, rd, band, 1, true, 1e-6, &dr);
-      else if (D == 3 && NA == 28 && band == 13)
-        okw = ldlt_band_warp_ns<float, 4, 28, 13>(L, NA, ld, rd, band, 1, true, 1e-6, &dr);
-      else
-        okw = ldlt_band_warp<float>(L, NA, ld, rd, band, 1, true, 1e-6, &dr);
-      if (tid == 0) {
-        fac_sh[0] = okw ? 1 : 0;
-        fac_sh[1] = dr;
-      }
-    } else {
-      form_residual(tid - 32, nthr - 32);
-    }
-    __syncthreads();
-    ok = fac_sh[0] != 0;
-    dropped = fac_sh[1];
-    if (tid < NA) band_inverse_dispatch<D>(L, rd, NA, ld, band, tid, X);
-    __syncthreads();
-    // keep J^{-1} where the factor was (the factor is no longer needed)
-    for (int i = tid; i < NA * ld; i += nthr) L[i] = X[i];
-    Xuse = X;
+    // ---- the residual, then the inverse, kept in place for the chord steps
+    form_residual(tid, nthr);
+    ok = sweep_inverse<Aug<D, true>::NT>(L, NA, ld, L, true, 1e-6f, &dropped);
   }
   // ---- the step y = J^{-1} R, then (c, alpha) += y and the convergence test
-  small_matvec<Aug<D, true>::NT>(Xuse, NA, ld, rf, dl);
+  small_matvec<Aug<D, true>::NT>(L, NA, ld, rf, dl);
   __syncthreads();
   newton_update_mixed<D>(A, dl, NH, S, dropped, ok, writer, red_sh);
 }
@@ -2101,7 +2019,7 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
 // The FP64 path's linear solve J y = R.  FP64 elimination on one warp is a chain of FP64
 // operations (a band LDL^T of 50 unknowns 28 us, the two substitutions 18 us, per Newton
 // iteration), so the system is solved by iterative refinement instead: an FP32 inverse X of the
-// first iteration's Jacobian (the mixed path's band LDL^T and inverse columns) is kept for the
+// first iteration's Jacobian (sweep_inverse, as in the mixed path) is kept for the
 // correction step, and y <- y + X (R - J y) with the residual, J and y in FP64 runs until the next
 // correction would be below the rounding of y.  The solution has FP64 accuracy whatever the
 // accuracy of X, which sets the rate only: about 1e-5 per sweep with its own J, ||I - X J|| with
@@ -2344,27 +2262,13 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
   const int band = aug_band<D>(A.nc);
   int dropped = 0;
   bool ok = true;
-  // X, then the FP32 factor and its reciprocal pivots, where the FP64 factor would be
+  // X (FP32) where the FP64 factor would be
   float* X = reinterpret_cast<float*>(L);
   if ((first || NA <= kRefineFresh) && !S.flags[2]) {
-    float* Lf = X + (size_t)NA * ld;
-    float* rd = Lf + (size_t)NA * ld;
-    for (int i = tid; i < NA * ld; i += nthr) Lf[i] = (float)M[i];
+    for (int i = tid; i < NA * ld; i += nthr) X[i] = (float)M[i];
     __syncthreads();
-    if (tid < 32) {
-      bool okw;
-      if (D == 2 && NA == 50 && band == 8)
-        okw = ldlt_band_warp_ns<float, 2, 50, 8>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
-      else if (D == 2 && NA == 10 && band == 4)
-        okw = ldlt_band_warp_ns<float, 1, 10, 4>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
-      else if (D == 3 && NA == 28 && band == 13)
-        okw = ldlt_band_warp_ns<float, 4, 28, 13>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
-      else
-        okw = ldlt_band_warp<float>(Lf, NA, ld, rd, band, 1, true, kRefinePivot, &dropped);
-      if (tid == 0 && (!okw || dropped)) S.flags[2] = 1;
-    }
-    __syncthreads();
-    if (!S.flags[2] && tid < NA) band_inverse_dispatch<D>(Lf, rd, NA, ld, band, tid, X);
+    const bool okw = sweep_inverse<nthr>(X, NA, ld, X, true, kRefinePivot, &dropped);
+    if (tid == 0 && (!okw || dropped)) S.flags[2] = 1;
     __syncthreads();
   }
   if (!S.flags[2]) {
@@ -2429,7 +2333,7 @@ __device__ void step_report(const AugArgs& A, const StepState& S, int it, bool w
 
 // Algorithm 3.2 step 1: Newton on A_1 U + w f(U) = w g, from U = 0 (one CTA).  The residual,
 // the iterate and the convergence test are FP64.  Mixed path: the Jacobian A_1 + diag(w f'(U)) is
-// factored in FP32 (an inexact Newton step whose error the next FP64 residual corrects, so the
+// inverted in FP32 (an inexact Newton step whose error the next FP64 residual corrects, so the
 // iteration converges to the same FP64 solution).  FP64 path: each step is solved to FP64 accuracy
 // by refinement on an FP32 inverse of its own Jacobian, as the augmented step's (the system is
 // bordered by an idle unknown, so that it has the augmented system's shape; the FP64 factor and
@@ -2445,10 +2349,10 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
   double* rhs = U + N;
   double* Fp = rhs + N + 1;   // (rhs: the FP64 path borders the system)
   T* L = reinterpret_cast<T*>(Fp + N);
-  T* work = L + (size_t)N * ld;
-  T* invd = work + N;
-  // FP64 path, bordered: the Jacobian M, the FP64 factor's place F (X, then the FP32 factor and its
-  // reciprocal pivots, until it is needed), an FP32 copy of A_1 and A_1's diagonal
+  T* work = L + (size_t)N * ld;   // mixed path: the right-hand side and the step in FP32
+  T* step = work + N;
+  // FP64 path, bordered: the Jacobian M, the FP64 factor's place F (the FP32 inverse X until it is
+  // needed), an FP32 copy of A_1 and A_1's diagonal
   constexpr bool kRefine = sizeof(T) == 8;
   const int NA = N + 1, lda = NA + 1;
   double* M = Fp + N;
@@ -2465,7 +2369,6 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
   const double w = dim == 2 ? h * h : h * h * h;
   const int band = dim == 2 ? m : m * m;   // lexicographic half-bandwidth of the 2d+1-point stencil
   for (int i = threadIdx.x; i < N; i += blockDim.x) U[i] = 0.0;
-  // entries outside the band are zero and the factorization never writes them
   if constexpr (kRefine) {
     for (int i = tid; i < NA * lda; i += blockDim.x) {
       const int p = i / lda, q = i - p * lda;
@@ -2475,8 +2378,6 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
       if (p == q && p < N) dg[p] = v;
     }
     if (tid == 0) use64 = 0;
-  } else {
-    for (int i = tid; i < N * ld; i += blockDim.x) L[i] = T(0);
   }
   if (tid == 0) done = 0;
   __syncthreads();
@@ -2519,16 +2420,14 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
     __syncthreads();
     if constexpr (kRefine) {
       float* X = reinterpret_cast<float*>(F);
-      float* Lf = X + (size_t)NA * lda;
-      float* rd = Lf + (size_t)NA * lda;
       if (!use64) {
-        for (int i = tid; i < NA * lda; i += blockDim.x) Lf[i] = A32[i];
+        for (int i = tid; i < NA * lda; i += blockDim.x) X[i] = A32[i];
         __syncthreads();
       }
       if (tid < N) {
         const double v = dg[tid] + Fp[tid];
         M[tid * lda + tid] = v;
-        if (!use64) Lf[tid * lda + tid] = (float)v;
+        if (!use64) X[tid * lda + tid] = (float)v;
       }
       if (tid == N) rhs[N] = 0.0;
       if (tid >= 64 && tid < 96) {   // max(1, ||U||_inf), for the solve's goal
@@ -2539,20 +2438,8 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
       }
       __syncthreads();
       if (!use64) {
-        if (tid < 32) {
-          const bool okw = (dim == 2 && NA == 50)   ? ldlt_band_warp_ns<float, 2, 50, 8>(Lf, NA, lda, rd, 8, 1, false, 0.0, nullptr)
-                           : (dim == 2 && NA == 10) ? ldlt_band_warp_ns<float, 1, 10, 4>(Lf, NA, lda, rd, 4, 1, false, 0.0, nullptr)
-                           : (dim == 3 && NA == 28) ? ldlt_band_warp_ns<float, 4, 28, 13>(Lf, NA, lda, rd, 13, 1, false, 0.0, nullptr)
-                                                    : ldlt_band_warp<float>(Lf, NA, lda, rd, band, 1, false, 0.0, nullptr);
-          if (tid == 0 && !okw) use64 = 1;
-        }
-        __syncthreads();
-        if (!use64 && tid < NA) {
-          if (dim == 2)
-            band_inverse_dispatch<2>(Lf, rd, NA, lda, NA == 50 ? 8 : NA == 10 ? 4 : band, tid, X);
-          else
-            band_inverse_dispatch<3>(Lf, rd, NA, lda, NA == 28 ? 13 : band, tid, X);
-        }
+        const bool okw = sweep_inverse<256>(X, NA, lda, X, false, 0.f, nullptr);
+        if (tid == 0 && !okw) use64 = 1;
         __syncthreads();
       }
       if (!use64) {
@@ -2604,23 +2491,24 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
       if (done) break;
       continue;
     }
-    // the lower band of the Jacobian A_1 + diag(w f'(U)) (the factor of the previous
-    // iteration overwrote it)
+    // the lower triangle of the Jacobian A_1 + diag(w f'(U)), where the previous inverse was
+    for (int idx = threadIdx.x; idx < N * ld; idx += blockDim.x) {
+      const int p = idx / ld, q = idx - p * ld;
+      if (p - q > band) L[idx] = T(0);
+    }
     for (int idx = threadIdx.x; idx < N * (band + 1); idx += blockDim.x) {
       const int p = idx / (band + 1), q = p - idx % (band + 1);
       if (q < 0) continue;
       const double v = level1_entry(p, q, m, dim, sigma, vc) + (p == q ? Fp[p] : 0.0);
       L[p * ld + q] = (T)v;
     }
+    if (threadIdx.x < N) work[threadIdx.x] = (T)rhs[threadIdx.x];
     __syncthreads();
-    if (threadIdx.x < 32) {
-      // the benchmark shapes (2D 1/H = 8, 3D 1/H = 4) with their size and band fixed at compile time
-      const bool okw = (dim == 2 && N == 49 && band == 7)
-                           ? ldlt_band_warp_ns<T, 1, 49, 7>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
-                       : (dim == 3 && N == 27 && band == 9)
-                           ? ldlt_band_warp_ns<T, 2, 27, 9>(L, N, ld, invd, band, 0, false, 0.0, nullptr)
-                           : ldlt_band_warp<T>(L, N, ld, invd, band, 0, false, 0.0, nullptr);
-      ldlt_solve_band_warp<T>(L, N, ld, invd, band, 0, rhs);
+    if constexpr (!kRefine) {
+      const bool okw = sweep_inverse<256>(L, N, ld, L, false, 0.f, nullptr);
+      small_matvec<256>(L, N, ld, work, step);
+      __syncthreads();
+      if (threadIdx.x < N) rhs[threadIdx.x] = (double)step[threadIdx.x];
       if (threadIdx.x == 0) ok_sh = okw ? 1 : 0;
     }
     __syncthreads();
