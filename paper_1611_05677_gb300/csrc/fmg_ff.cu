@@ -403,16 +403,20 @@ namespace {
 // is fine node (i, j[, l]) n_L / n_k), zero on its boundary, stored as FP64 where g[k] is given and
 // as float-float where gf[k] is.  src may be the fine level's own array (then only its boundary
 // ring is written).  Bound by HBM: the fine level reads 8 bytes and writes 8 per node and array.
-// Blocks boff[k] .. boff[k+1]-1 take level k, a block a row of nodes at a time (no index division
-// per node).  No block reads what another writes.
+// Blocks boff[k] .. boff[k+1]-1 take level k, kRhsChunk consecutive nodes each, eight loads per thread
+// in flight.  A row of nodes per turn instead left one load per thread in flight where rows are
+// short (257^3: 137 us, this 68; 2049^2: 28.6, this 22.6; ncu, cold caches).  No block reads
+// what another writes.
 struct RhsLevels {
   const double* src;
   double* g[kMaxLevels];
   double* gf[kMaxLevels];
   int n[kMaxLevels];
   unsigned boff[kMaxLevels + 1];
-  int nlev, dim, rows;   // rows per block
+  unsigned magic[kMaxLevels];   // ceil(2^32 / (n + 1)): exact quotients of rows and of nodes within a chunk
+  int nlev, dim;
 };
+constexpr int kRhsChunk = 2048;
 
 __global__ void __launch_bounds__(256) k_rhs_levels(const __grid_constant__ RhsLevels R) {
   pdl_start();
@@ -426,27 +430,29 @@ __global__ void __launch_bounds__(256) k_rhs_levels(const __grid_constant__ RhsL
   double* g = R.g[k];
   double* gf = R.gf[k];
   const bool self = g == R.src;
-  const int r0 = (int)(blockIdx.x - R.boff[k]) * R.rows;
-  for (int r = r0; r < min(r0 + R.rows, nrows); ++r) {
-    const int l = R.dim == 3 ? r / np : 0, j = r - l * np;
-    const bool edge = j == 0 || j == n || (R.dim == 3 && (l == 0 || l == n));
-    const double* in = R.src + ((long long)l * st * fp + (long long)j * st) * fp;
-    const long long o = (long long)r * np;
-    for (int i0 = threadIdx.x; i0 < np; i0 += 4 * 256) {
-      double v[4];
+  const unsigned magic = R.magic[k];
+  const unsigned n0 = (blockIdx.x - R.boff[k]) * (unsigned)kRhsChunk;   // at most 32769^2 or 1025^3 nodes
+  const unsigned rb = n0 / (unsigned)np, ib = n0 - rb * (unsigned)np;
+  double v[kRhsChunk / 256];
+  unsigned at[kRhsChunk / 256];
+  unsigned ring = 0u;   // bit q: a boundary node, bit 16 + q: past the level
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = i0 + q * 256;
-        v[q] = i > 0 && i < n && !edge ? in[(long long)i * st] : 0.0;
-      }
+  for (int q = 0; q < kRhsChunk / 256; ++q) {
+    const unsigned e = ib + threadIdx.x + q * 256u;
+    const unsigned dr = __umulhi(e, magic), r = rb + dr;
+    const int i = (int)(e - dr * (unsigned)np);
+    const int l = R.dim == 3 ? (int)__umulhi(r, magic) : 0, j = (int)r - l * np;
+    at[q] = n0 + threadIdx.x + q * 256u;
+    const bool here = (int)r < nrows;
+    const bool edge = i == 0 || i == n || j == 0 || j == n || (R.dim == 3 && (l == 0 || l == n));
+    ring |= (edge ? 1u : 0u) << q | (here ? 0u : 1u) << (16 + q);
+    v[q] = here && !edge ? R.src[(((long long)l * st * fp + (long long)j * st) * fp) + (long long)i * st] : 0.0;
+  }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = i0 + q * 256;
-        if (i >= np) break;
-        if (g && (!self || edge || i == 0 || i == n)) g[o + i] = v[q];
-        if (gf) ff_store(gf + o + i, ff_from_double_int(v[q]));
-      }
-    }
+  for (int q = 0; q < kRhsChunk / 256; ++q) {
+    if ((ring >> (16 + q)) & 1u) break;
+    if (g && (!self || ((ring >> q) & 1u))) g[at[q]] = v[q];
+    if (gf) ff_store(gf + at[q], ff_from_double_int(v[q]));
   }
 }
 
@@ -457,7 +463,6 @@ cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, const doub
   if (nlev < 1 || nlev > kMaxLevels) return cudaErrorInvalidValue;
   RhsLevels R = {};
   R.src = src;
-  R.rows = dim == 2 ? 1 : 4;
   long long off = 0;
   for (int k = 0; k < nlev; ++k) {
     // with float-float copies only level 1 (the exact semilinear solve) reads the FP64 ones, and the
@@ -466,7 +471,8 @@ cudaError_t launch_rhs_levels(int dim, int nlev, const LevelGeo* geo, const doub
     R.gf[k] = ff ? gf[k] : nullptr;
     R.n[k] = geo[k].n;
     R.boff[k] = (unsigned)off;
-    off += (ipow(geo[k].np, dim - 1) + R.rows - 1) / R.rows;
+    R.magic[k] = (unsigned)(((1ull << 32) + geo[k].np - 1) / geo[k].np);
+    off += (geo[k].nodes + kRhsChunk - 1) / kRhsChunk;
   }
   if (off < 1 || off > 0x7fffffffll) return cudaErrorInvalidValue;
   R.boff[nlev] = (unsigned)off;
