@@ -300,11 +300,16 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
   // makes at least `need` halo rows of array `off` current.  A deep halo is overwritten only when
   // no CTA reads it any more (the CTAs' passes are not in step between exchanges); with a halo of
   // one row every pass is followed by an exchange, and what a neighbour may still read of it is
-  // the other colour, whose values the store repeats, or the other Chebyshev buffer.
+  // the other colour, whose values the store repeats, or the other Chebyshev buffer.  Where that
+  // does not hold -- after the prolongation, which adds to the halo rows in place -- the CTAs have
+  // arrived at a barrier behind the pass in question (`behind`), and the store waits for it.
+  bool behind = false;
   auto ensure = [&](int off, int need) {
     if (CS == 1 || valid >= need) return;
     before_remote();
     if (W > 1) cluster.sync();
+    if (behind) cluster.barrier_wait();
+    behind = false;
     push_rows(off);
     cluster.sync();
     valid = W;
@@ -576,6 +581,11 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
       for_colour(L, ra, rb, 0, prol);
     else
       for_inner(L, ra, rb, prol);
+    // (the second half sweep's exchange is the first to store into the rows just corrected)
+    if (!CHEB && W == 1 && CS > 1 && j == jtop && A.nu_post >= 1) {
+      cluster.barrier_arrive();
+      behind = true;
+    }
     __syncthreads();
     if constexpr (CHEB) {
       cheb_steps(L, j, A.nu_post, 0);
