@@ -301,8 +301,9 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
   // no CTA reads it any more (the CTAs' passes are not in step between exchanges); with a halo of
   // one row every pass is followed by an exchange, and what a neighbour may still read of it is
   // the other colour, whose values the store repeats, or the other Chebyshev buffer.  Where that
-  // does not hold -- after the prolongation, which adds to the halo rows in place -- the CTAs have
-  // arrived at a barrier behind the pass in question (`behind`), and the store waits for it.
+  // does not hold -- after the prolongation, which adds to the halo rows in place, and after an odd
+  // number of Chebyshev steps, whose result is moved to the buffer that the last of them read -- the
+  // CTAs have arrived at a barrier behind the pass in question (`behind`), and the store waits for it.
   bool behind = false;
   auto ensure = [&](int off, int need) {
     if (CS == 1 || valid >= need) return;
@@ -350,8 +351,9 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
     });
     __syncthreads();
   };
-  // Chebyshev steps k0..steps-1, alternating between u and ua, ending in u
-  auto cheb_steps = [&](const CLevel& L, int j, int steps, int k0) {
+  // Chebyshev steps k0..steps-1, alternating between u and ua, ending in u.  exchanged: the top level's
+  // u goes to the neighbours next.
+  auto cheb_steps = [&](const CLevel& L, int j, int steps, int k0, bool exchanged) {
     const T inv2d = T(1) / T(2 * D);
     int us = k0 ? cheb_start_off(L) : L.u;
     int uo = us == L.u ? L.ua : L.u;
@@ -382,6 +384,11 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
       uo = t2;
     }
     if (us != L.u) {
+      if (W == 1 && CS > 1 && j == jtop && exchanged) {
+        before_remote();
+        cluster.barrier_arrive();
+        behind = true;
+      }
       // (current rows only: a neighbour may already store into the others)
       for_inner(L, row_a(j, valid), row_b(j, valid), [&](int c, int, int, int) { sm[L.u + c] = sm[us + c]; });
       __syncthreads();
@@ -394,7 +401,7 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
     const CLevel C = LV[j - 2];
     if constexpr (CHEB) {
       const bool started = A.nu_pre >= 1 && (j < jtop || A.zero_start);
-      cheb_steps(L, j, A.nu_pre, started ? 1 : 0);
+      cheb_steps(L, j, A.nu_pre, started ? 1 : 0, true);
     } else {
       for (int it = 0; it < A.nu_pre; ++it) {
         half_sweep(L, j, 0);
@@ -588,7 +595,7 @@ __device__ __forceinline__ void k_coarse_cluster_body(const CoarseArgs<T>& A) {
     }
     __syncthreads();
     if constexpr (CHEB) {
-      cheb_steps(L, j, A.nu_post, 0);
+      cheb_steps(L, j, A.nu_post, 0, false);
     } else {
       for (int it = 0; it < A.nu_post; ++it) {
         half_sweep(L, j, 1);

@@ -2,7 +2,9 @@
 the exchanges of the planes between CTAs that are not in step.
 
 After the prolongation a CTA has added the correction to its halo planes in place; a neighbour's
-plane that arrived before that would be corrected twice.  Every run has the same arithmetic in the
+plane that arrived before that would be corrected twice.  After an odd number of Chebyshev steps
+from a given iterate the result is moved to the buffer that the last step read; a plane of it that
+arrived in a neighbour still in that step would take the old one's place.  Every run has the same arithmetic in the
 same order, so many runs from one start give one set of bits, and those are the oracle's cycle to
 1e-12 (a few hundred FP64 operations' rounding relative to the iterate; 1e-4 for the FP32 cycles)."""
 import numpy as np
@@ -68,3 +70,9 @@ def test_red_black_after_prolongation(fmg, H, r, nu, precision):
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_red_black_after_prolongation_with_coefficient(fmg, precision):
     repeated_cycles(fmg, 4, 2, precision, "rbgs", (1, 2), coef=W.cell_coefficient(3, 4))
+
+
+@pytest.mark.parametrize("nu", [(1, 1), (3, 0), (5, 2), (2, 3)])
+@pytest.mark.parametrize("H,r", [(4, 2), (2, 3)])
+def test_odd_chebyshev_steps(fmg, H, r, nu):
+    repeated_cycles(fmg, H, r, "fp64", "chebyshev", nu)
