@@ -153,9 +153,10 @@ fmg_status fmg_workspace_bytes(const fmg_params* p, size_t* bytes);
  *                library copies it; the caller keeps ownership of its buffer.
  *   stream       cudaStream_t (as void*) all work of this context is ordered on; NULL = the
  *                legacy default stream.
- *   workspace    device memory of at least fmg_workspace_bytes bytes that the context uses
- *                for all its arrays, owned by the caller and kept alive until fmg_destroy; or
- *                NULL, in which case the library allocates (cudaMalloc) and frees it itself.
+ *   workspace    device memory of at least fmg_workspace_bytes bytes, at any address, that the
+ *                context uses for all its arrays, owned by the caller and kept alive until
+ *                fmg_destroy; or NULL, in which case the library allocates (cudaMalloc) and
+ *                frees it itself.
  * On success *out receives the context.  Returns FMG_ERR_OOM when the device does not have
  * the memory (checked with cudaMemGetInfo before allocating). */
 fmg_status fmg_create(const fmg_params* p, const double* g_fine, int g_on_device, void* stream,

@@ -128,7 +128,13 @@ const char* validate(const fmg_params* p) {
   return nullptr;
 }
 
-size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
+constexpr size_t kAlign = 256;
+size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
+
+// The arrays of a context start on kAlign bytes (the widest access is 16), wherever the caller's
+// workspace starts: fmg_workspace_bytes leaves room to move the first one up.
+constexpr size_t kWorkspaceSlack = kAlign - 1;
+char* workspace_start(void* p) { return reinterpret_cast<char*>(align_up(reinterpret_cast<size_t>(p))); }
 
 // Lays out (or only sizes, when base == nullptr) every device array of a context.
 size_t layout(fmg_ctx* c, const fmg_params* p, char* base) {
@@ -1005,7 +1011,7 @@ void fmg_default_params(fmg_params* p) {
 fmg_status fmg_workspace_bytes(const fmg_params* p, size_t* bytes) {
   if (const char* why = validate(p)) return fail(nullptr, FMG_ERR_INVALID, why);
   if (!bytes) return fail(nullptr, FMG_ERR_INVALID, "bytes is NULL");
-  *bytes = layout(nullptr, p, nullptr);
+  *bytes = layout(nullptr, p, nullptr) + kWorkspaceSlack;
   return FMG_OK;
 }
 
@@ -1034,11 +1040,11 @@ fmg_status fmg_create(const fmg_params* p, const double* g_fine, int g_on_device
   }
   const size_t need = layout(c, p, nullptr);
   if (workspace) {
-    if (workspace_bytes < need) {
+    if (workspace_bytes < need + kWorkspaceSlack) {
       delete c;
       return fail(nullptr, FMG_ERR_INVALID, "workspace smaller than fmg_workspace_bytes");
     }
-    c->arena = workspace;
+    c->arena = workspace_start(workspace);
     c->own_arena = false;
   } else {
     size_t free_b = 0, total_b = 0;
