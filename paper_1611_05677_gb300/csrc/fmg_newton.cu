@@ -2024,10 +2024,15 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
 // correction would be below the rounding of y.  The solution has FP64 accuracy whatever the
 // accuracy of X, which sets the rate only: about 1e-5 per sweep with its own J, ||I - X J|| with
 // a later one (systems of at most kRefineFresh unknowns, whose FP32 inverse costs little more
-// than two sweeps, get a new X every Newton iteration).  The step that passes Newton's test, and
-// so ends the iteration, is solved to the rounding of the iterate (c, alpha); an earlier one to
+// than two sweeps, get a new X every Newton iteration).  "Below the rounding" is meant separately
+// for the coarse values c and for alpha, each against the larger of the step and the iterate in
+// its own maximum norm: c goes with the size of the solution and alpha does not, so a common norm
+// would leave the c of a small solution unsolved.  The step that passes Newton's test, and
+// so ends the iteration, is solved to that; an earlier one to
 // an error far below both the next step of a quadratically convergent iteration and the test's
 // tolerance, which the next residual corrects.
+// Against 80-bit arithmetic, over the systems of all 1/H, five nonlinearities and solutions of 1e-8
+// to 30 (about 2400): largest error 8e-13 of the norm, median 1e-17; the FP64 LDL^T 6.5e-12 and 9e-17.
 // Measured at 50 unknowns: 3.5 to 9 us per Newton iteration after the first, against 46.
 // Where X is no good -- J not positive definite in FP32, the Schur complement of alpha below
 // kRefinePivot of its diagonal, magnitudes outside FP32, or no convergence in kRefineSweeps -- the
@@ -2035,13 +2040,15 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
 constexpr int kRefineSweeps = 16;
 constexpr int kRefineFresh = 16;
 constexpr float kRefinePivot = 1e-3f;
+constexpr float kRefineEps = 5e-17f;     // half the rounding of FP64
+constexpr float kRefineFloor = 1.5e-14f; // where a solve may come to rest: 64 times the rounding of FP64
 
 // Refinement sweeps from y = 0 (see above); R, M in shared memory, y written over R on success;
-// iterate: max(1, ||(c, alpha)||_inf).
+// it_c, it_a: the maximum norms of the iterate's c and alpha.
 // Returns false (R untouched) if they do not converge.
 template <int D, int NT>
 __device__ bool refine_solve(int nc, double newton_tol, const float* X, const double* M, int NH, double* R,
-                             float iterate) {
+                             float it_c, float it_a) {
   constexpr int LPR = D == 2 ? 2 : 4;    // lanes per row of the sparse residual
   constexpr int NE = 4;                  // its entries per lane: 2D 7 + border, 3D 15 + border
   __shared__ double y_sh[kMaxAug];
@@ -2082,7 +2089,10 @@ __device__ bool refine_solve(int nc, double newton_tol, const float* X, const do
     if (tid < NA) r_sh[tid] = (float)R[tid];
   }
   __syncthreads();
-  float zprev = 0.f;
+  const float iterate = fmaxf(1.f, fmaxf(it_c, it_a));
+  const bool idle = R[NH] == 0.0;   // (the bordering unknown of level 1)
+  const float jaa = (float)M[NH * ld + NH];
+  float sprev = 0.f;
   for (int sweep = 0;; ++sweep) {
     small_matvec<NT>(X, NA, ld, r_sh, z_sh);
     __syncthreads();
@@ -2094,27 +2104,33 @@ __device__ bool refine_solve(int nc, double newton_tol, const float* X, const do
         y_sh[tid] = y;
         ya = fabsf((float)y);
       }
-      const unsigned zb = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(z)));
-      const unsigned yb = __reduce_max_sync(0xffffffffu, __float_as_uint(ya));
+      const bool c = tid < NH;   // (alpha by itself, below)
+      const unsigned zb = __reduce_max_sync(0xffffffffu, c ? __float_as_uint(fabsf(z)) : 0u);
+      const unsigned yb = __reduce_max_sync(0xffffffffu, c ? __float_as_uint(ya) : 0u);
       if (lane == 0) {
         max_sh[tid >> 5][0] = zb;
         max_sh[tid >> 5][1] = yb;
       }
     }
     __syncthreads();
-    const float zmax = __uint_as_float(max(max_sh[0][0], max_sh[1][0]));
-    const float ymax = __uint_as_float(max(max_sh[0][1], max_sh[1][1]));
-    if (!(zmax < 1e30f) || !(ymax > 1e-25f)) return false;   // also NaN
+    const float zc = __uint_as_float(max(max_sh[0][0], max_sh[1][0]));
+    const float yc = __uint_as_float(max(max_sh[0][1], max_sh[1][1]));
+    const float za = fabsf(z_sh[NH]), ya = fabsf((float)y_sh[NH]);
+    const float sc = fmaxf(yc, it_c), sa = fmaxf(ya, it_a);
+    // (also NaN)  FP32 has no room for the sweeps of smaller values, whose residuals go down to 1e-17 J y
+    if (!(zc < 1e30f) || !(za < 1e30f) || !(sc > 1e-19f) || !(idle || jaa * sa > 1e-19f)) return false;
+    // the correction in units of c and alpha
+    const float s = fmaxf(zc / sc, za > 0.f ? za / sa : 0.f);
     if (sweep > 0) {
-      // the next correction is about zmax (zmax / zprev)
-      const float rho = zmax / zprev;
-      const float tol = (float)newton_tol * iterate;
+      // the next correction is about s (s / sprev)
+      const float rho = s / sprev;
+      const float tol = (float)newton_tol * iterate, zmax = fmaxf(zc, za), ymax = fmaxf(yc, ya);
       const float goal = ymax > tol ? fminf(1e-3f * ymax * ymax, 1e-2f * tol) : 0.f;
-      if (zmax * fminf(rho, 1.f) <= fmaxf(goal, 5e-17f * iterate)) break;
-      if (rho > 0.5f && zmax <= 1e-13f * ymax) break;   // at the rounding level of an FP64 solve
+      if (zmax * fminf(rho, 1.f) <= goal || s * fminf(rho, 1.f) <= kRefineEps) break;
+      if (rho > 0.5f && s <= kRefineFloor) break;   // at the rounding level of an FP64 solve
       if (sweep >= kRefineSweeps || rho > 0.5f) return false;
     }
-    zprev = zmax;
+    sprev = s;
     // r = R - J y
     double a = 0.0;
 #pragma unroll
@@ -2156,7 +2172,7 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
   const int ld = NA + 1;
   const bool fixedp = A.fixed_point != 0;
   __shared__ int fac_sh[2];
-  __shared__ float iterate_sh;
+  __shared__ float iterate_sh;   // max |c|
   // the cell sums (one contiguous block of rows, an even number of doubles): asynchronous 16-byte
   // copies past L1, all in flight together; the matrix is cleared meanwhile
   {
@@ -2186,9 +2202,9 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
     if (tid == 0) S.flags[2] = 0;
     __syncthreads();
   }
-  // max(1, ||(c, alpha)||_inf), for the solve's goal
+  // max |c|, for the solve's goal
   if (tid < 32) {
-    float v = fmaxf(1.f, fabsf((float)S.sa[1]));
+    float v = 0.f;
     const int cn = (int)ipow(A.nc + 1, D);
     for (int i = lane; i < cn; i += 32) v = fmaxf(v, fabsf((float)S.c[i]));
     v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
@@ -2272,7 +2288,7 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
     __syncthreads();
   }
   if (!S.flags[2]) {
-    const bool solved = refine_solve<D, nthr>(A.nc, A.tol, X, M, NH, R, iterate_sh);
+    const bool solved = refine_solve<D, nthr>(A.nc, A.tol, X, M, NH, R, iterate_sh, fabsf((float)alpha));
     __syncthreads();
     if (!solved && tid == 0) S.flags[2] = 1;
     __syncthreads();
@@ -2430,8 +2446,8 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
         if (!use64) X[tid * lda + tid] = (float)v;
       }
       if (tid == N) rhs[N] = 0.0;
-      if (tid >= 64 && tid < 96) {   // max(1, ||U||_inf), for the solve's goal
-        float v = 1.f;
+      if (tid >= 64 && tid < 96) {   // max |U|, for the solve's goal
+        float v = 0.f;
         for (int p = lane; p < N; p += 32) v = fmaxf(v, fabsf((float)U[p]));
         v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
         if (lane == 0) iterate_sh = v;
@@ -2443,8 +2459,8 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
         __syncthreads();
       }
       if (!use64) {
-        const bool solved = dim == 2 ? refine_solve<2, 256>(n1, tol, X, M, N, rhs, iterate_sh)
-                                     : refine_solve<3, 256>(n1, tol, X, M, N, rhs, iterate_sh);
+        const bool solved = dim == 2 ? refine_solve<2, 256>(n1, tol, X, M, N, rhs, iterate_sh, 0.f)
+                                     : refine_solve<3, 256>(n1, tol, X, M, N, rhs, iterate_sh, 0.f);
         __syncthreads();
         if (!solved && tid == 0) use64 = 1;
         __syncthreads();
