@@ -2027,10 +2027,9 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
 // than two sweeps, get a new X every Newton iteration).  "Below the rounding" is meant separately
 // for the coarse values c and for alpha, each against the larger of the step and the iterate in
 // its own maximum norm: c goes with the size of the solution and alpha does not, so a common norm
-// would leave the c of a small solution unsolved.  The step that passes Newton's test, and
-// so ends the iteration, is solved to that; an earlier one to
-// an error far below both the next step of a quadratically convergent iteration and the test's
-// tolerance, which the next residual corrects.
+// would leave the c of a small solution unsolved.  Every step is solved to that, the ones before the
+// last too: the iteration may end at any of them (its cap), and the fixed-point iteration does not
+// make up for an error in the next step as Newton's does.
 // Against 80-bit arithmetic, over the systems of all 1/H, five nonlinearities and solutions of 1e-8
 // to 30 (about 2400): largest error 8e-13 of the norm, median 1e-17; the FP64 LDL^T 6.5e-12 and 9e-17.
 // Measured at 50 unknowns: 3.5 to 9 us per Newton iteration after the first, against 46.
@@ -2047,8 +2046,7 @@ constexpr float kRefineFloor = 1.5e-14f; // where a solve may come to rest: 64 t
 // it_c, it_a: the maximum norms of the iterate's c and alpha.
 // Returns false (R untouched) if they do not converge.
 template <int D, int NT>
-__device__ bool refine_solve(int nc, double newton_tol, const float* X, const double* M, int NH, double* R,
-                             float it_c, float it_a) {
+__device__ bool refine_solve(int nc, const float* X, const double* M, int NH, double* R, float it_c, float it_a) {
   constexpr int LPR = D == 2 ? 2 : 4;    // lanes per row of the sparse residual
   constexpr int NE = 4;                  // its entries per lane: 2D 7 + border, 3D 15 + border
   __shared__ double y_sh[kMaxAug];
@@ -2089,7 +2087,6 @@ __device__ bool refine_solve(int nc, double newton_tol, const float* X, const do
     if (tid < NA) r_sh[tid] = (float)R[tid];
   }
   __syncthreads();
-  const float iterate = fmaxf(1.f, fmaxf(it_c, it_a));
   const bool idle = R[NH] == 0.0;   // (the bordering unknown of level 1)
   const float jaa = (float)M[NH * ld + NH];
   float sprev = 0.f;
@@ -2124,9 +2121,7 @@ __device__ bool refine_solve(int nc, double newton_tol, const float* X, const do
     if (sweep > 0) {
       // the next correction is about s (s / sprev)
       const float rho = s / sprev;
-      const float tol = (float)newton_tol * iterate, zmax = fmaxf(zc, za), ymax = fmaxf(yc, ya);
-      const float goal = ymax > tol ? fminf(1e-3f * ymax * ymax, 1e-2f * tol) : 0.f;
-      if (zmax * fminf(rho, 1.f) <= goal || s * fminf(rho, 1.f) <= kRefineEps) break;
+      if (s * fminf(rho, 1.f) <= kRefineEps) break;
       if (rho > 0.5f && s <= kRefineFloor) break;   // at the rounding level of an FP64 solve
       if (sweep >= kRefineSweeps || rho > 0.5f) return false;
     }
@@ -2288,7 +2283,7 @@ __device__ __noinline__ void newton_step_fp64(const AugArgs& A, const double* __
     __syncthreads();
   }
   if (!S.flags[2]) {
-    const bool solved = refine_solve<D, nthr>(A.nc, A.tol, X, M, NH, R, iterate_sh, fabsf((float)alpha));
+    const bool solved = refine_solve<D, nthr>(A.nc, X, M, NH, R, iterate_sh, fabsf((float)alpha));
     __syncthreads();
     if (!solved && tid == 0) S.flags[2] = 1;
     __syncthreads();
@@ -2459,8 +2454,8 @@ __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const doub
         __syncthreads();
       }
       if (!use64) {
-        const bool solved = dim == 2 ? refine_solve<2, 256>(n1, tol, X, M, N, rhs, iterate_sh, 0.f)
-                                     : refine_solve<3, 256>(n1, tol, X, M, N, rhs, iterate_sh, 0.f);
+        const bool solved = dim == 2 ? refine_solve<2, 256>(n1, X, M, N, rhs, iterate_sh, 0.f)
+                                     : refine_solve<3, 256>(n1, X, M, N, rhs, iterate_sh, 0.f);
         __syncthreads();
         if (!solved && tid == 0) use64 = 1;
         __syncthreads();

@@ -86,3 +86,50 @@ def test_small_solution(fmg, dim, H, r, amp, f):
     fmg.fmg_op_correction_step(s.ctx, r + 1, u)
     s.close()
     assert np.max(np.abs(u.cpu().numpy() - want)) <= 1e-10 * np.max(np.abs(want))
+
+
+def iterations(hier, k, ut, G, f, a, count, fixed_point):
+    """`count` iterations of (3.6) from (c, alpha) = (0, 1), in FP64 with a dense factorization."""
+    lev = hier.level(k)
+    B = np.hstack([hier.P_H[k - 1].toarray(), ut[:, None]])
+    K = B.T @ (lev.A @ B)
+    y = np.zeros(B.shape[1])
+    y[-1] = 1.0
+    for _ in range(count):
+        U = B @ y
+        R = K @ y + B.T @ (lev.w * O.f_val(f, a, U) - G)
+        J = K if fixed_point else K + B.T @ ((lev.w * O.f_der(f, a, U))[:, None] * B)
+        d = np.linalg.solve(J, R)
+        y = y - d
+        if np.max(np.abs(d)) <= 1e-6 * max(1.0, np.max(np.abs(y))):
+            break
+    return B @ y
+
+
+@pytest.mark.parametrize("nonlinear", ["newton", "fixed_point"])
+@pytest.mark.parametrize("count", [1, 2, 3])
+@pytest.mark.parametrize("dim,H,r", [(2, 4, 3), (2, 8, 3), (3, 4, 2)])
+def test_iteration_cut_short(fmg, dim, H, r, count, nonlinear):
+    """The iterate after any number of steps is that of steps solved in FP64, whose dense solves have
+    errors of up to 3e-13 on these systems: 1e-12 of the solution."""
+    prob = problem(dim, H, r, "cubic", 2.0)
+    g = prob.g_nodal()
+    hier = O.build_hierarchy(dim, H, r)
+    lev = hier.level(r + 1)
+    G = O.load_vector(lev, g)
+    rng = np.random.default_rng(6)
+    U = O.from_nodal(lev, prob.u_star()) * (1.0 + 0.5 * rng.standard_normal(lev.A.shape[0]))
+    b = G - lev.w * O.f_val(prob.f, prob.a, U)
+    ut = U.copy()
+    for _ in range(2):
+        ut = O.vcycle(hier, r + 1, b, ut, 2, 2)
+    want = O.to_nodal(lev, iterations(hier, r + 1, ut, G, prob.f, prob.a, count, nonlinear == "fixed_point"))
+    s = fmg.Solver(fmg.make_params(prob, precision="fp64", nonlinear=nonlinear, newton_maxit=count), g)
+    u = torch.tensor(O.to_nodal(lev, U), device="cuda")
+    try:
+        fmg.fmg_op_correction_step(s.ctx, r + 1, u)
+    except fmg.FMGError:
+        pass   # (the cap is reported)
+    got = u.cpu().numpy()
+    s.close()
+    assert np.max(np.abs(got - want)) <= 1e-12 * np.max(np.abs(want))
