@@ -26,13 +26,14 @@
 // segment's moments sum X, sum X z, sum X z^2.  The thread accumulates those moments in
 // registers (FP64 for the residual; FP32 or FP64 for the Jacobian) and converts them to the
 // cell's vertex channels once per segment.  The lanes of a warp walk neighbouring columns, whose
-// segments end at different z, so all walk the same z range (a chunk) with running moments, and a
-// lane keeps a copy of them where its segment ends: the segments' moments are differences of the
-// copies.  (A loop per segment runs as long as the longest lane's in each: up to twice the chunk in
-// 2D, three times in 3D.  Measured, loop per segment against this: mixed first pass at 257^3 719
-// and 496 us, at 2049^2 75 and 61; FP64 first pass at 129^3 380 and 239 us.)  The residual sums carry f(U) - g, so G_H and gamma
-// are never formed apart; the first pass also gathers t and s
-// (at (c, alpha) = (0, 1), U = u~), so no separate precompute pass is needed.
+// segments end at different z, so all walk the same z range (a chunk), and where a lane's segment
+// ends it puts the moments aside and begins the next segment's from zero.  (A loop per segment
+// runs as long as the longest lane's in each: up to twice the chunk in 2D, three times in 3D.
+// Measured, loop per segment against this: mixed first pass at 257^3 719 and 496 us, at 2049^2 75
+// and 61; FP64 first pass at 129^3 380 and 239 us.  Moments taken as differences of running sums
+// over the chunk cost the same but carry the chunk's rounding: up to twice the error in FP32.)
+// The residual sums carry f(U) - g, so G_H and gamma are never formed apart; the first pass also
+// gathers t and s (at (c, alpha) = (0, 1), U = u~), so no separate precompute pass is needed.
 //
 // Reductions are deterministic: per-thread channel rows in shared memory, fixed-order block
 // sums, fixed-order sums over blocks and cells.
@@ -656,6 +657,11 @@ __device__ __forceinline__ void delta_f(int kind, double a, ff ut, float utf, fl
 struct FirstMoments {
   ff q0, q1, sa, t0, t1, ss;
   float d0, d1, d2, e0, e1, js;
+  // the sums that belong to a segment start again (sa, ss and js are the whole run's)
+  __device__ __forceinline__ void restart() {
+    q0 = q1 = t0 = t1 = ff{0.f, 0.f};
+    d0 = d1 = d2 = e0 = e1 = 0.f;
+  }
 };
 
 // One node of the mixed first pass: u~ = U and g = G at the node, its axis neighbours um[ax]
@@ -749,7 +755,10 @@ __device__ __forceinline__ void first_batch(const AugArgs& A, FirstMoments& m, F
     first_node<D, CUBIC, VC>(A, m, uz[q + 1], gv[q], nm, nq, z + q, x, y, zc);
 #pragma unroll
     for (int t = 0; t < D - 1; ++t)
-      if (z + q == zb[t]) snap[t] = m;
+      if (z + q == zb[t]) {
+        snap[t] = m;
+        m.restart();
+      }
   }
 }
 
@@ -757,7 +766,7 @@ __device__ __forceinline__ void first_batch(const AugArgs& A, FirstMoments& m, F
 // of B nodes (B smaller in 3D, whose nodes have two more in-plane neighbours to hold).  x, y:
 // the column's fine in-plane coordinates; zc: the fine z of local z = 0 (the coefficient's
 // edge weights need the node's position); zb: where the column's segments end (snap: the moments
-// up to there).
+// of the segment that ends there).
 template <int D, bool CUBIC, bool VC>
 __device__ __forceinline__ void first_pass_run(const AugArgs& A, long long off, int z0, int z1, long long zstride,
                                                FirstMoments& m, FirstMoments* snap, const int* zb, int x, int y,
@@ -793,9 +802,9 @@ __device__ __forceinline__ Deal64 deal64(const AugArgs& A) {
   return d;
 }
 
-// The FP64 path's running moments of a column chunk, summed over the nodes in order of z with the
-// weights m = number of nodes from z to the last one summed: sum f, sum f m and sum f m (m + 1) / 2
-// are prefix sums, one FP64 add each per node.
+// The FP64 path's moments of a segment, summed over the nodes in order of z with the weights
+// m = number of nodes from z to the last one summed: sum f, sum f m and sum f m (m + 1) / 2 are
+// prefix sums, one FP64 add each per node.
 struct Moments64 {
   double q0, q1, d0, d1, d2, e0, e1, t0, t1;
 };
@@ -810,7 +819,7 @@ struct Totals64 {
 // P c (pc at z0) advances along z by one add of the segment's slope.  2D: 20 operations in the first
 // pass and 15 in the others, against 26 and 20 for the plain form (2049^2: first pass 303 -> 193
 // us, others 217 -> 153, the running moments included).  Values are loaded B nodes at a time into registers, one memory latency
-// per batch.  zb: where the column's segments end (snap: the moments up to there).
+// per batch.  zb: where the column's segments end (snap: the moments of the segment that ends there).
 template <int D, bool CUBIC, bool FIRST, bool VC>
 __device__ __forceinline__ void run64(const AugArgs& A, Moments64& m, Totals64& tot, Moments64* snap, const int* zb,
                                       long long off, int z0, int z1, long long zstride, long long np, double alpha,
@@ -897,7 +906,10 @@ __device__ __forceinline__ void run64(const AugArgs& A, Moments64& m, Totals64& 
       }
 #pragma unroll
       for (int t = 0; t < D - 1; ++t)
-        if (z + q == zb[t]) snap[t] = m;
+        if (z + q == zb[t]) {
+          snap[t] = m;
+          m = Moments64{};
+        }
     }
   }
 }
@@ -1010,25 +1022,7 @@ __device__ void fine_pass64(const AugArgs& A, int phase, double* acc, const doub
       const SegW<D> S = sg[si];
       const int z0 = max(S.z0, za), z1 = min(S.z1, ze);
       if (z0 > z1) continue;
-      // the segment's own moments: the running ones at z1 less the earlier segments' part
-      Moments64 g = (si < D - 1 && z1 < ze) ? snap[si < D - 1 ? si : 0] : m;
-      if (si > 0 && z0 > za) {
-        const Moments64& h = snap[si > 0 ? si - 1 : 0];
-        const double k = int_to_double(z1 - z0 + 1), k2 = int_to_double(((z1 - z0 + 1) * (z1 - z0 + 2)) >> 1);
-        g.q1 -= fma(k, h.q0, h.q1);
-        g.q0 -= h.q0;
-        if (phase == kFirst) {
-          g.t1 -= fma(k, h.t0, h.t1);
-          g.t0 -= h.t0;
-        }
-        if (!A.fixed_point) {
-          g.e1 -= fma(k, h.e0, h.e1);
-          g.e0 -= h.e0;
-          g.d2 -= fma(k2, h.d0, fma(k, h.d1, h.d2));
-          g.d1 -= fma(k, h.d0, h.d1);
-          g.d0 -= h.d0;
-        }
-      }
+      const Moments64 g = (si < D - 1 && S.z1 <= ze) ? snap[si < D - 1 ? si : 0] : m;   // ended here, or cut off
       // weights in m = z1 + 1 - z: p - z = a + m, z - q = b - m
       const double a = int_to_double(S.p - z1 - 1), b = int_to_double(z1 + 1 - S.q);
       double c[D - 1];
@@ -1176,6 +1170,7 @@ __device__ void fine_pass32(const AugArgs& A, int phase, double* acc, const doub
           if (z == zb[t]) {
             cs0[t] = q0;
             cs1[t] = q1;
+            q0 = q1 = 0.f;
           }
       };
       // sixteen independent loads in flight before the arithmetic, one memory latency per
@@ -1227,33 +1222,16 @@ __device__ void fine_pass32(const AugArgs& A, int phase, double* acc, const doub
       const Seg<D>& S = sg[si];
       const int z0 = max(S.z0, za), z1 = min(S.z1, ze);
       if (z0 > z1) continue;
-      const bool cut = si < D - 1 && z1 < ze;   // the segment ends inside the chunk
-      const bool cont = si > 0 && z0 > za;      // and begins inside it
+      const bool ended = si < D - 1 && S.z1 <= ze;   // in this chunk; else the chunk cut it off
       constexpr int L1 = D - 2;
       if (phase != kFirst) {
-        float q0 = cut ? cs0[si < L1 ? si : L1] : cq0, q1 = cut ? cs1[si < L1 ? si : L1] : cq1;
-        if (cont) {
-          q0 -= cs0[si > 0 ? si - 1 : 0];
-          q1 -= cs1[si > 0 ? si - 1 : 0];
-        }
+        const float q0 = ended ? cs0[si < L1 ? si : L1] : cq0, q1 = ended ? cs1[si < L1 ? si : L1] : cq1;
 #pragma unroll
         for (int t = 0; t <= D; ++t)
           add(G::RA + S.vid[t], ff{fmaf((float)S.P[t], q0, (float)S.R[t] * q1), 0.f});
         continue;
       }
-      FirstMoments g = cut ? fsnap[si < L1 ? si : L1] : fm;
-      if (cont) {
-        const FirstMoments& h = fsnap[si > 0 ? si - 1 : 0];
-        g.q0 = ff_sub(g.q0, h.q0);
-        g.q1 = ff_sub(g.q1, h.q1);
-        g.t0 = ff_sub(g.t0, h.t0);
-        g.t1 = ff_sub(g.t1, h.t1);
-        g.d0 -= h.d0;
-        g.d1 -= h.d1;
-        g.d2 -= h.d2;
-        g.e0 -= h.e0;
-        g.e1 -= h.e1;
-      }
+      const FirstMoments g = ended ? fsnap[si < L1 ? si : L1] : fm;
 #pragma unroll
       for (int t = 0; t <= D; ++t) {
         const float Pt = (float)S.P[t], Rt = (float)S.R[t];
