@@ -3115,9 +3115,11 @@ AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const Aug
     // moments to channels (per segment); a block's warps are dealt as Deal64 says, and the blocks
     // an SM holds share its sub-partitions; a second block per cell adds the cell's reduction
     // and a longer barrier (a node's and a conversion's FP64 operations: 2D 20 and 35, 3D 22 and 50).
+    // Chunks of 2 to 32 nodes: the shapes that fmg_autotune_augmented times, so that it never keeps one
+    // slower than this.
     const int node = dim == 2 ? 20 : 22, conv = dim == 2 ? 35 : 50, again = 30;
     long long best = -1;
-    for (int chunk = 1; chunk <= 32 && chunk <= sfine; chunk *= 2)
+    for (int chunk = 2; chunk <= 32 && chunk <= sfine; chunk *= 2)
       for (int bpc = 1; bpc <= ab.bpc; ++bpc) {
         const long long items = ncol * (sfine / chunk), n = (items + bpc - 1) / bpc;
         const long long warps = (n + 31) / 32;   // of one segment (or of all, when they are not split)
