@@ -69,7 +69,10 @@ typedef enum {
 } fmg_nonlin;
 
 typedef enum {
-  FMG_PREC_FP64 = 0,   /* every step in FP64 */
+  FMG_PREC_FP64 = 0,   /* every step in FP64; the small dense systems (level 1 and eq. 3.6) by
+                          refinement on an FP32 inverse with residual and solution in FP64, to an
+                          error no larger than an FP64 factorization's, which takes over where
+                          the refinement does not converge */
   FMG_PREC_MIXED = 1   /* multigrid cycles in FP32 inside a defect correction whose level
                           iterate, right-hand side, residual and update are float-float (an
                           unevaluated sum of two FP32 numbers, ~48 significant bits); the

@@ -818,7 +818,7 @@ struct Totals64 {
 // 3a is part of the channel weights) and a u^3 - g is one product and one fused multiply-add;
 // P c (pc at z0) advances along z by one add of the segment's slope.  2D: 20 operations in the first
 // pass and 15 in the others, against 26 and 20 for the plain form (2049^2: first pass 303 -> 193
-// us, others 217 -> 153, the running moments included).  Values are loaded B nodes at a time into registers, one memory latency
+// us, others 217 -> 153, the moments included).  Values are loaded B nodes at a time into registers, one memory latency
 // per batch.  zb: where the column's segments end (snap: the moments of the segment that ends there).
 template <int D, bool CUBIC, bool FIRST, bool VC>
 __device__ __forceinline__ void run64(const AugArgs& A, Moments64& m, Totals64& tot, Moments64* snap, const int* zb,
@@ -2010,7 +2010,8 @@ __device__ void newton_update(const AugArgs& A, const double* R, int NH, const S
 // make up for an error in the next step as Newton's does.
 // Against 80-bit arithmetic, over the systems of all 1/H, five nonlinearities and solutions of 1e-8
 // to 30 (about 2400): largest error 8e-13 of the norm, median 1e-17; the FP64 LDL^T 6.5e-12 and 9e-17.
-// Measured at 50 unknowns: 3.5 to 9 us per Newton iteration after the first, against 46.
+// Measured at 50 unknowns: 3.5 to 9 us per Newton iteration after the first with early steps solved
+// loosely, about a sweep (1.2 us) more as it is, against 46 for the factorization.
 // Where X is no good -- J not positive definite in FP32, the Schur complement of alpha below
 // kRefinePivot of its diagonal, magnitudes outside FP32, or no convergence in kRefineSweeps -- the
 // step falls back to the FP64 factorization, for the rest of the correction step (S.flags[2]).
@@ -2326,7 +2327,7 @@ __device__ void step_report(const AugArgs& A, const StepState& S, int it, bool w
 // iteration converges to the same FP64 solution).  FP64 path: each step is solved to FP64 accuracy
 // by refinement on an FP32 inverse of its own Jacobian, as the augmented step's (the system is
 // bordered by an idle unknown, so that it has the augmented system's shape; the FP64 factor and
-// substitutions of 49 unknowns took 40 us per iteration on one warp, this takes 19).
+// substitutions of 49 unknowns took 40 us per iteration on one warp, this takes 20).
 template <typename T>
 __device__ __forceinline__ void k_level1_newton_body(int dim, int n1, const double* __restrict__ g, double* __restrict__ u, int kind,
                                 double a, double tol, int maxit, DevState* st, int out_ff, VarCoef vc) {
@@ -3114,7 +3115,8 @@ AugShape aug_shape(int dim, int coarse_cells, int level, bool jac_f32, const Aug
     // instructions per SM sub-partition.  A chunk costs its nodes and one conversion of its
     // moments to channels (per segment); a block's warps are dealt as Deal64 says, and the blocks
     // an SM holds share its sub-partitions; a second block per cell adds the cell's reduction
-    // and a longer barrier (a node's and a conversion's FP64 operations: 2D 20 and 35, 3D 22 and 50).
+    // and a longer barrier.  A node counts as its FP64 operations (2D 20, 3D 22), a conversion as 35 and 50:
+    // 24 and 32 operations with their rows' loads and stores.
     // Chunks of 2 to 32 nodes: the shapes that fmg_autotune_augmented times, so that it never keeps one
     // slower than this.
     const int node = dim == 2 ? 20 : 22, conv = dim == 2 ? 35 : 50, again = 30;
